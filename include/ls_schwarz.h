@@ -139,9 +139,12 @@ typedef struct {
                           SMs, which share its factor stream and exchange partial sums
                           and solution blocks through distributed shared memory (when
                           twice the subdomain count does not exceed the SM count); 0 (the
-                          default) times those that fit at the end of setup and keeps
-                          the fastest (1 without timing on batched handles, whose solves
-                          run the multi right-hand-side path, and with test_stall);
+                          default) takes sweeps over superblocks of 128 rows, on one CTA
+                          or a cluster per subdomain by rule (reported as 4), where a
+                          subdomain's vector fits their shared memory; else it times
+                          those of 1 to 3 that fit at the end of setup and keeps the
+                          fastest.  Batched handles, whose solves run the multi
+                          right-hand-side path, and test_stall take 1.
                           LS_ERR_UNSUPPORTED when a forced one does not fit.
                           ls_info.local_config reports it.                             */
 } ls_options;

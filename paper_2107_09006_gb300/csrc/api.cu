@@ -101,8 +101,25 @@ void mark(ls_handle* h, int k) {
   else record_event(h->ev[k], h->st);
 }
 
-// y = local solves of rin (and, with_coarse, the fused coarse restriction r0 = R_0 rin)
+// r0 = R_0 v on stream st
+void launch_restriction(ls_handle* h, const double* v, cudaStream_t st) {
+  lsq::launch_restrict(h->N, h->sinfo.kmax, h->int_off.p, h->int_glob.p, h->zoff.p, h->coff.p, h->Z.p, v, h->r0.p, st);
+}
+
+// y = local solves of rin (and, with_coarse, the fused coarse restriction r0 = R_0 rin:
+// configurations 1 to 3; precond runs it beside configuration 4)
 void launch_local(ls_handle* h, const double* rin, bool with_coarse) {
+  if (h->local_cfg == 4) {
+    lsq::SuperArgs s{};
+    s.order = h->sb_order.p;
+    s.om_off = h->om_off.p; s.om_glob = h->om_glob.p; s.eqs = h->eqs.p;
+    s.blk_off = h->blk_off.p; s.tf = h->sb_tf.p; s.toff = h->sb_toff.p; s.fac = h->sb_fac.p;
+    s.r = rin; s.y = h->ybuf.p; s.err = h->scal.p + lsq::S_ERR;
+    s.n_cols = h->n; s.fac_bytes = (int64_t)h->sb_fac.n;
+    if (!lsq::launch_local_super(s, h->sb_shape, h->prec, h->N, h->max_nb, (size_t)h->sb_optin, h->st))
+      throw LsError(LS_ERR_CUDA, std::string("local solve (superblocks): ") + cudaGetErrorString(cudaGetLastError()));
+    return;
+  }
   lsq::LocalArgs a{};
   a.om_off = h->om_off.p; a.om_glob = h->om_glob.p; a.eqs = h->eqs.p;
   a.blk_off = h->blk_off.p; a.blk_tf = h->blk_tf.p; a.blk_poff = h->blk_poff.p;
@@ -143,6 +160,10 @@ void choose_local_config(ls_handle* h, int optin) {
     return;
   }
   if (h->opt.test_stall || h->nprob > 1) return;  // (batched handles solve through the block path)
+  if (h->sb_ok) {
+    h->local_cfg = 4;
+    return;
+  }
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
@@ -171,10 +192,20 @@ void choose_local_config(ls_handle* h, int optin) {
   h->local_cfg = pick;
 }
 
+// Whether the single-vector local solve runs over superblocks (configuration 4, chosen by
+// rule) and in which shape.  A forced configuration, the stalled test hook and batched
+// handles (whose solves run the multi right-hand-side path) keep the 32-row sweeps.
+void plan_super(ls_handle* h, int optin, int sms) {
+  h->sb_optin = optin;
+  h->sb_ok = h->opt.local_config == 0 && !h->opt.test_stall && h->nprob == 1 &&
+             lsq::local_super_plan(h->prec, h->N, h->max_nb, std::max(h->wmax, lsq::kSuperRows),
+                                   (double)h->fac_elems / 1024.0 / (double)h->total_blocks, sms, (size_t)optin, h->sb_shape);
+}
+
 // out = Q v = R_0^T C_00^{-1} R_0 v (restriction, dense coarse solve, prolongation)
 void coarse_term(ls_handle* h, const double* v, double* out) {
   cudaStream_t st = h->st;
-  lsq::launch_restrict(h->N, h->int_off.p, h->int_glob.p, h->zoff.p, h->coff.p, h->Z.p, v, h->r0.p, st);
+  launch_restriction(h, v, st);
   lsq::launch_gemv(h->n0p, h->Xinv.p, h->r0.p, h->y0.p, st);
   lsq::ScatterArgs s{};
   s.n = h->n; s.map_ptr = h->map_ptr.p; s.map_idx = h->map_idx.p; s.y = h->ybuf.p;
@@ -265,9 +296,28 @@ void precond(ls_handle* h, const double* rin, double* zout, int which, bool dots
   if (which != 0 && which != 1) throw LsError(LS_ERR_INVALID, "precond: which must be 0 or 1");
   if (timed) mark(h, 2);
   const bool use_coarse = h->coarse && h->n0 > 0 && which != 1;
-  if (which != 2) launch_local(h, rin, use_coarse);
-  if (timed) mark(h, 3);
-  if (use_coarse) lsq::launch_gemv(h->n0p, h->Xinv.p, h->r0.p, h->y0.p, st);
+  if (h->local_cfg == 4 && use_coarse) {
+    // The coarse correction reads only rin, and the local solves leave SMs idle (or wait on
+    // their chains): both run at once, the coarse kernels on the second stream, joined
+    // before the scatter.  With kernel timing they run one after the other.
+    cudaStream_t sc = timed ? st : h->st2;
+    if (!timed) {
+      CK(cudaEventRecord(h->ev_fork, st));
+      CK(cudaStreamWaitEvent(sc, h->ev_fork, 0));
+    }
+    launch_local(h, rin, false);
+    if (timed) mark(h, 3);
+    launch_restriction(h, rin, sc);
+    lsq::launch_gemv(h->n0p, h->Xinv.p, h->r0.p, h->y0.p, sc);
+    if (!timed) {
+      CK(cudaEventRecord(h->ev_coarse, sc));
+      CK(cudaStreamWaitEvent(st, h->ev_coarse, 0));
+    }
+  } else {
+    launch_local(h, rin, use_coarse);
+    if (timed) mark(h, 3);
+    if (use_coarse) lsq::launch_gemv(h->n0p, h->Xinv.p, h->r0.p, h->y0.p, st);
+  }
   if (timed) mark(h, 4);
   lsq::ScatterArgs s{};
   s.n = h->n; s.map_ptr = h->map_ptr.p; s.map_idx = h->map_idx.p; s.y = h->ybuf.p;
@@ -284,7 +334,8 @@ void precond(ls_handle* h, const double* rin, double* zout, int which, bool dots
 // Kernels one iteration launches (for the launch count reported in ls_info).
 int iteration_launches(const ls_handle* h) {
   if (balanced(h)) return 4 + kBalancedLaunches;
-  return 6 + ((h->coarse && h->n0 > 0) ? 1 : 0);
+  const bool coarse = h->coarse && h->n0 > 0;
+  return 6 + (coarse ? 1 : 0) + (coarse && h->local_cfg == 4 && h->opt.variant == 0 ? 1 : 0);
 }
 
 void iteration(ls_handle* h, bool flex, bool copy_scalars = true) {
@@ -1241,6 +1292,36 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     }
     lsq::launch_to_solve_layout(h->prec, h->total_blocks, h->blk_poff.p, Cst.p, dinv.p, dst,
                                 h->prec == LS_PREC_BF16 ? h->tsc.p : nullptr, st);
+    {
+      int optin = 0;
+      CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
+      plan_super(h, optin, sms);
+    }
+    if (h->sb_ok) {
+      // superblock storage: the tile columns of a block row reach back to its superblock's first
+      std::vector<int32_t> stf((size_t)h->total_blocks), order(N);
+      std::vector<int64_t> stoff((size_t)h->total_blocks);
+      int64_t bytes = 0;
+      const int64_t rec = (int64_t)lsq::local_super_record(h->prec, false), recx = (int64_t)lsq::local_super_record(h->prec, true);
+      for (int i = 0; i < N; ++i) {
+        order[i] = i;
+        for (int64_t g = hs.blk_off[i]; g < hs.blk_off[i + 1]; ++g) {
+          const int b = (int)(g - hs.blk_off[i]);
+          const int b0 = b / lsq::kSuperRows * lsq::kSuperRows;
+          stf[g] = std::min(hs.blk_tf[g], b0);
+          stoff[g] = bytes;
+          bytes += (b0 - stf[g]) * rec + (b - b0 + 1) * recx;
+        }
+      }
+      std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        return hs.blk_off[a + 1] - hs.blk_off[a] > hs.blk_off[b + 1] - hs.blk_off[b];
+      });
+      h->sb_tf.upload(stf, st); h->sb_toff.upload(stoff, st); h->sb_order.upload(order, st);
+      h->sb_fac.alloc((size_t)bytes);
+      lsq::launch_super_pack(h->prec, N, h->max_nb, h->blk_off.p, h->blk_tf.p, h->blk_poff.p, h->sb_tf.p,
+                             h->sb_toff.p, Cst.p, dinv.p, h->sb_fac.p, st);
+      CK(cudaStreamSynchronize(st));
+    }
     CK(cudaStreamSynchronize(st));
     check_launch("solve storage");
     Cst.release();
@@ -1461,6 +1542,11 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   CK(cudaHostAlloc((void**)&h->pin, sizeof(double) * lsq::S_NSLOT, cudaHostAllocDefault));
   if (h->opt.time_kernels)
     for (auto& e : h->ev) CK(cudaEventCreate(&e));
+  if (h->sb_ok && h->coarse && h->n0 > 0) {
+    CK(cudaStreamCreateWithFlags(&h->st2, cudaStreamNonBlocking));
+    CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
+    CK(cudaEventCreateWithFlags(&h->ev_coarse, cudaEventDisableTiming));
+  }
   std::memset(h->pin, 0, sizeof(double) * lsq::S_NSLOT);
   phase.next("ls_setup: sparse-product copies and autotuning");
   job.join();

@@ -157,6 +157,9 @@ struct ls_handle {
   int dev = 0;
   cudaStream_t st = nullptr;
   bool own_stream = false;
+  // the coarse correction runs beside the local solves on st2 (forked from and joined to st)
+  cudaStream_t st2 = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_coarse = nullptr;
   cudaEvent_t ev_join = nullptr;  // orders a call against the caller's stream (ls_solve, ls_backward)
   ls_options opt{};
   double tau = 0.0;  // threshold given to ls_setup (<= 0: automatic)
@@ -195,6 +198,13 @@ struct ls_handle {
   DevBuf<__nv_bfloat16> L16;
   int max_nb = 0;
   int local_cfg = 1;  // configuration of the single-vector local solve (option local_config)
+  // superblock storage of the single-vector local solve (local_cfg 4)
+  bool sb_ok = false;
+  int sb_optin = 0;
+  lsq::SuperShape sb_shape{};
+  DevBuf<int32_t> sb_tf, sb_order;
+  DevBuf<int64_t> sb_toff;
+  DevBuf<unsigned char> sb_fac;
   int64_t total_local = 0, total_blocks = 0, fac_elems = 0;
 
   bool coarse = false;
@@ -254,6 +264,9 @@ struct ls_handle {
     for (auto& e : ev)
       if (e) cudaEventDestroy(e);
     if (ev_join) cudaEventDestroy(ev_join);
+    if (ev_fork) cudaEventDestroy(ev_fork);
+    if (ev_coarse) cudaEventDestroy(ev_coarse);
+    if (st2) cudaStreamDestroy(st2);
     if (pin) cudaFreeHost(pin);
     if (own_stream && st) cudaStreamDestroy(st);
   }

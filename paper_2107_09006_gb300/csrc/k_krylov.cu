@@ -302,24 +302,46 @@ __global__ void __launch_bounds__(kThreads) k_scatter(ScatterArgs a) {
   if (a.dots.parts) finish_dots(acc_rz, acc_rzo, a.r_old != nullptr, a.dots);
 }
 
-// r0[c0 + t] = sum_jj Zbar_i[t, jj] v[Omega_I,i[jj]] (one block per subdomain, one warp
-// per coarse vector): the coarse restriction R_0 v on its own.
+// r0[c0 + t] = sum_jj Zbar_i[t, jj] v[Omega_I,i[jj]]: the coarse restriction R_0 v.  A block
+// takes four vectors of one subdomain (blockIdx.y), its threads stride the columns: each
+// gathered v entry is used four times and five loads per step are independent.  (One block
+// per subdomain with a warp per vector, its gathers on one dependent chain, took 25-68 us
+// for 25-64 subdomains of 1,600-2,304 columns, where this is a few.)
+constexpr int kRestrictVecs = 4;
 __global__ void __launch_bounds__(kThreads) k_restrict(const int64_t* __restrict__ int_off,
                                                        const int32_t* __restrict__ int_glob,
                                                        const int64_t* __restrict__ zoff,
                                                        const int32_t* __restrict__ coff, const double* __restrict__ Z,
                                                        const double* __restrict__ v, double* __restrict__ r0) {
-  const int i = blockIdx.x;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __shared__ double red[kWarps][kRestrictVecs];
+  const int i = blockIdx.x, t0 = blockIdx.y * kRestrictVecs;
   const int c0 = coff[i], kk = coff[i + 1] - c0;
+  if (t0 >= kk) return;
   const int64_t io = int_off[i];
-  const int64_t nIi = int_off[i + 1] - io;
+  const int nIi = (int)(int_off[i + 1] - io);
   const double* Zi = Z + zoff[i];
-  for (int t = w; t < kk; t += kWarps) {
-    double acc = 0.0;
-    for (int64_t jj = lane; jj < nIi; jj += 32) acc += Zi[(int64_t)t * nIi + jj] * v[int_glob[io + jj]];
-    acc = warp_sum(acc);
-    if (lane == 0) r0[c0 + t] = acc;
+  const double* row[kRestrictVecs];
+#pragma unroll
+  for (int u = 0; u < kRestrictVecs; ++u) row[u] = Zi + (int64_t)min(t0 + u, kk - 1) * nIi;
+  double acc[kRestrictVecs] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+  for (int jj = threadIdx.x; jj < nIi; jj += kThreads) {
+    const double g = v[__ldg(int_glob + io + jj)];
+#pragma unroll
+    for (int u = 0; u < kRestrictVecs; ++u) acc[u] += __ldg(row[u] + jj) * g;
+  }
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int u = 0; u < kRestrictVecs; ++u) {
+    const double sum = warp_sum(acc[u]);
+    if (lane == 0) red[w][u] = sum;
+  }
+  __syncthreads();
+  if (threadIdx.x < kRestrictVecs && t0 + (int)threadIdx.x < kk) {
+    double sum = 0.0;
+#pragma unroll
+    for (int k = 0; k < kWarps; ++k) sum += red[k][threadIdx.x];
+    r0[c0 + t0 + threadIdx.x] = sum;
   }
 }
 
@@ -723,9 +745,10 @@ void launch_multi_axpy(int64_t n, const double* V, int64_t ld, int k, const doub
   k_multi_axpy<<<grid_for(n, kThreads, kVecGrid), kThreads, 0, st>>>(n, V, ld, k, coef, sign, out);
 }
 
-void launch_restrict(int N, const int64_t* int_off, const int32_t* int_glob, const int64_t* zoff, const int32_t* coff,
-                     const double* Z, const double* v, double* r0, cudaStream_t st) {
-  k_restrict<<<N, kThreads, 0, st>>>(int_off, int_glob, zoff, coff, Z, v, r0);
+void launch_restrict(int N, int kmax, const int64_t* int_off, const int32_t* int_glob, const int64_t* zoff,
+                     const int32_t* coff, const double* Z, const double* v, double* r0, cudaStream_t st) {
+  const dim3 grid((unsigned)N, (unsigned)((kmax + kRestrictVecs - 1) / kRestrictVecs));
+  if (kmax > 0) k_restrict<<<grid, kThreads, 0, st>>>(int_off, int_glob, zoff, coff, Z, v, r0);
 }
 
 void launch_combine3(int64_t n, const double* a, const double* b, const double* c, double* z, const double* r,

@@ -124,8 +124,8 @@ void launch_multi_dot(int64_t n, const double* V, int64_t ld, int k, const doubl
 // out += sign * V coef (V column-major, ld; coef on the device)
 void launch_multi_axpy(int64_t n, const double* V, int64_t ld, int k, const double* coef, double sign, double* out,
                        cudaStream_t st);
-// r0 = R_0 v (coarse restriction alone, FP64)
-void launch_restrict(int N, const int64_t* int_off, const int32_t* int_glob, const int64_t* zoff, const int32_t* coff,
+// r0 = R_0 v (coarse restriction alone, FP64); kmax: most coarse vectors of a subdomain
+void launch_restrict(int N, int kmax, const int64_t* int_off, const int32_t* int_glob, const int64_t* zoff, const int32_t* coff,
                      const double* Z, const double* v, double* r0, cudaStream_t st);
 // z = a + b - c with r.z -> ds.out[0] and (r_old != nullptr) r_old.z -> ds.out[ds.out2]
 void launch_combine3(int64_t n, const double* a, const double* b, const double* c, double* z, const double* r,
@@ -181,6 +181,34 @@ void launch_local_solve(int prec, int config, int N, int max_nb, const LocalArgs
 size_t local_split_smem(int max_nb);
 int local_split_cluster();
 bool local_split_launch(int N, int max_nb, const LocalArgs& a, cudaStream_t st);
+// Superblock local solves (k_local_super.cu): block rows in groups of kSuperRows; block row
+// g (global) stores tile columns [tf[g], b] from byte toff[g] on, those before its own
+// superblock as tiles of L, those of its superblock from the inverse of the superblock's
+// diagonal, in records of local_super_record(prec, x) bytes (multiples of 16; tf[g] never
+// lies inside the superblock).
+constexpr int kSuperRows = 4;
+struct SuperArgs {
+  const int32_t* order;  // subdomains by decreasing size
+  const int64_t* om_off; const int32_t* om_glob; const double* eqs;
+  const int64_t* blk_off; const int32_t* tf; const int64_t* toff;
+  const unsigned char* fac;
+  const double* r; double* y;
+  double* err;            // error slot (bounds-checked build)
+  int depth;              // units in flight per warp (set by the launcher)
+  int ring;               // tile columns of the backward sums (set by the launcher)
+  int64_t n_cols, fac_bytes;  // bounds of the gather indices and the records (bounds-checked build)
+};
+size_t local_super_record(int prec, bool x);
+// Launch shape: CTAs per subdomain, consumer warps and CTAs per SM, tile columns of the
+// backward sums.  local_super_plan picks it by rule (block rows of at most wmax tiles, wmean
+// on average); false if none fits.
+struct SuperShape { int cluster, warps, occ, ring; };
+bool local_super_plan(int prec, int N, int max_nb, int wmax, double wmean, int sms, size_t optin, SuperShape& out);
+bool launch_local_super(const SuperArgs& a, const SuperShape& f, int prec, int N, int max_nb, size_t optin,
+                        cudaStream_t st);
+void launch_super_pack(int prec, int N, int max_nb, const int64_t* blk_off, const int32_t* blk_tf,
+                       const int64_t* blk_poff, const int32_t* stf, const int64_t* stoff, const double* L,
+                       const double* dinv, unsigned char* dst, cudaStream_t st);
 // Block-envelope factor + inverse diagonal tiles (FP64) -> solve storage (prec 0/1/2);
 // tsc receives one scale per 32x32 tile for BF16.
 void launch_to_solve_layout(int prec, int64_t nblocks, const int64_t* poff, const double* L, const double* dinv,

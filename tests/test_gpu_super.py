@@ -1,0 +1,58 @@
+"""The superblock local solve (the default configuration 4) against the 32-row sweeps
+(configuration 1, which test_gpu_parity.py holds to the oracle), in every launch shape the
+rule picks: one CTA per subdomain, clusters of 2, 4 and 8, two CTAs per SM, last
+superblocks of one to four block rows, subdomains of a single block row, envelopes that
+start inside a superblock, block rows wider and narrower than the warps deal at once.
+
+Tolerances: both configurations evaluate the same operator in different summation orders
+(BF16: from the same rounded factors), so they differ by a small multiple of kappa(C_ii)
+times the unit roundoff of the arithmetic: 1e-12 (FP64) and 1e-5 (FP32 sums), as between
+the other configurations in test_gpu_parity.py.
+"""
+import numpy as np
+import pytest
+import torch
+
+from workloads.grid import bisection_partition, block_partition, make_grid_ls, strip_partition
+
+pytestmark = pytest.mark.gpu
+
+# name: W, H, rows of the matrix (k, radius), partition
+SHAPES = {
+    "one-row": (4, 5, (4, 2), lambda W, H: np.zeros(W * H, np.int32)),
+    "strips": (32, 32, (4, 2), lambda W, H: strip_partition(W, H, 4)),
+    "blocks8": (24, 24, (8, 3), lambda W, H: block_partition(W, H, 8, 8)),
+    "blocks32-ragged": (90, 75, (8, 3), lambda W, H: block_partition(W, H, 32, 32)),
+    "bisect30": (100, 60, (6, 2), lambda W, H: bisection_partition(W, H, 300, 5)),
+    "n100": (60, 60, (6, 2), lambda W, H: block_partition(W, H, 6, 6)),
+    "n169": (65, 65, (6, 2), lambda W, H: block_partition(W, H, 5, 5)),
+    "n400": (80, 80, (8, 3), lambda W, H: block_partition(W, H, 4, 4)),
+    "wide": (128, 128, (8, 3), lambda W, H: block_partition(W, H, 64, 64)),
+    "scattered": (40, 30, (6, 2), lambda W, H: (np.arange(W * H) % 3).astype(np.int32)),
+}
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("name", sorted(SHAPES))
+def test_super_matches_row_sweeps(name, prec):
+    import paper_2107_09006_gb300 as L
+
+    W, H, (k, radius), split = SHAPES[name]
+    m, n, rp, col, val, b, _ = make_grid_ls(W, H, 4, k, radius, 7)
+    part = split(W, H)
+    r = torch.from_numpy(np.random.default_rng(2).standard_normal(n)).cuda()
+    z = {}
+    for config in (0, 1):
+        S = L.Solver(m, n, rp, col, val, part, int(part.max()) + 1, nev_max=4, factor_prec=prec, local_config=config)
+        assert S.info()["local_config"] == (4 if config == 0 else 1)
+        z[config] = S.apply_preconditioner(r, 1)
+        # both levels: the coarse correction runs beside the local solves
+        both = S.apply_preconditioner(r, 0)
+        apart = z[config] + S.apply_preconditioner(r, 2)
+        assert float((both - apart).norm() / apart.norm()) < 1e-13
+        if config == 0:
+            x, info = S.solve(b, rtol=1e-9)
+            assert info["relres_true"] <= 1e-9
+        S.close()
+    tol = 1e-12 if prec == "f64" else 1e-5
+    assert float((z[0] - z[1]).norm() / z[1].norm()) < tol
