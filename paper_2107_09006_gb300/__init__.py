@@ -237,9 +237,24 @@ def ls_normal_product_noalloc(m, n, row_ptr, col, val, col_ptr, row, cval, nnz, 
     int32[nnz], cval float64[nnz] (CSC), p and w float64[n]; anything else raises
     ValueError before the call.  Asynchronous on ``stream`` (a raw cudaStream_t handle
     or None)."""
-    _check_noalloc_args(m, n, nnz, row_ptr, col, val, col_ptr, row, cval, p, w)
-    st = _lib.ls_normal_product_noalloc(int(m), int(n), _ptr(row_ptr), _ptr(col), _ptr(val), _ptr(col_ptr),
-                                        _ptr(row), _ptr(cval), int(nnz), _ptr(p), _ptr(w), stream)
+    import torch
+    m, n, nnz = int(m), int(n), int(nnz)
+    # One pass over the arguments of a good call (a small product is bound by this host
+    # work: 26 us a call with the full check and the generic pointer conversion); whatever
+    # it does not recognise takes the full check, which names what is wrong.
+    i64, i32, f64 = torch.int64, torch.int32, torch.float64
+    dev = torch.cuda.current_device() if torch.cuda.is_initialized() else -1
+    ptrs = []
+    for t, dt, length in ((row_ptr, i64, m + 1), (col, i32, nnz), (val, f64, nnz), (col_ptr, i64, n + 1),
+                          (row, i32, nnz), (cval, f64, nnz), (p, f64, n), (w, f64, n)):
+        if not (type(t) is torch.Tensor and t.dtype is dt and t.shape == (length,) and t.is_contiguous()
+                and t.get_device() == dev >= 0):
+            _check_noalloc_args(m, n, nnz, row_ptr, col, val, col_ptr, row, cval, p, w)
+            ptrs = [_ptr(a) for a in (row_ptr, col, val, col_ptr, row, cval, p, w)]
+            break
+        ptrs.append(t.data_ptr())
+    rp, c, v, cp, r, cv, pp, pw = ptrs
+    st = _lib.ls_normal_product_noalloc(m, n, rp, c, v, cp, r, cv, nnz, pp, pw, stream)
     if st != LS_OK:
         raise LSError(st, _lib.ls_noalloc_last_error().decode())
 
