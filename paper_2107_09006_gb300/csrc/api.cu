@@ -1268,7 +1268,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   dinv.alloc((size_t)h->total_blocks * 1024);
   status.alloc(N);
   idiag.alloc((size_t)h->total_blocks * 32);
-  lsq::launch_band_cholesky(plan, Cst.p, idiag.p, dinv.p, status.p, st);
+  lsq::launch_band_cholesky(plan, h->max_nb, h->wmax, Cst.p, idiag.p, dinv.p, status.p, st);
   std::vector<int> hst(N);
   CK(cudaMemcpyAsync(hst.data(), status.p, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -1345,7 +1345,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     const double te0 = now_s();
     phase.next("ls_setup: local eigensolves and coarse operator");
     Bidiag.alloc((size_t)h->total_blocks * 32);
-    lsq::launch_band_cholesky(plan, Bst.p, Bidiag.p, dinv.p, status.p, st);
+    lsq::launch_band_cholesky(plan, h->max_nb, h->wmax, Bst.p, Bidiag.p, dinv.p, status.p, st);
     CK(cudaMemcpyAsync(hst.data(), status.p, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     check_launch("Cholesky of C~_ii + s I");

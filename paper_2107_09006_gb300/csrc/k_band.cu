@@ -1,6 +1,5 @@
 // Local matrices in block-envelope storage: assembly of C_ii and C~_ii, the shifts of
-// Section 4.1.2, batched Cholesky (one CTA per subdomain, left-looking over 32x32
-// tiles) and the batched local solves of the preconditioner apply.
+// Section 4.1.2 and the batched Cholesky (right-looking over 32x32 tiles).
 #include "band.cuh"
 #include "tile.cuh"
 #include "kernels.h"
@@ -132,60 +131,74 @@ __global__ void __launch_bounds__(kThreads) k_prep(BandPlan P, const double* __r
   }
 }
 
-// Left-looking tiled Cholesky of every subdomain's block-envelope matrix, in place.
-// dinv: scratch of 1024 doubles per block row holding the inverse diagonal tiles.
-__global__ void __launch_bounds__(kThreads) k_band_cholesky(BandPlan P, double* __restrict__ F,
-                                                            double* __restrict__ idiag, double* __restrict__ dinv,
-                                                            int* __restrict__ status) {
-  __shared__ double S[kT * 33], Pm[kT * 33], Qm[kT * 33];
+// Right-looking tiled Cholesky of every subdomain's block-envelope matrix, in place, block
+// column by block column for all subdomains at once: the diagonal tile (and its inverse, kept
+// in dinv, 1024 doubles per block row), the tiles below it, the update of the window's
+// tiles, one CTA per tile.  FP64-bound: a tile update is 32,768 FMAs, 8 us of one SM's two
+// per cycle; one CTA per subdomain ran the whole factor on as many SMs as there were
+// subdomains (16 of 1,936 columns: 33 ms).
+__global__ void __launch_bounds__(kThreads) k_chol_diag(BandPlan P, double* __restrict__ F, double* __restrict__ idiag,
+                                                        double* __restrict__ dinv, int* __restrict__ status, int k) {
+  __shared__ double S[kT * 33], Q[kT * 33];
   __shared__ int fail;
   const int i = blockIdx.x;
   const int64_t b0 = P.blk_off[i];
-  const int nb = (int)(P.blk_off[i + 1] - b0);
+  if (k >= (int)(P.blk_off[i + 1] - b0)) return;
+  const int t0 = P.blk_tf[b0 + k];
+  const int width = (k - t0 + 1) * kT;
+  double* pan = F + P.blk_poff[b0 + k];
   if (threadIdx.x == 0) fail = 0;
+  load_tile(S, pan, width, width - kT);
+  tile_potrf_inv(S, Q, &fail, k * kT);
+  store_tile(S, pan, width, width - kT);
+  double* dv = dinv + (b0 + k) * (int64_t)(kT * kT);
+  for (int e = threadIdx.x; e < kT * kT; e += blockDim.x) dv[e] = Q[(e >> 5) * 33 + (e & 31)];
+  if (threadIdx.x < kT) idiag[b0 * kT + k * kT + threadIdx.x] = Q[threadIdx.x * 33 + threadIdx.x];
+  if (threadIdx.x == 0 && fail && status[i] == 0) status[i] = fail;
+}
+
+// L(b, k) = A(b, k) L(k, k)^{-T} for the block rows b > k that reach column k.
+__global__ void __launch_bounds__(kThreads) k_chol_col(BandPlan P, double* __restrict__ F,
+                                                       const double* __restrict__ dinv, int k) {
+  __shared__ double S[kT * 33], A[kT * 33], Q[kT * 33];
+  const int i = blockIdx.x, b = k + 1 + blockIdx.y;
+  const int64_t b0 = P.blk_off[i];
+  if (b >= (int)(P.blk_off[i + 1] - b0)) return;
+  const int t0 = P.blk_tf[b0 + b];
+  if (t0 > k) return;
+  const int width = (b - t0 + 1) * kT;
+  double* pan = F + P.blk_poff[b0 + b];
+  load_tile(A, pan, width, (k - t0) * kT);
+  const double* dv = dinv + (b0 + k) * (int64_t)(kT * kT);
+  for (int e = threadIdx.x; e < kT * kT; e += blockDim.x) Q[(e >> 5) * 33 + (e & 31)] = dv[e];
   __syncthreads();
-  for (int b = 0; b < nb; ++b) {
-    const int tb = P.blk_tf[b0 + b];
-    const int wb = (b - tb + 1) * kT;
-    double* panb = F + P.blk_poff[b0 + b];
-    for (int c = tb; c <= b; ++c) {
-      const int tc = P.blk_tf[b0 + c];
-      const int wc = (c - tc + 1) * kT;
-      const double* panc = F + P.blk_poff[b0 + c];
-      load_tile(S, panb, wb, (c - tb) * kT);
-      __syncthreads();
-      for (int k = max(tb, tc); k < c; ++k) {
-        load_tile(Pm, panb, wb, (k - tb) * kT);
-        load_tile(Qm, panc, wc, (k - tc) * kT);
-        __syncthreads();
-        tile_mm<false, true>(S, Pm, Qm, -1);
-        __syncthreads();
-      }
-      if (c < b) {
-        // L(b,c) = S L(c,c)^{-T} = S * (L(c,c)^{-1})^T
-        const double* dv = dinv + (b0 + c) * (int64_t)(kT * kT);
-        for (int e = threadIdx.x; e < kT * kT; e += blockDim.x) Qm[(e >> 5) * 33 + (e & 31)] = dv[e];
-        for (int e = threadIdx.x; e < kT * kT; e += blockDim.x) Pm[(e >> 5) * 33 + (e & 31)] = S[(e >> 5) * 33 + (e & 31)];
-        __syncthreads();
-        tile_mm<false, true>(S, Pm, Qm, 0);
-        __syncthreads();
-      } else {
-        tile_potrf_inv(S, Qm, &fail, b * kT);
-        double* dv = dinv + (b0 + b) * (int64_t)(kT * kT);
-        for (int e = threadIdx.x; e < kT * kT; e += blockDim.x) dv[e] = Qm[(e >> 5) * 33 + (e & 31)];
-        if (threadIdx.x < kT) idiag[b0 * kT + b * kT + threadIdx.x] = Qm[threadIdx.x * 33 + threadIdx.x];
-        // zero the strict upper part of the diagonal tile
-        for (int e = threadIdx.x; e < kT * kT; e += blockDim.x) {
-          const int a = e >> 5, l = e & 31;
-          if (l > a) S[a * 33 + l] = 0.0;
-        }
-        __syncthreads();
-      }
-      store_tile(S, panb, wb, (c - tb) * kT);
-      __syncthreads();
-    }
-  }
-  if (threadIdx.x == 0) status[i] = fail;
+  tile_mm<false, true>(S, A, Q, 0);
+  __syncthreads();
+  store_tile(S, pan, width, (k - t0) * kT);
+}
+
+// A(b, c) -= L(b, k) L(c, k)^T for k < c <= b, both reaching column k (blockIdx.y enumerates
+// the pairs of the window below k).
+__global__ void __launch_bounds__(kThreads) k_chol_update(BandPlan P, double* __restrict__ F, int k) {
+  __shared__ double S[kT * 33], A[kT * 33], Q[kT * 33];
+  int ii = (int)((sqrtf(8.f * (float)blockIdx.y + 1.f) - 1.f) * 0.5f);
+  while ((ii + 1) * (ii + 2) / 2 <= (int)blockIdx.y) ++ii;
+  while (ii * (ii + 1) / 2 > (int)blockIdx.y) --ii;
+  const int i = blockIdx.x, b = k + 1 + ii, c = k + 1 + (int)blockIdx.y - ii * (ii + 1) / 2;
+  const int64_t b0 = P.blk_off[i];
+  if (b >= (int)(P.blk_off[i + 1] - b0)) return;
+  const int tb = P.blk_tf[b0 + b], tc = P.blk_tf[b0 + c];
+  if (tb > k || tc > k) return;
+  const int wb = (b - tb + 1) * kT, wc = (c - tc + 1) * kT;
+  double* panb = F + P.blk_poff[b0 + b];
+  const double* panc = F + P.blk_poff[b0 + c];
+  load_tile(S, panb, wb, (c - tb) * kT);
+  load_tile(A, panb, wb, (k - tb) * kT);
+  load_tile(Q, panc, wc, (k - tc) * kT);
+  __syncthreads();
+  tile_mm<false, true>(S, A, Q, -1);
+  __syncthreads();
+  store_tile(S, panb, wb, (c - tb) * kT);
 }
 
 int grid_for(int64_t work, int cap) {
@@ -210,9 +223,17 @@ void launch_prep(const BandPlan& P, const double* dsub, const double* s, double*
   k_prep<<<P.N, kThreads, 0, st>>>(P, dsub, s, Cst, eqs, Ctst, Bst);
 }
 
-void launch_band_cholesky(const BandPlan& P, double* F, double* idiag, double* dinv, int* status,
-                               cudaStream_t st) {
-  k_band_cholesky<<<P.N, kThreads, 0, st>>>(P, F, idiag, dinv, status);
+void launch_band_cholesky(const BandPlan& P, int max_nb, int wmax, double* F, double* idiag, double* dinv, int* status,
+                          cudaStream_t st) {
+  cudaMemsetAsync(status, 0, sizeof(int) * P.N, st);
+  for (int k = 0; k < max_nb; ++k) {
+    k_chol_diag<<<P.N, kThreads, 0, st>>>(P, F, idiag, dinv, status, k);
+    const int below = wmax - 1 < max_nb - 1 - k ? wmax - 1 : max_nb - 1 - k;  // block rows that can reach column k
+    if (below > 0) {
+      k_chol_col<<<dim3(P.N, below), kThreads, 0, st>>>(P, F, dinv, k);
+      k_chol_update<<<dim3(P.N, below * (below + 1) / 2), kThreads, 0, st>>>(P, F, k);
+    }
+  }
 }
 
 }  // namespace lsq

@@ -156,8 +156,9 @@ void launch_prep(const BandPlan& P, const double* dsub, const double* s, double*
 // In-place Cholesky of every subdomain's matrix; idiag = 1 / diag(L);
 // status[i] = 0 or 1 + the local row of the first nonpositive pivot.
 // dinv: scratch of 1024 doubles per block row (inverse diagonal tiles).
-void launch_band_cholesky(const BandPlan& P, double* st_fac, double* idiag, double* dinv, int* status,
-                          cudaStream_t st);
+// max_nb, wmax: most block rows of a subdomain and most tiles of a block row.
+void launch_band_cholesky(const BandPlan& P, int max_nb, int wmax, double* st_fac, double* idiag, double* dinv,
+                          int* status, cudaStream_t st);
 
 // ---- batched local solves (k_local.cu) -----------------------------------------------
 struct LocalArgs {
