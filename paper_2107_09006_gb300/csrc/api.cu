@@ -115,6 +115,7 @@ void launch_local(ls_handle* h, const double* rin, bool with_coarse) {
     s.om_off = h->om_off.p; s.om_glob = h->om_glob.p; s.eqs = h->eqs.p;
     s.blk_off = h->blk_off.p; s.tf = h->sb_tf.p; s.toff = h->sb_toff.p; s.fac = h->sb_fac.p;
     s.r = rin; s.y = h->ybuf.p; s.err = h->scal.p + lsq::S_ERR;
+    s.sweeps = 3;
     s.n_cols = h->n; s.fac_bytes = (int64_t)h->sb_fac.n;
     if (!lsq::launch_local_super(s, h->sb_shape, h->prec, h->N, h->max_nb, (size_t)h->sb_optin, h->st))
       throw LsError(LS_ERR_CUDA, std::string("local solve (superblocks): ") + cudaGetErrorString(cudaGetLastError()));
@@ -200,6 +201,35 @@ void plan_super(ls_handle* h, int optin, int sms) {
   h->sb_ok = h->opt.local_config == 0 && !h->opt.test_stall && h->nprob == 1 &&
              lsq::local_super_plan(h->prec, h->N, h->max_nb, std::max(h->wmax, lsq::kSuperRows),
                                    (double)h->fac_elems / 1024.0 / (double)h->total_blocks, sms, (size_t)optin, h->sb_shape);
+}
+
+// Superblock storage of the block-envelope plan in factor precision prec: first tile column
+// (reaching back to the superblock's first) and byte offset of every block row, subdomains by
+// decreasing size.  Returns the bytes.
+struct SuperHost {
+  std::vector<int32_t> tf, order;
+  std::vector<int64_t> off;
+  int64_t bytes = 0;
+};
+SuperHost super_storage(const lsq::HostSets& hs, int N, int prec) {
+  SuperHost s;
+  const size_t nblk = (size_t)hs.blk_off[N];
+  s.tf.resize(nblk); s.off.resize(nblk); s.order.resize(N);
+  const int64_t rec = (int64_t)lsq::local_super_record(prec, false), recx = (int64_t)lsq::local_super_record(prec, true);
+  for (int i = 0; i < N; ++i) {
+    s.order[i] = i;
+    for (int64_t g = hs.blk_off[i]; g < hs.blk_off[i + 1]; ++g) {
+      const int b = (int)(g - hs.blk_off[i]);
+      const int b0 = b / lsq::kSuperRows * lsq::kSuperRows;
+      s.tf[g] = std::min(hs.blk_tf[g], b0);
+      s.off[g] = s.bytes;
+      s.bytes += (b0 - s.tf[g]) * rec + (b - b0 + 1) * recx;
+    }
+  }
+  std::stable_sort(s.order.begin(), s.order.end(), [&](int a, int b) {
+    return hs.blk_off[a + 1] - hs.blk_off[a] > hs.blk_off[b + 1] - hs.blk_off[b];
+  });
+  return s;
 }
 
 // out = Q v = R_0^T C_00^{-1} R_0 v (restriction, dense coarse solve, prolongation)
@@ -1298,26 +1328,9 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
       plan_super(h, optin, sms);
     }
     if (h->sb_ok) {
-      // superblock storage: the tile columns of a block row reach back to its superblock's first
-      std::vector<int32_t> stf((size_t)h->total_blocks), order(N);
-      std::vector<int64_t> stoff((size_t)h->total_blocks);
-      int64_t bytes = 0;
-      const int64_t rec = (int64_t)lsq::local_super_record(h->prec, false), recx = (int64_t)lsq::local_super_record(h->prec, true);
-      for (int i = 0; i < N; ++i) {
-        order[i] = i;
-        for (int64_t g = hs.blk_off[i]; g < hs.blk_off[i + 1]; ++g) {
-          const int b = (int)(g - hs.blk_off[i]);
-          const int b0 = b / lsq::kSuperRows * lsq::kSuperRows;
-          stf[g] = std::min(hs.blk_tf[g], b0);
-          stoff[g] = bytes;
-          bytes += (b0 - stf[g]) * rec + (b - b0 + 1) * recx;
-        }
-      }
-      std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        return hs.blk_off[a + 1] - hs.blk_off[a] > hs.blk_off[b + 1] - hs.blk_off[b];
-      });
-      h->sb_tf.upload(stf, st); h->sb_toff.upload(stoff, st); h->sb_order.upload(order, st);
-      h->sb_fac.alloc((size_t)bytes);
+      const SuperHost sh = super_storage(hs, N, h->prec);
+      h->sb_tf.upload(sh.tf, st); h->sb_toff.upload(sh.off, st); h->sb_order.upload(sh.order, st);
+      h->sb_fac.alloc((size_t)sh.bytes);
       lsq::launch_super_pack(h->prec, N, h->max_nb, h->blk_off.p, h->blk_tf.p, h->blk_poff.p, h->sb_tf.p,
                              h->sb_toff.p, Cst.p, dinv.p, h->sb_fac.p, st);
       CK(cudaStreamSynchronize(st));
@@ -1372,7 +1385,51 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     ea.kwant_cap = kw; ea.Kmax = K; ea.keep = keep; ea.maxit = h->opt.eig_maxit; ea.tol = h->opt.eig_tol;
     ea.V = V.p; ea.V2 = V2.p; ea.vstride = vs; ea.H = H.p; ea.S = S.p; ea.vec = vec.p; ea.lam = lam.p;
     ea.nconv = nconv.p; ea.steps = steps.p; ea.status = est.p;
-    lsq::launch_lanczos(ea, st);
+    // over the whole GPU where a subdomain's FP64 vector fits the superblock kernel, else one
+    // CTA per subdomain
+    lsq::LanczosGrid lg{};
+    DevBuf<int> lz_state, lz_rr, lz_ord;
+    DevBuf<double> lz_beta, lz_err;
+    {
+      int optin = 0;
+      CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
+      if (lsq::local_super_plan(0, N, h->max_nb, std::max(h->wmax, lsq::kSuperRows),
+                                (double)h->fac_elems / 1024.0 / (double)h->total_blocks, sms, (size_t)optin, lg.shape)) {
+        Ctst.release();  // (the operator runs from A)
+        const SuperHost sh = super_storage(hs, N, LS_PREC_F64);
+        DevBuf<int32_t> etf, eorder, locpos;
+        DevBuf<int64_t> eoff;
+        DevBuf<unsigned char> efac;
+        etf.upload(sh.tf, st); eoff.upload(sh.off, st); eorder.upload(sh.order, st);
+        efac.alloc((size_t)sh.bytes);
+        lsq::launch_super_pack(LS_PREC_F64, N, h->max_nb, h->blk_off.p, h->blk_tf.p, h->blk_poff.p, etf.p, eoff.p,
+                               Bst.p, dinv.p, efac.p, st);
+        std::vector<int32_t> lp((size_t)h->n, 0);
+        for (int i = 0; i < N; ++i)
+          for (int64_t a = hs.int_off[i]; a < hs.int_off[i + 1]; ++a)
+            lp[hs.om_glob[hs.om_off[i] + hs.int_loc[a]]] = hs.int_loc[a];
+        locpos.upload(lp, st);
+        lz_state.alloc((size_t)N * lsq::kLanczosState); lz_rr.alloc((size_t)N * 2); lz_ord.alloc((size_t)N * K);
+        lz_beta.alloc(N); lz_err.alloc(1); lz_err.zero(st);
+        lg.fac.order = eorder.p;
+        lg.fac.om_off = h->om_off.p; lg.fac.om_glob = h->om_glob.p; lg.fac.eqs = h->eqs.p;
+        lg.fac.blk_off = h->blk_off.p; lg.fac.tf = etf.p; lg.fac.toff = eoff.p; lg.fac.fac = efac.p;
+        lg.fac.n_cols = h->n; lg.fac.fac_bytes = sh.bytes;
+        lg.max_nb = h->max_nb; lg.optin = (size_t)optin;
+        lg.A = csr(h); lg.At = csc(h); lg.part = h->part.p; lg.locpos = locpos.p; lg.total_local = h->total_local;
+        lg.state = lz_state.p; lg.rr = lz_rr.p; lg.ord = lz_ord.p; lg.beta = lz_beta.p; lg.err = lz_err.p;
+        if (!lsq::run_lanczos_grid(ea, lg, st)) {
+          CK(cudaStreamSynchronize(st));
+          double err = 0.0;
+          CK(cudaMemcpy(&err, lz_err.p, sizeof(double), cudaMemcpyDeviceToHost));
+          if (err == lsq::kErrBounds) throw LsError(LS_ERR_INVALID, "an index out of range was met (bounds-checked build) in the eigensolves");
+          if (err != 0.0) throw LsError(LS_ERR_DEVICE_TIMEOUT, "a bounded wait in the eigensolves gave up");
+          throw LsError(LS_ERR_CUDA, "a launch of the eigensolves was refused");
+        }
+      } else {
+        lsq::launch_lanczos(ea, st);
+      }
+    }
     h->h_lam.assign((size_t)N * kw, 0.0);
     CK(cudaMemcpyAsync(h->h_lam.data(), lam.p, sizeof(double) * N * kw, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(h->h_steps.data(), steps.p, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
@@ -1425,7 +1482,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     h->coff.upload(hcoff, st);
     h->zoff.upload(hzoff, st);
     h->Z.alloc(std::max<int64_t>(hzoff[N], 1));
-    lsq::launch_eigvec(ea, h->coff.p, h->zoff.p, h->int_off.p, h->int_loc.p, h->Z.p, st);
+    lsq::launch_eigvec(ea, lz_state.p ? lz_state.p + 3 * (size_t)N : nullptr, kmax, h->coff.p, h->zoff.p, h->int_off.p, h->int_loc.p, h->Z.p, st);
     check_launch("coarse basis");
     V.release(); V2.release(); H.release(); S.release(); vec.release();
     if (h->n0 > 0) {

@@ -10,6 +10,9 @@
 // D C_ii D x = D (C~_ii (D x)) + delta D x, since the interior block of C~_ii equals
 // that of C_ii = A(:,Omega)^T A(:,Omega) + delta I.  Every loop is bounded by
 // maxit; a subdomain that does not converge reports status 2.
+#include <algorithm>
+#include <vector>
+
 #include "band.cuh"
 #include "kernels.h"
 
@@ -340,8 +343,330 @@ __global__ void __launch_bounds__(kThreads) k_lanczos(EigArgs a, int use_smem) {
   }
 }
 
-// Z_i[t, :] = interior entries of L^{-T} U_t (U_t = Ritz vector t in V).
-__global__ void __launch_bounds__(kThreads) k_eigvec(EigArgs a, const int32_t* __restrict__ coff,
+// ---- the same iteration over the whole GPU ----------------------------------------------------
+// k_lanczos keeps a subdomain on one CTA: with 16 subdomains of 1,900 columns, 16 SMs, each
+// bound by its two FP64 FMAs per cycle (2 ms a step, 226 ms in all).  Here every stage of a
+// step is a kernel over all subdomains: the triangular solves on the clusters of the
+// superblock kernel, the product with D C~ D as two sparse products with the subdomain's
+// part of A (264 multiplications per interior column instead of the 1,088 entries its row of
+// the band holds), the re-orthogonalisation on a cluster of eight CTAs per subdomain.  The
+// recurrences, tolerances, restarts and start vectors are those of k_lanczos.
+
+// Phases of a subdomain: 0 expanding, 1 expansion complete (Rayleigh-Ritz next), 2 done, 3
+// restarting (its kept vectors are rotated, the residual direction is to be appended).
+struct LzState {
+  int* nV; int* steps; int* phase; int* buf; int* fresh;
+};
+__device__ __forceinline__ LzState lz_state(const LanczosGrid& g, int N) {
+  return LzState{g.state, g.state + N, g.state + 2 * N, g.state + 3 * N, g.state + 4 * N};
+}
+__device__ __forceinline__ double* lz_basis(const EigArgs& a, int i, int buf) {
+  return (buf ? a.V2 : a.V) + (int64_t)i * a.Kmax * a.vstride;
+}
+
+__global__ void __launch_bounds__(kThreads) k_lz_start(EigArgs a, LanczosGrid g) {
+  __shared__ double red[kWarps];
+  const int i = blockIdx.x;
+  const int ni = (int)(a.P.om_off[i + 1] - a.P.om_off[i]);
+  const int npad = (int)(a.P.blk_off[i + 1] - a.P.blk_off[i]) * kT;
+  double* V = a.V + (int64_t)i * a.Kmax * a.vstride;
+  double* x1 = a.vec + (int64_t)i * 2 * a.vstride;
+  double s = 0.0;
+  for (int k = threadIdx.x; k < ni; k += kThreads) {
+    const double h = hash_unit(i, k) + 0.5;
+    s += h * h;
+  }
+  s = sqrt(block_sum(s, red));
+  for (int k = threadIdx.x; k < npad; k += kThreads) {
+    V[k] = x1[k] = k < ni ? (hash_unit(i, k) + 0.5) / s : 0.0;
+    x1[a.vstride + k] = 0.0;  // (the operator writes entries below n_i only)
+  }
+  if (threadIdx.x == 0) {
+    const LzState t = lz_state(g, a.P.N);
+    t.nV[i] = 1; t.steps[i] = 0; t.phase[i] = 0; t.buf[i] = 0; t.fresh[i] = 1;
+    a.nconv[i] = 0; a.status[i] = 0;
+  }
+}
+
+// x2 = D (A_i^T (A_i (D x1))) + delta D x1, A_i the rows of A that touch the subdomain's
+// interior columns, restricted to them (= D C~_ii D x1 + delta D x1).  A warp per local
+// entry: lane per row of its column, whose interior entries it walks.  Bound by the
+// gathers' latency; one pass without a stored A_i (D x1), whose rows would belong to
+// several subdomains.
+__global__ void __launch_bounds__(kThreads) k_lz_op(EigArgs a, LanczosGrid g) {
+  const int lane = threadIdx.x & 31;
+  const int* phase = g.state + 2 * a.P.N;
+  for (int64_t e = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5; e < g.total_local;
+       e += ((int64_t)gridDim.x * kThreads) >> 5) {
+    const int i = a.P.row_sub[e];
+    if (phase[i] != 0) continue;
+    const int k = (int)(e - a.P.om_off[i]);
+    const double* x1 = a.vec + (int64_t)i * 2 * a.vstride;
+    double y = 0.0;
+    if (a.P.om_int[e]) {
+      const int32_t j = a.P.om_glob[e];
+      for (int64_t t = g.At.col_ptr[j] + lane; t < g.At.col_ptr[j + 1]; t += 32) {
+        const int32_t r = g.At.row[t];
+        double s = 0.0;
+        for (int64_t q = g.A.row_ptr[r]; q < g.A.row_ptr[r + 1]; ++q) {
+          const int32_t c = g.A.col[q];
+          if (g.part[c] == i) s += g.A.val[q] * x1[g.locpos[c]];
+        }
+        y += g.At.val[t] * s;
+      }
+      y = warp_sum(y) + a.delta[i] * x1[k];
+    }
+    if (lane == 0) const_cast<double*>(x1)[a.vstride + k] = y;
+  }
+}
+
+constexpr int kOrthCluster = 8;
+__device__ __forceinline__ void lz_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ double lz_peer(const double* p, int rank) {
+  uint32_t r;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
+  return v;
+}
+
+// One cluster per subdomain, each CTA an eighth of the entries: x2 orthogonalised twice
+// against the basis (h = V^T x2, x2 -= V h), the column of H, the new basis vector (or, at
+// the end of an expansion, the residual left in x2); phase 3: the residual direction (or a
+// fresh one) appended to the kept vectors.  The ranks' partial sums are read through
+// distributed shared memory and added in rank order.
+__global__ void __cluster_dims__(kOrthCluster, 1, 1) __launch_bounds__(kThreads) k_lz_orth(EigArgs a, LanczosGrid g) {
+  extern __shared__ __align__(16) double lsm[];
+  __shared__ double hp[3][kMaxK + 1];  // this rank's partial sums (three places in turn: read by peers after a barrier)
+  __shared__ double h1[kMaxK], h2[kMaxK], red[kWarps], bc[2];
+  const int i = blockIdx.x / kOrthCluster, rank = blockIdx.x % kOrthCluster;
+  const LzState st = lz_state(g, a.P.N);
+  const int ph = st.phase[i];
+  if (ph == 1 || ph == 2) return;  // (the whole cluster)
+  const int ni = (int)(a.P.om_off[i + 1] - a.P.om_off[i]);
+  const int npad = (int)(a.P.blk_off[i + 1] - a.P.blk_off[i]) * kT;
+  const int K = a.Kmax, Keff = min(K, ni);
+  const int nV = st.nV[i], steps = st.steps[i] + (ph == 0 ? 1 : 0);
+  int fresh = st.fresh[i];
+  const int64_t vs = a.vstride;
+  double* V = lz_basis(a, i, st.buf[i]);
+  double* x1g = a.vec + (int64_t)i * 2 * vs;
+  const int sl = (npad / kT + kOrthCluster - 1) / kOrthCluster * kT;
+  const int k0 = min(npad, rank * sl), len = min(npad, k0 + sl) - k0;
+  double* x = lsm;  // this rank's slice
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int turn = 0;
+  auto project = [&](double* h) {
+    double* mine = hp[turn];
+    for (int t = w; t < nV; t += kWarps) {
+      const double* vt = V + t * vs + k0;
+      double acc = 0.0;
+#pragma unroll 4
+      for (int k = lane; k < len; k += 32) acc += vt[k] * x[k];
+      acc = warp_sum(acc);
+      if (lane == 0) mine[t] = acc;
+    }
+    lz_cluster_sync();
+    for (int t = threadIdx.x; t < nV; t += kThreads) {
+      double s = 0.0;
+#pragma unroll
+      for (int r = 0; r < kOrthCluster; ++r) s += lz_peer(&mine[t], r);
+      h[t] = s;
+    }
+    turn = turn == 2 ? 0 : turn + 1;
+    __syncthreads();
+  };
+  auto subtract = [&](const double* h) {
+    for (int k = threadIdx.x; k < len; k += kThreads) {
+      double acc = 0.0;
+      const double* vk = V + k0 + k;
+#pragma unroll 8
+      for (int t = 0; t < nV; ++t) acc += vk[t * vs] * h[t];
+      x[k] -= acc;
+    }
+    __syncthreads();
+  };
+  auto norm = [&]() -> double {
+    double acc = 0.0;
+    for (int k = threadIdx.x; k < len; k += kThreads) acc += x[k] * x[k];
+    acc = block_sum(acc, red);
+    if (threadIdx.x == 0) hp[turn][kMaxK] = acc;
+    lz_cluster_sync();
+    double s = 0.0;
+#pragma unroll
+    for (int r = 0; r < kOrthCluster; ++r) s += lz_peer(&hp[turn][kMaxK], r);
+    turn = turn == 2 ? 0 : turn + 1;
+    return sqrt(s);
+  };
+  auto orthogonalise = [&]() {
+    project(h1);
+    subtract(h1);
+    project(h2);
+    subtract(h2);
+  };
+  auto fresh_start = [&]() -> double {  // a new direction orthogonal to the basis: its norm
+    for (int k = threadIdx.x; k < len; k += kThreads)
+      x[k] = k0 + k < ni ? hash_unit(i + 7919u * (uint32_t)(fresh + 1), k0 + k) : 0.0;
+    ++fresh;
+    __syncthreads();
+    orthogonalise();
+    return norm();
+  };
+  auto append = [&](double scale) {
+    double* vn = V + (int64_t)nV * vs + k0;
+    for (int k = threadIdx.x; k < len; k += kThreads) vn[k] = x1g[k0 + k] = x[k] / scale;
+  };
+  for (int k = threadIdx.x; k < len; k += kThreads) x[k] = x1g[vs + k0 + k];
+  __syncthreads();
+  double beta = 0.0;
+  int next = 0;
+  if (ph == 0) {
+    orthogonalise();
+    double* H = a.H + (int64_t)i * K * K;
+    if (rank == 0)
+      for (int t = threadIdx.x; t < nV; t += kThreads) H[t * K + (nV - 1)] = h1[t] + h2[t];
+    if (w == 0) {
+      double hn = 0.0;
+      for (int t = lane; t < nV; t += 32) hn += (h1[t] + h2[t]) * (h1[t] + h2[t]);
+      hn = warp_sum(hn);
+      if (lane == 0) bc[0] = hn;
+    }
+    beta = norm();
+    __syncthreads();
+    const bool breakdown = !(beta > 1e-12 * sqrt(bc[0] + beta * beta));
+    if (nV < Keff && steps < a.maxit) {
+      if (!breakdown) append(beta);
+      else append(fresh_start());
+    } else {
+      next = 1;
+      if (breakdown) beta = 0.0;
+      for (int k = threadIdx.x; k < len; k += kThreads) x1g[vs + k0 + k] = x[k];
+    }
+  } else {
+    beta = g.beta[i];
+    if (beta > 0.0) append(beta);
+    else append(fresh_start());
+  }
+  lz_cluster_sync();  // (peers have read this rank's sums; every rank has read the state)
+  if (rank == 0 && threadIdx.x == 0) {
+    st.steps[i] = steps;
+    st.fresh[i] = fresh;
+    st.phase[i] = next;
+    if (next == 0) st.nV[i] = nV + 1;
+    else g.beta[i] = beta;
+  }
+}
+
+// Rayleigh-Ritz of the subdomains whose expansion is complete (one CTA each): eigenvalues and
+// vectors of the projected matrix, convergence count, whether it is done, and the restarted
+// projected matrix.
+__global__ void __launch_bounds__(kThreads) k_lz_ritz(EigArgs a, LanczosGrid g, int use_smem) {
+  extern __shared__ __align__(16) double lsm[];
+  __shared__ double cs[kMaxK / 2], sn[kMaxK / 2], red[kWarps], th[kMaxK];
+  __shared__ int pp[kMaxK / 2], qq[kMaxK / 2], ord[kMaxK];
+  const int i = blockIdx.x;
+  const LzState st = lz_state(g, a.P.N);
+  if (st.phase[i] != 1) return;
+  const int ni = (int)(a.P.om_off[i + 1] - a.P.om_off[i]);
+  const int K = a.Kmax, nV = st.nV[i], steps = st.steps[i];
+  const int kw = min(a.kwant_cap, ni), Keff = min(K, ni);
+  const int keep = max(kw, min(a.keep, Keff - 1));
+  double* Hg = a.H + (int64_t)i * K * K;
+  double* Sg = a.S + (int64_t)i * K * K;
+  double* H = use_smem ? lsm : Hg;
+  double* S = use_smem ? lsm + K * K : Sg;
+  Shared s{};
+  s.cs = cs; s.sn = sn; s.red = red; s.pp = pp; s.qq = qq; s.ord = ord;
+  if (use_smem) {
+    for (int e = threadIdx.x; e < K * K; e += kThreads) H[e] = Hg[e];
+    __syncthreads();
+  }
+  jacobi(H, S, K, nV, s);
+  const double beta = g.beta[i];
+  const int kk = min(kw, nV);
+  int nconv = 0;
+  const double th0 = fabs(H[ord[0] * K + ord[0]]);
+  for (int t = 0; t < kk; ++t) {
+    const double res = beta * fabs(S[(nV - 1) * K + ord[t]]);
+    if (res <= a.tol * fmax(th0, 1e-300)) ++nconv; else break;
+  }
+  const bool done = nconv >= kk || nV >= ni || steps >= a.maxit;
+  const int cnt = done ? kk : keep;
+  for (int t = threadIdx.x; t < cnt; t += kThreads) th[t] = H[ord[t] * K + ord[t]];
+  for (int t = threadIdx.x; t < nV; t += kThreads) g.ord[(int64_t)i * K + t] = ord[t];
+  __syncthreads();
+  for (int e = threadIdx.x; e < K * K; e += kThreads) {
+    const int r = e / K, c = e % K;
+    if (use_smem) Sg[e] = (r < nV && c < nV) ? S[e] : 0.0;
+    Hg[e] = (r == c && r < cnt) ? th[r] : 0.0;
+  }
+  if (done)
+    for (int t = threadIdx.x; t < kk; t += kThreads) a.lam[(int64_t)i * a.kwant_cap + t] = th[t];
+  if (threadIdx.x == 0) {
+    g.rr[i] = cnt;
+    g.rr[a.P.N + i] = done ? 1 : 0;
+    a.nconv[i] = nconv;
+    a.steps[i] = steps;
+    if (done && nconv < kk && nV < ni) a.status[i] = 2;
+  }
+}
+
+// Kept vectors of the other buffer: V'_t = sum_s V_s S[s][ord[t]] (blockIdx.y: 256 entries;
+// eight vectors per pass over the basis, their coefficients in shared memory).
+constexpr int kRotVecs = 8;
+__global__ void __launch_bounds__(kThreads) k_lz_rotate(EigArgs a, LanczosGrid g) {
+  __shared__ double co[kMaxK][kRotVecs];
+  const int i = blockIdx.x;
+  const LzState st = lz_state(g, a.P.N);
+  if (st.phase[i] != 1) return;
+  const int npad = (int)(a.P.blk_off[i + 1] - a.P.blk_off[i]) * kT;
+  const int K = a.Kmax, nV = st.nV[i], cnt = g.rr[i];
+  const double* in = lz_basis(a, i, st.buf[i]);
+  double* out = lz_basis(a, i, st.buf[i] ^ 1);
+  const double* S = a.S + (int64_t)i * K * K;
+  const int* ord = g.ord + (int64_t)i * K;
+  const int k = blockIdx.y * kThreads + threadIdx.x;
+  if (blockIdx.y * kThreads >= npad) return;
+  for (int t0 = 0; t0 < cnt; t0 += kRotVecs) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < nV * kRotVecs; e += kThreads) {
+      const int t = t0 + e % kRotVecs;
+      co[e / kRotVecs][e % kRotVecs] = t < cnt ? S[(e / kRotVecs) * K + ord[t]] : 0.0;
+    }
+    __syncthreads();
+    if (k < npad) {
+      double acc[kRotVecs];
+#pragma unroll
+      for (int u = 0; u < kRotVecs; ++u) acc[u] = 0.0;
+#pragma unroll 4
+      for (int s = 0; s < nV; ++s) {
+        const double v = in[s * a.vstride + k];
+#pragma unroll
+        for (int u = 0; u < kRotVecs; ++u) acc[u] += v * co[s][u];
+      }
+#pragma unroll
+      for (int u = 0; u < kRotVecs; ++u)
+        if (t0 + u < cnt) out[(int64_t)(t0 + u) * a.vstride + k] = acc[u];
+    }
+  }
+}
+
+__global__ void k_lz_flip(EigArgs a, LanczosGrid g) {
+  const LzState st = lz_state(g, a.P.N);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.P.N; i += gridDim.x * blockDim.x)
+    if (st.phase[i] == 1) {
+      st.buf[i] ^= 1;
+      st.nV[i] = g.rr[i];
+      st.phase[i] = g.rr[a.P.N + i] ? 2 : 3;
+    }
+}
+
+// Z_i[t, :] = interior entries of L^{-T} U_t (U_t = Ritz vector t); blockIdx.y: the vector,
+// or all of them on one CTA when the solve's vector lives in global memory.
+__global__ void __launch_bounds__(kThreads) k_eigvec(EigArgs a, const int* __restrict__ buffer,
+                                                     const int32_t* __restrict__ coff,
                                                      const int64_t* __restrict__ zoff,
                                                      const int64_t* __restrict__ int_off,
                                                      const int32_t* __restrict__ int_loc, double* __restrict__ Z,
@@ -354,14 +679,14 @@ __global__ void __launch_bounds__(kThreads) k_eigvec(EigArgs a, const int32_t* _
   const int64_t vs = a.vstride;
   double* base = reinterpret_cast<double*>(smem_raw);
   double* x1 = use_smem ? base : a.vec + (int64_t)i * 2 * vs;
-  double* dt = base + (use_smem ? 2 * vs : 0);
+  double* dt = base + (use_smem ? vs : 0);
   double* tmp = dt + kT * 33;
   BandRef B{a.P.blk_tf + b0, a.P.blk_poff + b0, nb};
-  const double* V = a.V + (int64_t)i * a.Kmax * vs;
+  const double* V = lz_basis(a, i, buffer ? buffer[i] : 0);
   const int k = coff[i + 1] - coff[i];
   const int64_t io = int_off[i];
   const int nIi = (int)(int_off[i + 1] - io);
-  for (int t = 0; t < k; ++t) {
+  for (int t = blockIdx.y; t < k; t += gridDim.y) {
     for (int e = threadIdx.x; e < npad; e += blockDim.x) x1[e] = V[t * vs + e];
     __syncthreads();
     band_backward<double, double>(a.Bfac, nullptr, a.Bidiag + b0 * kT, B, x1, dt, tmp);
@@ -386,13 +711,65 @@ void launch_lanczos(const EigArgs& a, cudaStream_t st) {
   k_lanczos<<<a.P.N, kThreads, sm, st>>>(a, use);
 }
 
-void launch_eigvec(const EigArgs& a, const int32_t* coff, const int64_t* zoff, const int64_t* int_off,
-                   const int32_t* int_loc, double* Z, cudaStream_t st) {
-  const size_t full = (2 * (size_t)a.vstride + kT * 33 + kT) * sizeof(double);
+bool run_lanczos_grid(const EigArgs& a, const LanczosGrid& g, cudaStream_t st) {
+  const int N = a.P.N, K = a.Kmax;
+  SuperArgs bwd = g.fac;
+  bwd.src = a.vec; bwd.src_stride = 2 * a.vstride;  // x1 <- L^{-T} x1
+  bwd.dst = a.vec; bwd.dst_stride = 2 * a.vstride;
+  bwd.skip = g.state + 2 * N;
+  bwd.sweeps = 2;
+  bwd.err = g.err;
+  SuperArgs fwd = bwd;
+  fwd.src = a.vec + a.vstride;  // x2 <- L^{-1} x2
+  fwd.dst = a.vec + a.vstride;
+  fwd.sweeps = 1;
+  const size_t orth_sm = (size_t)((a.vstride / kT + kOrthCluster - 1) / kOrthCluster * kT) * sizeof(double);
+  const size_t ritz_full = 2 * (size_t)K * K * sizeof(double);
+  const int ritz_use = ritz_full <= 200 * 1024;
+  const size_t ritz_sm = ritz_use ? ritz_full : 0;
+  if (cudaFuncSetAttribute(k_lz_orth, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess ||
+      cudaFuncSetAttribute(k_lz_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
+    return false;
+  int64_t op_grid = (g.total_local + kWarps - 1) / kWarps;
+  if (op_grid > (1 << 15)) op_grid = 1 << 15;
+  const dim3 rot_grid((unsigned)N, (unsigned)((a.vstride + kThreads - 1) / kThreads));
+  std::vector<int> phase((size_t)N);
+  double err = 0.0;
+  k_lz_start<<<N, kThreads, 0, st>>>(a, g);
+  int steps = 0, basis = 1;
+  for (;;) {
+    const int run = std::max(1, std::min(K - basis + 1, a.maxit - steps));
+    for (int k = 0; k < run; ++k) {
+      if (!launch_local_super(bwd, g.shape, 0, N, g.max_nb, g.optin, st)) return false;
+      k_lz_op<<<(unsigned)op_grid, kThreads, 0, st>>>(a, g);
+      if (!launch_local_super(fwd, g.shape, 0, N, g.max_nb, g.optin, st)) return false;
+      k_lz_orth<<<N * kOrthCluster, kThreads, orth_sm, st>>>(a, g);
+    }
+    steps += run;
+    basis = a.keep + 1;
+    k_lz_ritz<<<N, kThreads, ritz_sm, st>>>(a, g, ritz_use);
+    k_lz_rotate<<<rot_grid, kThreads, 0, st>>>(a, g);
+    k_lz_flip<<<(N + 127) / 128, 128, 0, st>>>(a, g);
+    k_lz_orth<<<N * kOrthCluster, kThreads, orth_sm, st>>>(a, g);  // (the restarting ones append their residual)
+    if (cudaMemcpyAsync(phase.data(), g.state + 2 * N, sizeof(int) * N, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(&err, g.err, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess || err != 0.0)
+      return false;
+    bool all = true;
+    for (int p : phase) all = all && p == 2;
+    if (all) return true;
+  }
+}
+
+void launch_eigvec(const EigArgs& a, const int* buffer, int kmax, const int32_t* coff, const int64_t* zoff,
+                   const int64_t* int_off, const int32_t* int_loc, double* Z, cudaStream_t st) {
+  if (kmax < 1) return;
+  const size_t full = ((size_t)a.vstride + kT * 33 + kT) * sizeof(double);
   const int use = full <= 200 * 1024;
   const size_t sm = use ? full : (kT * 33 + kT) * sizeof(double);
   cudaFuncSetAttribute(k_eigvec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_eigvec<<<a.P.N, kThreads, sm, st>>>(a, coff, zoff, int_off, int_loc, Z, use);
+  const dim3 grid((unsigned)a.P.N, use ? (unsigned)kmax : 1u);
+  k_eigvec<<<grid, kThreads, sm, st>>>(a, buffer, coff, zoff, int_off, int_loc, Z, use);
 }
 
 }  // namespace lsq

@@ -182,15 +182,24 @@ struct UnitList {
   const int32_t* tf;
   const int32_t* toff;
   int nb, nsb, q, cls, clx;
+  int sweeps;  // 1 forward, 2 backward, 3 both
   int s = 0, sweep = 0, ph = -1, u = 0, end = 0, step = 0;
   int64_t row = 0;  // byte offset that tile column 0 of the row would have, tiles of rec bytes
   int rec = 0;
+  __device__ void start() {
+    if (!(sweeps & 1)) { sweep = 1; s = nsb - 1; }
+    seek();
+  }
   __device__ void seek() {  // to the next phase that has a unit
     while (u >= end) {
       if (++ph == 2) {
         ph = 0;
         if (sweep == 0) {
-          if (++s == nsb) { sweep = 1; s = nsb - 1; }
+          if (++s == nsb) {
+            sweep = (sweeps & 2) ? 1 : 2;
+            if (sweep == 2) return;
+            s = nsb - 1;
+          }
         } else if (--s < 0) {
           sweep = 2;
           return;
@@ -425,7 +434,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
   const int ni = (int)(a.om_off[i + 1] - o0);
   const int64_t g0 = a.blk_off[i];
   const int nb = (int)(a.blk_off[i + 1] - g0);
-  if (nb == 0) return;  // (the host rejects empty subdomains; the whole cluster leaves)
+  if (nb == 0 || (a.skip && a.skip[i] != 0)) return;  // (the whole cluster leaves)
   const int nsb = (nb + kQ - 1) / kQ;
   int32_t* tf = reinterpret_cast<int32_t*>(v + (size_t)nb * kT);
   int32_t* toff = tf + nb;
@@ -445,11 +454,11 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
     // ---- producer: lane k streams the units of consumer warp k, in its order ----------------
     if (lane < NW) {
       const int cls = rank + C * (lane % JW);
-      List l{tf, toff, nb, nsb, lane / JW, cls, kSplitX ? cls : lane % JW};
+      List l{tf, toff, nb, nsb, lane / JW, cls, kSplitX ? cls : lane % JW, a.sweeps};
       unsigned char* slots = sm + (size_t)lane * depth * K::UB;
       uint64_t* fb = full + lane * depth;
       uint64_t* eb = empty + lane * depth;
-      l.seek();
+      l.start();
       int slot = 0, used = 0;  // used: slots filled so far, at most depth
       uint32_t par = 1;        // parity of the empty phase a slot waits for (0 after the first wrap)
       int64_t issued = 0;
@@ -494,7 +503,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
     uint64_t* eb = empty + w * depth;
     int slot = 0;
     uint32_t par = 0;
-    List l{tf, toff, nb, nsb, q, cls, clx};
+    List l{tf, toff, nb, nsb, q, cls, clx, a.sweeps};
     auto fetch = [&]() {  // (registers) the next unit of the list
       if constexpr (!kRing)
         if (!l.done()) {
@@ -506,7 +515,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
         }
     };
     if constexpr (!kRing) {
-      l.seek();
+      l.start();
       fetch();
     }
     auto acquire = [&]() -> const unsigned char* {  // the next unit of the list has arrived
@@ -523,6 +532,9 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
       }
     };
     // r(Omega_i), scaled by the equilibration, while the first units load
+    if (a.src) {
+      for (int k = tid; k < nb * kT; k += NT) v[k] = (TA)a.src[(int64_t)i * a.src_stride + k];
+    } else
     for (int k = tid; k < nb * kT; k += NT)
       v[k] = (k < ni && in_range(a.om_glob[o0 + k], a.n_cols, a.err))
                  ? (TA)(a.r[a.om_glob[o0 + k]] * a.eqs[o0 + k])
@@ -532,7 +544,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
     all_barrier();
 
     // ---- forward sweep ------------------------------------------------------------------------
-    for (int s = 0; s < nsb; ++s) {
+    for (int s = 0; s < nsb && (a.sweeps & 1); ++s) {
       const int b0 = s * kQ, b = b0 + q, lim = U * b0, nr = min(nb - b0, kQ);
       const bool has = b < nb;
       const uint32_t mpar = (uint32_t)((s >> 1) & 1);
@@ -595,10 +607,10 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
       all_barrier();
     }
     // ---- backward sweep -----------------------------------------------------------------------
-    for (int s = nsb - 1; s >= 0; --s) {
+    for (int s = nsb - 1; s >= 0 && (a.sweeps & 2); --s) {
       const int b0 = s * kQ, b = b0 + q, lim = U * b0, nr = min(nb - b0, kQ);
       const bool has = b < nb;
-      const int m = nsb - 1 - s, e = nsb + m;  // exchanges so far: of w_s, of X shares
+      const int m = nsb - 1 - s, e = m + ((a.sweeps & 1) ? nsb : 0);  // exchanges so far: of w_s, of X shares
       if (C > 1 && tid == 0) {
         bar_expect(&mbar[2 + (m & 1)], (uint32_t)(nr * 32 * sizeof(TA)));
         if (kSplitX) bar_expect(&mbar[4 + (e & 1)], (uint32_t)(U * nr * (nr + 1) / 2 * UC * sizeof(TA)));
@@ -663,10 +675,12 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
       }
       all_barrier();
     }
-    if (!*abort_flag) {
+    if (*abort_flag) {
+      if (tid == 0 && a.err[0] == 0.0) a.err[0] = kErrTimeout;
+    } else if (a.dst) {
+      for (int k = rank * NT + tid; k < nb * kT; k += C * NT) a.dst[(int64_t)i * a.dst_stride + k] = (double)v[k];
+    } else {
       for (int k = rank * NT + tid; k < ni; k += C * NT) a.y[o0 + k] = (double)v[k] * a.eqs[o0 + k];
-    } else if (tid == 0 && a.err[0] == 0.0) {
-      a.err[0] = kErrTimeout;
     }
   }
   if (C > 1) {

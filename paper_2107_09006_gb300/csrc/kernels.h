@@ -194,7 +194,12 @@ struct SuperArgs {
   const int64_t* blk_off; const int32_t* tf; const int64_t* toff;
   const unsigned char* fac;
   const double* r; double* y;
-  double* err;            // error slot (bounds-checked build)
+  // or (src, dst set) on vectors in local order, subdomain i's of its padded length at
+  // src + i src_stride and dst + i dst_stride, without the scales
+  const double* src; int64_t src_stride; double* dst; int64_t dst_stride;
+  const int* skip;        // subdomains with skip[i] != 0 are left out (null: none)
+  int sweeps;             // 1 the forward sweep (L^{-1}), 2 the backward one (L^{-T}), 3 both
+  double* err;            // error slot
   int depth;              // units in flight per warp (set by the launcher)
   int ring;               // tile columns of the backward sums (set by the launcher)
   int64_t n_cols, fac_bytes;  // bounds of the gather indices and the records (bounds-checked build)
@@ -232,8 +237,32 @@ struct EigArgs {
 };
 size_t lanczos_smem(int max_nb);
 void launch_lanczos(const EigArgs& a, cudaStream_t st);
-// Z_i = interior rows of L_B^{-T} U_i for the first k_i Ritz vectors U_i (V holds them).
-void launch_eigvec(const EigArgs& a, const int32_t* coff, const int64_t* zoff,
+// The same iteration, a kernel per stage over all subdomains in lockstep (k_lanczos.cu):
+// the operator's triangular solves run on the superblock kernel (fac: the superblock
+// storage of chol(C~_ii + s I), FP64), its middle part as A^T (A .) on the interior columns.
+struct LanczosGrid {
+  SuperArgs fac;
+  SuperShape shape;
+  int max_nb;
+  size_t optin;
+  CsrDev A; CscDev At;
+  const int32_t* part;
+  const int32_t* locpos;  // position of column j in its own subdomain's Omega
+  int64_t total_local;
+  int* state;             // [5][N]: basis size, steps, phase, buffer (0: V, 1: V2), fresh starts
+  int* rr;                // [2][N]: kept vectors, done
+  int* ord;               // [N][K] Ritz order
+  double* beta;           // [N]
+  double* err;
+};
+constexpr int kLanczosState = 5;
+// Runs to completion (the host waits once per restart); a.status, a.steps, a.nconv, a.lam as
+// launch_lanczos; the Ritz vectors lie in the buffer g.state[3] names.  False if a launch
+// was refused or a wait gave up.
+bool run_lanczos_grid(const EigArgs& a, const LanczosGrid& g, cudaStream_t st);
+// Z_i = interior rows of L_B^{-T} U_i for the first k_i (at most kmax) Ritz vectors U_i, in
+// V, or where buffer[i] != 0 in V2 (buffer may be null).
+void launch_eigvec(const EigArgs& a, const int* buffer, int kmax, const int32_t* coff, const int64_t* zoff,
                    const int64_t* int_off, const int32_t* int_loc, double* Z, cudaStream_t st);
 
 // ---- coarse operator (k_coarse.cu) -------------------------------------------------
