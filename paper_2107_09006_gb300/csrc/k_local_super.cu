@@ -453,8 +453,8 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
   if (kRing && w == NW) {
     // ---- producer: lane k streams the units of consumer warp k, in its order ----------------
     if (lane < NW) {
-      const int cls = rank + C * (lane % JW);
-      List l{tf, toff, nb, nsb, lane / JW, cls, kSplitX ? cls : lane % JW, a.sweeps};
+      const int q = lane / JW, jq = (lane % JW + q) % JW, cls = rank + C * jq;
+      List l{tf, toff, nb, nsb, q, cls, kSplitX ? cls : jq, a.sweeps};
       unsigned char* slots = sm + (size_t)lane * depth * K::UB;
       uint64_t* fb = full + lane * depth;
       uint64_t* eb = empty + lane * depth;
@@ -490,7 +490,9 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
   } else {
     // ---- consumers ----------------------------------------------------------------------------
     const int q = w / JW, j = w % JW;  // team (block row of the superblock), warp of the team
-    const int cls = rank + C * j, clx = kSplitX ? cls : j;
+    // (the teams deal their columns to warps one further on: a warp with one unit more than the
+    // others then sits in another sub-partition of the SM in every team)
+    const int jq = (j + q) % JW, cls = rank + C * jq, clx = kSplitX ? cls : jq;
     auto first_u = [&](int b) {
       const int lo = U * tf[b];
       return cls + (lo > cls ? (lo - cls + ST - 1) / ST * ST : 0);
