@@ -696,7 +696,17 @@ int block_local_umma_tmem_cols(int max_step_tiles) {
 int block_local_umma_ncol(int max_step_tiles) { return max_step_tiles <= 4 * kChunkTiles ? 64 : 32; }
 
 bool block_local_umma_prepare(size_t smem) {
-  return cudaFuncSetAttribute(k_b_local_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+  // The kernel's limit is the device's (less its static shared memory), not this handle's
+  // need: handles with wider windows share the kernel.
+  int dev = 0, cap = 0;
+  cudaFuncAttributes fa{};
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaFuncGetAttributes(&fa, k_b_local_umma) != cudaSuccess)
+    return false;
+  const int dyn = cap - (int)fa.sharedSizeBytes;
+  return smem <= (size_t)dyn &&
+         cudaFuncSetAttribute(k_b_local_umma, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) == cudaSuccess;
 }
 
 void launch_b_local_umma(const BUmmaArgs& a, int grid, cudaStream_t st) {
