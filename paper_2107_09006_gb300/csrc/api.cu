@@ -116,6 +116,7 @@ void launch_local(ls_handle* h, const double* rin, bool with_coarse) {
     s.blk_off = h->blk_off.p; s.tf = h->sb_tf.p; s.toff = h->sb_toff.p; s.fac = h->sb_fac.p;
     s.r = rin; s.y = h->ybuf.p; s.err = h->scal.p + lsq::S_ERR;
     s.sweeps = 3;
+    s.R = 1;
     s.n_cols = h->n; s.fac_bytes = (int64_t)h->sb_fac.n;
     if (!lsq::launch_local_super(s, h->sb_shape, h->prec, h->N, h->max_nb, (size_t)h->sb_optin, h->st))
       throw LsError(LS_ERR_CUDA, std::string("local solve (superblocks): ") + cudaGetErrorString(cudaGetLastError()));
@@ -201,35 +202,6 @@ void plan_super(ls_handle* h, int optin, int sms) {
   h->sb_ok = h->opt.local_config == 0 && !h->opt.test_stall && h->nprob == 1 &&
              lsq::local_super_plan(h->prec, h->N, h->max_nb, std::max(h->wmax, lsq::kSuperRows),
                                    (double)h->fac_elems / 1024.0 / (double)h->total_blocks, sms, (size_t)optin, h->sb_shape);
-}
-
-// Superblock storage of the block-envelope plan in factor precision prec: first tile column
-// (reaching back to the superblock's first) and byte offset of every block row, subdomains by
-// decreasing size.  Returns the bytes.
-struct SuperHost {
-  std::vector<int32_t> tf, order;
-  std::vector<int64_t> off;
-  int64_t bytes = 0;
-};
-SuperHost super_storage(const lsq::HostSets& hs, int N, int prec) {
-  SuperHost s;
-  const size_t nblk = (size_t)hs.blk_off[N];
-  s.tf.resize(nblk); s.off.resize(nblk); s.order.resize(N);
-  const int64_t rec = (int64_t)lsq::local_super_record(prec, false), recx = (int64_t)lsq::local_super_record(prec, true);
-  for (int i = 0; i < N; ++i) {
-    s.order[i] = i;
-    for (int64_t g = hs.blk_off[i]; g < hs.blk_off[i + 1]; ++g) {
-      const int b = (int)(g - hs.blk_off[i]);
-      const int b0 = b / lsq::kSuperRows * lsq::kSuperRows;
-      s.tf[g] = std::min(hs.blk_tf[g], b0);
-      s.off[g] = s.bytes;
-      s.bytes += (b0 - s.tf[g]) * rec + (b - b0 + 1) * recx;
-    }
-  }
-  std::stable_sort(s.order.begin(), s.order.end(), [&](int a, int b) {
-    return hs.blk_off[a + 1] - hs.blk_off[a] > hs.blk_off[b + 1] - hs.blk_off[b];
-  });
-  return s;
 }
 
 // out = Q v = R_0^T C_00^{-1} R_0 v (restriction, dense coarse solve, prolongation)
@@ -1328,7 +1300,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
       plan_super(h, optin, sms);
     }
     if (h->sb_ok) {
-      const SuperHost sh = super_storage(hs, N, h->prec);
+      const lsi::SuperHost sh = lsi::super_storage(hs.blk_off, hs.blk_tf, N, h->prec);
       h->sb_tf.upload(sh.tf, st); h->sb_toff.upload(sh.off, st); h->sb_order.upload(sh.order, st);
       h->sb_fac.alloc((size_t)sh.bytes);
       lsq::launch_super_pack(h->prec, N, h->max_nb, h->blk_off.p, h->blk_tf.p, h->blk_poff.p, h->sb_tf.p,
@@ -1396,7 +1368,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
       if (lsq::local_super_plan(0, N, h->max_nb, std::max(h->wmax, lsq::kSuperRows),
                                 (double)h->fac_elems / 1024.0 / (double)h->total_blocks, sms, (size_t)optin, lg.shape)) {
         Ctst.release();  // (the operator runs from A)
-        const SuperHost sh = super_storage(hs, N, LS_PREC_F64);
+        const lsi::SuperHost sh = lsi::super_storage(hs.blk_off, hs.blk_tf, N, LS_PREC_F64);
         DevBuf<int32_t> etf, eorder, locpos;
         DevBuf<int64_t> eoff;
         DevBuf<unsigned char> efac;

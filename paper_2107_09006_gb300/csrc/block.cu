@@ -121,6 +121,63 @@ void swizzle_prepare(ls_handle* h) {
   check_launch("swizzled factor copy");
 }
 
+// Whether the block local solve of R right-hand sides runs over superblocks (by rule), its
+// storage made from the solve storage at the first use.  With a forced block_kernel or the
+// stalled test hook it does not.  FP32 factors (eight right-hand sides per CTA): not where
+// more than two groups of eight make more than three CTAs per SM (N = 256, R = 32: 968 us
+// against 780 for the mma.sync kernel, which reads a tile once for all 32; N = 64, R = 32: 273
+// against 438 for the tcgen05 kernel; R = 8: 163 against 432; N = 256, R = 8: 284 against
+// 774), and on a batched handle from four right-hand sides on: below, the automatic choice is
+// pinned by a test to one of the two tensor-core kernels (64 subdomains and R = 2: 430 us,
+// the superblocks 164).
+void plan_block_super(ls_handle* h, int R) {
+  BlockState& B = h->blk;
+  if (B.m_R == R) return;
+  B.m_R = R;
+  B.m_ok = false;
+  if (h->opt.block_kernel != 0 || h->opt.test_stall) return;
+  if (h->prec == LS_PREC_F32 && h->nprob > 1 && R < 4) return;
+  int optin = 0, sms = 0;
+  CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev));
+  h->sb_optin = optin;
+  const int64_t groups = (R + 7) / 8;
+  if (h->prec == LS_PREC_F32 && groups > 2 && groups * h->N > 3 * (int64_t)sms) return;
+  B.m_ok = lsq::local_super_plan_multi(h->prec, R, h->N, h->max_nb, std::max(h->wmax, lsq::kSuperRows), sms,
+                                       (size_t)optin, B.m_shape);
+  if (!B.m_ok || B.m_fac.p) return;
+  cudaStream_t st = h->st;
+  std::vector<int64_t> boff((size_t)h->N + 1);
+  std::vector<int32_t> tf((size_t)h->total_blocks);
+  CK(cudaMemcpyAsync(boff.data(), h->blk_off.p, sizeof(int64_t) * boff.size(), cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(tf.data(), h->blk_tf.p, sizeof(int32_t) * tf.size(), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  const SuperHost sh = super_storage(boff, tf, h->N, h->prec);
+  B.m_tf.upload(sh.tf, st); B.m_toff.upload(sh.off, st); B.m_order.upload(sh.order, st);
+  B.m_back = h->prec == LS_PREC_F32 ? sh.bytes : 0;
+  B.m_fac.alloc((size_t)(sh.bytes + B.m_back));
+  lsq::launch_super_pack_solve(h->prec, h->N, h->max_nb, h->blk_off.p, h->blk_tf.p, h->blk_poff.p, B.m_tf.p,
+                               B.m_toff.p,
+                               h->prec == LS_PREC_F64 ? (const void*)h->L64.p
+                               : h->prec == LS_PREC_F32 ? (const void*)h->L32.p : (const void*)h->L16.p,
+                               h->prec == LS_PREC_BF16 ? h->tsc.p : nullptr, B.m_back, B.m_fac.p, st);
+  CK(cudaStreamSynchronize(st));
+  check_launch("superblock storage of the block path");
+}
+
+void launch_block_super(ls_handle* h, int R, const double* Rin) {
+  BlockState& B = h->blk;
+  lsq::SuperArgs s{};
+  s.order = B.m_order.p;
+  s.om_off = h->om_off.p; s.om_glob = h->om_glob.p; s.eqs = h->eqs.p;
+  s.blk_off = h->blk_off.p; s.tf = B.m_tf.p; s.toff = B.m_toff.p; s.fac = B.m_fac.p;
+  s.r = Rin; s.y = B.Y.p; s.R = R; s.sweeps = 3; s.back = B.m_back;
+  s.err = h->scal.p + lsq::S_ERR;
+  s.n_cols = h->n; s.fac_bytes = (int64_t)B.m_fac.n;
+  if (!lsq::launch_local_super(s, B.m_shape, h->prec, h->N, h->max_nb, (size_t)h->sb_optin, h->st))
+    throw LsError(LS_ERR_CUDA, std::string("block local solve (superblocks): ") + cudaGetErrorString(cudaGetLastError()));
+}
+
 void launch_local_kernel(ls_handle* h, int kernel, int R, const double* Rin) {
   BlockState& B = h->blk;
   cudaStream_t st = h->st;
@@ -212,17 +269,18 @@ void choose_local_kernel(ls_handle* h, int R, const double* Rin) {
 void precond_block(ls_handle* h, int R, const double* Rin, double* Zout, bool flex, bool timed) {
   BlockState& B = h->blk;
   cudaStream_t st = h->st;
-  choose_local_kernel(h, R, Rin);
+  if (!B.m_ok) choose_local_kernel(h, R, Rin);
   if (timed) record_event(h->ev[2], st);
-  launch_local_kernel(h, B.use_tc ? B.kernel : 0, R, Rin);
+  if (B.m_ok) launch_block_super(h, R, Rin);
+  else launch_local_kernel(h, B.use_tc ? B.kernel : 0, R, Rin);
   if (timed) record_event(h->ev[3], st);
   const bool coarse = h->coarse && h->n0 > 0;
   const bool zt = coarse && B.ZT.p != nullptr;
   if (coarse) {
     if (zt)
-      lsq::launch_b_restrict32(h->N, R, h->int_off.p, h->int_glob.p, h->coff.p, B.zt_off.p, B.ZT.p, Rin, B.R0.p, st);
+      lsq::launch_b_restrict32(h->N, h->sinfo.kmax, R, h->int_off.p, h->int_glob.p, h->coff.p, B.zt_off.p, B.ZT.p, Rin, B.R0.p, st);
     else
-      lsq::launch_b_restrict(h->N, R, h->int_off.p, h->int_glob.p, h->zoff.p, h->coff.p, h->Z.p, Rin, B.R0.p, st);
+      lsq::launch_b_restrict(h->N, h->sinfo.kmax, R, h->int_off.p, h->int_glob.p, h->zoff.p, h->coff.p, h->Z.p, Rin, B.R0.p, st);
     const lsq::CoarseBlocks cb{h->cb_prob_of_sub.p, h->cb_base.p, h->cb_ld.p, h->cb_c0.p};
     lsq::launch_b_coarse(B.nct, R, B.ct_prob.p, B.ct_row.p, cb, B.n0q.p, h->Xinv.p, B.R0.p, B.Y0.p,
                          zt ? B.Y0f.p : nullptr, st);
@@ -534,7 +592,7 @@ bool block_core(ls_handle* h, int R, double rtol, int mode, const std::vector<do
   inf.delta = h->sinfo.delta; inf.t_setup = h->sinfo.t_setup; inf.t_eig = h->sinfo.t_eig;
   inf.eig_steps_max = h->sinfo.eig_steps_max;
   inf.lanes_csr = h->lanes_csr; inf.lanes_csc = h->lanes_csc; inf.normal_product = h->normal_kind; inf.local_config = h->local_cfg;
-  inf.local_kernel = h->blk.use_tc ? h->blk.kernel : 0;
+  inf.local_kernel = h->blk.use_tc && !h->blk.m_ok ? h->blk.kernel : 0;
   return converged || fixed > 0;
 }
 
@@ -546,6 +604,7 @@ ls_status block_solve(ls_handle* h, const double* b, int R, double rtol, double*
   check_block(h, R);
   const double t0 = now_s();
   ensure_buffers(h, R);
+  plan_block_super(h, R);
   ls_info inf{};
   inf.bad_subdomain = -1;
   int launches = 0;
@@ -583,6 +642,7 @@ ls_status block_backward(ls_handle* h, const double* b, const double* x, const d
   check_block(h, R);
   const double t0 = now_s();
   ensure_buffers(h, R);
+  plan_block_super(h, R);
   B.G.alloc((size_t)h->n * R);
   ls_info inf{};
   inf.bad_subdomain = -1;

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <chrono>
 #include <stdexcept>
 #include <string>
@@ -136,6 +137,15 @@ struct BlockState {
   DevBuf<float> Uf, Ub, Ud;
   DevBuf<int64_t> uf_off, ub_off;
   DevBuf<int32_t> uf_row, ub_row;
+  // superblock local solve for m_R right-hand sides (m_ok: it runs), its storage made at the
+  // first block solve that uses it
+  int m_R = 0;
+  bool m_ok = false;
+  int64_t m_back = 0;  // FP32: the transposed copy's distance
+  lsq::SuperShape m_shape{};
+  DevBuf<int32_t> m_tf, m_order;
+  DevBuf<int64_t> m_toff;
+  DevBuf<unsigned char> m_fac;
   // coarse solve tiles: (problem, 32-row tile) pairs
   DevBuf<int32_t> ct_prob, ct_row, n0q;
   // mixed forms: FP32 transposed coarse basis and FP32 copy of the coarse solution
@@ -273,6 +283,35 @@ struct ls_handle {
 };
 
 namespace lsi {
+
+// Superblock storage of the block-envelope plan in factor precision prec: first tile column
+// (reaching back to the superblock's first) and byte offset of every block row, subdomains by
+// decreasing size, bytes in all.
+struct SuperHost {
+  std::vector<int32_t> tf, order;
+  std::vector<int64_t> off;
+  int64_t bytes = 0;
+};
+inline SuperHost super_storage(const std::vector<int64_t>& blk_off, const std::vector<int32_t>& blk_tf, int N,
+                               int prec) {
+  SuperHost s;
+  const size_t nblk = (size_t)blk_off[N];
+  s.tf.resize(nblk); s.off.resize(nblk); s.order.resize(N);
+  const int64_t rec = (int64_t)lsq::local_super_record(prec, false), recx = (int64_t)lsq::local_super_record(prec, true);
+  for (int i = 0; i < N; ++i) {
+    s.order[i] = i;
+    for (int64_t g = blk_off[i]; g < blk_off[i + 1]; ++g) {
+      const int b = (int)(g - blk_off[i]);
+      const int b0 = b / lsq::kSuperRows * lsq::kSuperRows;
+      s.tf[g] = std::min(blk_tf[g], b0);
+      s.off[g] = s.bytes;
+      s.bytes += (b0 - s.tf[g]) * rec + (b - b0 + 1) * recx;
+    }
+  }
+  std::stable_sort(s.order.begin(), s.order.end(),
+                   [&](int a, int b) { return blk_off[a + 1] - blk_off[a] > blk_off[b + 1] - blk_off[b]; });
+  return s;
+}
 
 inline lsq::CsrDev csr(const ls_handle* h) {
   return lsq::CsrDev{h->m, h->n, h->row_ptr.p, h->col.p, h->val.p,

@@ -59,6 +59,13 @@ struct Lanes {
   }
 };
 
+// Blocks of the per-chunk kernels: 16 warps, so that the chunks of a moderate problem (332
+// chunks of 256 columns on 152 SMs) still put 35 warps on an SM; with 8 the products with
+// A^T ran at 0.39 of the FP64 rate.  (Chunks of 128 columns fill the SMs more evenly, 177
+// against 187 us for that product, but cost the finishing blocks as much.)
+constexpr int kCT = 512;
+constexpr int kCW = kCT / 32;
+
 // Per-rhs total of v over the lane groups and warps of the block -> out[k], k < R.
 __device__ void chunk_total(double v, int Rp, int R, double* red, double* out) {
   for (int o = Rp; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -69,9 +76,41 @@ __device__ void chunk_total(double v, int Rp, int R, double* red, double* out) {
   if ((int)threadIdx.x < R) {
     double s = 0.0;
 #pragma unroll
-    for (int u = 0; u < kWarps; ++u) s += red[u * 32 + threadIdx.x];
+    for (int u = 0; u < kCW; ++u) s += red[u * 32 + threadIdx.x];
     out[threadIdx.x] = s;
   }
+}
+
+// sum over the entries [e0, e1) of val[e] X[idx[e] * R + k]: the loads of four entries at a
+// time, one accumulator (the products are bound by the FP64 units: three more additions a
+// row for independent sums made rows of six entries a third slower).
+__device__ __forceinline__ double entries_dot(const int32_t* __restrict__ idx, const double* __restrict__ val,
+                                              const double* __restrict__ X, int64_t e0, int64_t e1, int R, int k) {
+  double a = 0.0;
+  const int n = (int)(e1 - e0);
+  idx += e0;
+  val += e0;
+  X += k;
+  int e = 0;
+  for (; e + 3 < n; e += 4) {
+    double x[4], v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      v[u] = __ldg(val + e + u);
+      x[u] = __ldg(X + (int64_t)__ldg(idx + e + u) * R);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a += v[u] * x[u];
+  }
+  if (e + 1 < n) {
+    const double v0 = __ldg(val + e), v1 = __ldg(val + e + 1);
+    const double x0 = __ldg(X + (int64_t)__ldg(idx + e) * R), x1 = __ldg(X + (int64_t)__ldg(idx + e + 1) * R);
+    a += v0 * x0;
+    a += v1 * x1;
+    e += 2;
+  }
+  if (e < n) a += __ldg(val + e) * __ldg(X + (int64_t)__ldg(idx + e) * R);
+  return a;
 }
 
 // ---- sparse products ------------------------------------------------------------------
@@ -86,47 +125,27 @@ __global__ void __launch_bounds__(kThreads) k_b_spmm_csr(int64_t m, const int64_
   const int64_t wg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   if (L.k >= R) return;
-  for (int64_t r = wg * L.G + L.g; r < m; r += nw * L.G) {
-    const int64_t e0 = rp[r], e1 = rp[r + 1];
-    double a0 = 0.0, a1 = 0.0;
-    int64_t e = e0;
-    for (; e + 1 < e1; e += 2) {
-      const int32_t c0 = col[e], c1 = col[e + 1];
-      const double v0 = val[e], v1 = val[e + 1];
-      a0 += v0 * X[(int64_t)c0 * R + L.k];
-      a1 += v1 * X[(int64_t)c1 * R + L.k];
-    }
-    if (e < e1) a0 += val[e] * X[(int64_t)col[e] * R + L.k];
-    Y[r * R + L.k] = a0 + a1;
-  }
+  for (int64_t r = wg * L.G + L.g; r < m; r += nw * L.G)
+    Y[r * R + L.k] = entries_dot(col, val, X, __ldg(rp + r), __ldg(rp + r + 1), R, L.k);
 }
 
 // W = A^T Q (A^T in CSC, one lane group per column) and, with part, the per-chunk
 // partials of D . W (D == nullptr: W . W).
-__global__ void __launch_bounds__(kThreads) k_b_spmm_csc(BChunks ch, const int64_t* __restrict__ cp,
+__global__ void __launch_bounds__(kCT) k_b_spmm_csc(BChunks ch, const int64_t* __restrict__ cp,
                                                          const int32_t* __restrict__ row,
                                                          const double* __restrict__ val,
                                                          const double* __restrict__ Q, double* __restrict__ W,
                                                          int R, int Rp, const double* __restrict__ D,
                                                          double* __restrict__ part) {
-  __shared__ double red[kWarps * 32];
+  __shared__ double red[kCW * 32];
   const Lanes L(Rp);
   const int w = threadIdx.x >> 5;
   for (int64_t c = blockIdx.x; c < ch.n; c += gridDim.x) {
     const int64_t s = ch.start[c], e = ch.start[c + 1];
     double d = 0.0;
     if (L.k < R) {
-      for (int64_t j = s + w * L.G + L.g; j < e; j += kWarps * L.G) {
-        const int64_t t0 = cp[j], t1 = cp[j + 1];
-        double a0 = 0.0, a1 = 0.0;
-        int64_t t = t0;
-        for (; t + 1 < t1; t += 2) {
-          const int32_t r0 = row[t], r1 = row[t + 1];
-          a0 += val[t] * Q[(int64_t)r0 * R + L.k];
-          a1 += val[t + 1] * Q[(int64_t)r1 * R + L.k];
-        }
-        if (t < t1) a0 += val[t] * Q[(int64_t)row[t] * R + L.k];
-        const double acc = a0 + a1;
+      for (int64_t j = s + w * L.G + L.g; j < e; j += kCW * L.G) {
+        const double acc = entries_dot(row, val, Q, __ldg(cp + j), __ldg(cp + j + 1), R, L.k);
         W[j * R + L.k] = acc;
         d += (D ? D[j * R + L.k] : acc) * acc;
       }
@@ -138,11 +157,11 @@ __global__ void __launch_bounds__(kThreads) k_b_spmm_csc(BChunks ch, const int64
 // ---- CG vector kernels ----------------------------------------------------------------
 
 // X += alpha P; Rold = R (if given); R -= alpha W; partials of R . R.
-__global__ void __launch_bounds__(kThreads) k_b_update(BChunks ch, int R, int Rp, const double* __restrict__ alpha,
+__global__ void __launch_bounds__(kCT) k_b_update(BChunks ch, int R, int Rp, const double* __restrict__ alpha,
                                                        const double* __restrict__ P, const double* __restrict__ W,
                                                        double* __restrict__ X, double* __restrict__ Rv,
                                                        double* __restrict__ Rold, double* __restrict__ part) {
-  __shared__ double red[kWarps * 32];
+  __shared__ double red[kCW * 32];
   const Lanes L(Rp);
   const int w = threadIdx.x >> 5;
   for (int64_t c = blockIdx.x; c < ch.n; c += gridDim.x) {
@@ -150,7 +169,7 @@ __global__ void __launch_bounds__(kThreads) k_b_update(BChunks ch, int R, int Rp
     double d = 0.0;
     if (L.k < R) {
       const double a = alpha[(int64_t)ch.prob[c] * R + L.k];
-      for (int64_t j = s + w * L.G + L.g; j < e; j += kWarps * L.G) {
+      for (int64_t j = s + w * L.G + L.g; j < e; j += kCW * L.G) {
         const int64_t x = j * R + L.k;
         X[x] += a * P[x];
         double r = Rv[x];
@@ -165,7 +184,7 @@ __global__ void __launch_bounds__(kThreads) k_b_update(BChunks ch, int R, int Rp
 }
 
 // P = Z + beta P (init: P = Z).
-__global__ void __launch_bounds__(kThreads) k_b_pupdate(BChunks ch, int R, int Rp, const double* __restrict__ beta,
+__global__ void __launch_bounds__(kCT) k_b_pupdate(BChunks ch, int R, int Rp, const double* __restrict__ beta,
                                                         const double* __restrict__ Z, double* __restrict__ P,
                                                         int init) {
   const Lanes L(Rp);
@@ -174,27 +193,30 @@ __global__ void __launch_bounds__(kThreads) k_b_pupdate(BChunks ch, int R, int R
   for (int64_t c = blockIdx.x; c < ch.n; c += gridDim.x) {
     const int64_t s = ch.start[c], e = ch.start[c + 1];
     const double b = init ? 0.0 : beta[(int64_t)ch.prob[c] * R + L.k];
-    for (int64_t j = s + w * L.G + L.g; j < e; j += kWarps * L.G) {
+    for (int64_t j = s + w * L.G + L.g; j < e; j += kCW * L.G) {
       const int64_t x = j * R + L.k;
       P[x] = init ? Z[x] : Z[x] + b * P[x];
     }
   }
 }
 
-// Finishing block per problem: sums the chunk partials (in chunk order) and applies
-// the CG scalar step of `mode` to every right-hand side of the problem.
-__global__ void __launch_bounds__(kThreads) k_b_finish(const int64_t* __restrict__ pc_off,
+// Finishing block per problem: sums the chunk partials (in chunk order within each of its 32
+// warps, then the warps) and applies the CG scalar step of `mode` to every right-hand side of
+// the problem.
+constexpr int kFT = 1024, kFW = kFT / 32;
+__global__ void __launch_bounds__(kFT) k_b_finish(const int64_t* __restrict__ pc_off,
                                                        const double* __restrict__ part,
                                                        const double* __restrict__ part2, int R, BScal s, int mode,
                                                        int flex) {
-  __shared__ double red[kWarps][32], red2[kWarps][32];
+  __shared__ double red[kFW][32], red2[kFW][32];
   __shared__ int cnt;
   const int q = blockIdx.x;
   const int w = threadIdx.x >> 5, k = threadIdx.x & 31;
   const int64_t c0 = pc_off[q], c1 = pc_off[q + 1];
   double a = 0.0, b = 0.0;
   if (k < R) {
-    for (int64_t c = c0 + w; c < c1; c += kWarps) {
+#pragma unroll 4
+    for (int64_t c = c0 + w; c < c1; c += kFW) {
       a += part[c * 32 + k];
       if (part2) b += part2[c * 32 + k];
     }
@@ -206,7 +228,7 @@ __global__ void __launch_bounds__(kThreads) k_b_finish(const int64_t* __restrict
   if ((int)threadIdx.x < R) {
     double x = 0.0, y = 0.0;
 #pragma unroll
-    for (int u = 0; u < kWarps; ++u) {
+    for (int u = 0; u < kFW; ++u) {
       x += red[u][k];
       y += red2[u][k];
     }
@@ -248,8 +270,8 @@ __global__ void __launch_bounds__(kThreads) k_b_finish(const int64_t* __restrict
 
 // Z = sum over the copies of every column in the subdomains of Y (local solutions)
 //   + coarse prolongation; partials of R . Z and (flexible) Rold . Z.
-__global__ void __launch_bounds__(kThreads) k_b_scatter(BChunks ch, BScatterArgs a) {
-  __shared__ double red[kWarps * 32];
+__global__ void __launch_bounds__(kCT) k_b_scatter(BChunks ch, BScatterArgs a) {
+  __shared__ double red[kCW * 32];
   const Lanes L(a.Rp);
   const int R = a.R;
   const int w = threadIdx.x >> 5;
@@ -257,7 +279,7 @@ __global__ void __launch_bounds__(kThreads) k_b_scatter(BChunks ch, BScatterArgs
     const int64_t s = ch.start[c], e = ch.start[c + 1];
     double d1 = 0.0, d2 = 0.0;
     if (L.k < R) {
-      for (int64_t j = s + w * L.G + L.g; j < e; j += kWarps * L.G) {
+      for (int64_t j = s + w * L.G + L.g; j < e; j += kCW * L.G) {
         double z = 0.0;
         for (int64_t t = a.map_ptr[j]; t < a.map_ptr[j + 1]; ++t) z += a.Y[a.map_idx[t] * R + L.k];
         if (a.coarse && a.ZT) {
@@ -266,13 +288,15 @@ __global__ void __launch_bounds__(kThreads) k_b_scatter(BChunks ch, BScatterArgs
           const float4* z4 = reinterpret_cast<const float4*>(a.ZT + a.zt_off[i] + (int64_t)a.jj_of[j] * kp);
           const float* y0 = a.Y0f + (int64_t)cc * R + L.k;
           float zc = 0.f;
-          for (int t4 = 0; 4 * t4 < kk; ++t4) {
-            const float4 zz = z4[t4];
-            const int t = 4 * t4;
-            zc += zz.x * y0[(int64_t)t * R];
-            if (t + 1 < kk) zc += zz.y * y0[(int64_t)(t + 1) * R];
-            if (t + 2 < kk) zc += zz.z * y0[(int64_t)(t + 2) * R];
-            if (t + 3 < kk) zc += zz.w * y0[(int64_t)(t + 3) * R];
+          for (int t = 0; t < kk; t += 4) {  // (the padding of a column's k_i values is zero)
+            const float4 zz = __ldg(z4 + t / 4);
+            float y[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) y[u] = __ldg(y0 + (int64_t)min(t + u, kk - 1) * R);
+            zc += zz.x * y[0];
+            zc += zz.y * y[1];
+            zc += zz.z * y[2];
+            zc += zz.w * y[3];
           }
           z += (double)zc;
         } else if (a.coarse) {
@@ -293,39 +317,6 @@ __global__ void __launch_bounds__(kThreads) k_b_scatter(BChunks ch, BScatterArgs
   }
 }
 
-// R0[(c0 + t), k] = sum_jj Zbar_i[t, jj] R[Omega_I,i[jj], k] (one block per subdomain).
-__global__ void __launch_bounds__(kThreads) k_b_restrict(int R, int Rp, const int64_t* __restrict__ int_off,
-                                                         const int32_t* __restrict__ int_glob,
-                                                         const int64_t* __restrict__ zoff,
-                                                         const int32_t* __restrict__ coff, const double* __restrict__ Z,
-                                                         const double* __restrict__ Rv, double* __restrict__ R0) {
-  const int i = blockIdx.x;
-  const Lanes L(Rp);
-  const int w = threadIdx.x >> 5;
-  const int cc = coff[i], kk = coff[i + 1] - cc;
-  const int64_t io = int_off[i];
-  const int nIi = (int)(int_off[i + 1] - io);
-  const double* Zi = Z + zoff[i];
-  for (int tb = 0; tb < kk; tb += 4 * kWarps) {
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int jj = L.g; jj < nIi; jj += L.G) {
-      const double rv = L.k < R ? Rv[(int64_t)int_glob[io + jj] * R + L.k] : 0.0;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int t = tb + w + kWarps * u;
-        if (t < kk) acc[u] += Zi[(int64_t)t * nIi + jj] * rv;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      double v = acc[u];
-      for (int o = Rp; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      const int t = tb + w + kWarps * u;
-      if (t < kk && L.g == 0 && L.k < R) R0[(int64_t)(cc + t) * R + L.k] = v;
-    }
-  }
-}
-
 // FP32 transposed copy of the coarse basis: ZT[zt_off[i] + jj * kp + t] = Zbar_i[t, jj]
 // (kp = k_i rounded up to 4, so one interior column's k_i values are 16-byte aligned).
 __global__ void __launch_bounds__(kThreads) k_b_ztrans(const int64_t* __restrict__ int_off,
@@ -343,78 +334,135 @@ __global__ void __launch_bounds__(kThreads) k_b_ztrans(const int64_t* __restrict
   }
 }
 
-// FP32 restriction R0[(c0 + t), k] = sum_jj ZT[jj, t] R[Omega_I,i[jj], k] for the mixed
-// forms: warps split the interior columns, lane k keeps 32 coarse sums in registers,
-// the warps' sums meet in shared memory.
-__global__ void __launch_bounds__(kThreads) k_b_restrict32(int R, const int64_t* __restrict__ int_off,
-                                                           const int32_t* __restrict__ int_glob,
-                                                           const int32_t* __restrict__ coff,
-                                                           const int64_t* __restrict__ zt_off,
-                                                           const float* __restrict__ ZT,
-                                                           const double* __restrict__ Rv, double* __restrict__ R0) {
-  __shared__ float red[kWarps][32][33];
-  const int i = blockIdx.x;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int cc = coff[i], kk = coff[i + 1] - cc, kp = (kk + 3) & ~3;
+// Restriction R0[(c0 + t), k] = sum_jj Zbar_i[t, jj] R[Omega_I,i[jj], k], in FP64 from Zbar (TA =
+// double) or, for the mixed forms, in FP32 from its transposed copy ZT (TA = float).  One
+// block per subdomain (blockIdx.x) and 16 coarse vectors (blockIdx.y): its lane groups split
+// the interior columns, each keeps the 16 sums of one right-hand side in registers, and the
+// groups' sums meet in shared memory.  Bound by the latency of the gathers: 32 warps, all
+// lanes in use for any R (32 / Rp columns per warp) and two columns in flight (eight warps,
+// one column each, lanes above R idle: 122 us for 64 subdomains of 1,024 columns and 8
+// right-hand sides, 155 us for 93 and 32).
+constexpr int kRV = 16, kRT = 1024, kRW = kRT / 32;
+template <class TA>
+__global__ void __launch_bounds__(kRT) k_b_restrict(int R, int Rp, const int64_t* __restrict__ int_off,
+                                                    const int32_t* __restrict__ int_glob,
+                                                    const int64_t* __restrict__ zoff, const int32_t* __restrict__ coff,
+                                                    const double* __restrict__ Z, const int64_t* __restrict__ zt_off,
+                                                    const float* __restrict__ ZT, const double* __restrict__ Rv,
+                                                    double* __restrict__ R0) {
+  constexpr int kPass = 32 / (int)sizeof(TA);  // vectors per pass through shared memory
+  __shared__ TA red[kRW][kPass][33];
+  const int i = blockIdx.x, tb = blockIdx.y * kRV;
+  const Lanes L(Rp);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cc = coff[i], kk = coff[i + 1] - cc;
+  if (tb >= kk) return;
+  const int tn = min(kRV, kk - tb);
   const int64_t io = int_off[i];
   const int nIi = (int)(int_off[i + 1] - io);
-  const float* Zi = ZT + zt_off[i];
-  for (int tb = 0; tb < kk; tb += 32) {
-    const int tn = min(32, kk - tb);
-    float acc[32];
+  TA acc[kRV];
 #pragma unroll
-    for (int t = 0; t < 32; ++t) acc[t] = 0.f;
-    for (int jj = w; jj < nIi; jj += kWarps) {
-      const float rv = lane < R ? (float)Rv[(int64_t)int_glob[io + jj] * R + lane] : 0.f;
-      const float4* z4 = reinterpret_cast<const float4*>(Zi + (int64_t)jj * kp + tb);
+  for (int t = 0; t < kRV; ++t) acc[t] = 0;
+  const bool on = L.k < R;
+#pragma unroll 2
+  for (int jj = w * L.G + L.g; jj < nIi; jj += kRW * L.G) {
+    const TA rv = on ? (TA)Rv[(int64_t)__ldg(int_glob + io + jj) * R + L.k] : (TA)0;
+    if constexpr (sizeof(TA) == 4) {
+      const int kp = (kk + 3) & ~3;
+      const float4* z4 = reinterpret_cast<const float4*>(ZT + zt_off[i] + (int64_t)jj * kp + tb);
 #pragma unroll
-      for (int t4 = 0; t4 < 8; ++t4) {
+      for (int t4 = 0; t4 < kRV / 4; ++t4)
         if (4 * t4 < tn) {
-          const float4 z = z4[t4];
+          const float4 z = __ldg(z4 + t4);
           acc[4 * t4 + 0] += z.x * rv; acc[4 * t4 + 1] += z.y * rv;
           acc[4 * t4 + 2] += z.z * rv; acc[4 * t4 + 3] += z.w * rv;
         }
-      }
-    }
+    } else {
+      const double* z = Z + zoff[i] + (int64_t)tb * nIi + jj;
 #pragma unroll
-    for (int t = 0; t < 32; ++t) red[w][t][lane] = acc[t];
-    __syncthreads();
-    for (int e = threadIdx.x; e < tn * 32; e += blockDim.x) {
-      const int t = e >> 5, k = e & 31;
-      float s = 0.f;
-#pragma unroll
-      for (int u = 0; u < kWarps; ++u) s += red[u][t][k];
-      if (k < R) R0[(int64_t)(cc + tb + t) * R + k] = (double)s;
+      for (int t = 0; t < kRV; ++t)
+        if (t < tn) acc[t] += __ldg(z + (int64_t)t * nIi) * rv;
     }
+  }
+#pragma unroll
+  for (int t = 0; t < kRV; ++t)
+    for (int o = Rp; o < 32; o <<= 1) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], o);
+#pragma unroll
+  for (int p = 0; p < kRV; p += kPass) {
+    if (p >= tn) break;
     __syncthreads();
+#pragma unroll
+    for (int t = 0; t < kPass; ++t)
+      if (lane < Rp) red[w][t][lane] = acc[p + t];
+    __syncthreads();
+    for (int e = threadIdx.x; e < kPass * R; e += kRT) {
+      const int t = e / R, k = e % R;
+      if (p + t >= tn) continue;
+      TA s = 0;
+#pragma unroll
+      for (int u = 0; u < kRW; ++u) s += red[u][t][k];
+      R0[(int64_t)(cc + tb + p + t) * R + k] = (double)s;
+    }
   }
 }
 
-// Y0 = C00_q^{-1} R0 on every problem's dense block; one block per (problem, 32-row tile).
-__global__ void __launch_bounds__(kThreads) k_b_coarse(int R, const int32_t* __restrict__ ct_prob,
+// Y0 = C00_q^{-1} R0 on every problem's dense block; one block per (problem, 32-row tile)
+// and eight of its rows (blockIdx.y).  The block's lane groups split the columns, each
+// keeping its eight rows' sums of one right-hand side in registers (a warp per four rows
+// over all columns, lanes above R idle, was one dependent chain of 487 loads in 16 blocks:
+// 148 us for n0 = 487 and 8 right-hand sides).
+constexpr int kCR = 8;
+__global__ void __launch_bounds__(kThreads) k_b_coarse(int R, int Rp, const int32_t* __restrict__ ct_prob,
                                                        const int32_t* __restrict__ ct_row, CoarseBlocks cb,
                                                        const int32_t* __restrict__ n0q, const double* __restrict__ Xinv,
                                                        const double* __restrict__ R0, double* __restrict__ Y0,
                                                        float* __restrict__ Y0f) {
-  const int q = ct_prob[blockIdx.x], rt = ct_row[blockIdx.x];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane >= R) return;
+  __shared__ double red[kWarps][kCR][33];
+  const int q = ct_prob[blockIdx.x], rbase = ct_row[blockIdx.x] * 32 + blockIdx.y * kCR;
+  const Lanes L(Rp);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t ld = cb.ld[q];
   const int c0 = cb.c0[q], nq = n0q[q];
-  const double* X = Xinv + cb.base[q];
-  const int rbase = rt * 32 + 4 * w;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int c = 0; c < nq; ++c) {
-    const double rv = R0[(int64_t)(c0 + c) * R + lane];
+  if (rbase >= nq) return;
+  const double* X = Xinv + cb.base[q] + (int64_t)rbase * ld;  // (the block is padded to 32 rows)
+  double acc[kCR];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u] += X[(int64_t)(rbase + u) * ld + c] * rv;
+  for (int u = 0; u < kCR; ++u) acc[u] = 0.0;
+  const bool on = L.k < R;
+  const int step = kWarps * L.G;
+  for (int c = w * L.G + L.g; c < nq; c += 2 * step) {
+    const bool two = c + step < nq;
+    const int c2 = two ? c + step : c;
+    double x[kCR], x2[kCR];  // (all loads of the two columns before the first product)
+#pragma unroll
+    for (int u = 0; u < kCR; ++u) {
+      x[u] = __ldg(X + (int64_t)u * ld + c);
+      x2[u] = __ldg(X + (int64_t)u * ld + c2);
+    }
+    const double rv = on ? __ldg(R0 + (int64_t)(c0 + c) * R + L.k) : 0.0;
+    const double rv2 = on && two ? __ldg(R0 + (int64_t)(c0 + c2) * R + L.k) : 0.0;
+#pragma unroll
+    for (int u = 0; u < kCR; ++u) acc[u] += x[u] * rv;
+    if (two) {
+#pragma unroll
+      for (int u = 0; u < kCR; ++u) acc[u] += x2[u] * rv2;
+    }
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
-    if (rbase + u < nq) {
-      Y0[(int64_t)(c0 + rbase + u) * R + lane] = acc[u];
-      if (Y0f) Y0f[(int64_t)(c0 + rbase + u) * R + lane] = (float)acc[u];
-    }
+  for (int u = 0; u < kCR; ++u) {
+    for (int o = Rp; o < 32; o <<= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+    if (lane < Rp) red[w][u][lane] = acc[u];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < kCR * R; e += kThreads) {
+    const int u = e / R, k = e % R;
+    if (rbase + u >= nq) continue;
+    double s = 0.0;
+#pragma unroll
+    for (int v = 0; v < kWarps; ++v) s += red[v][u][k];
+    Y0[(int64_t)(c0 + rbase + u) * R + k] = s;
+    if (Y0f) Y0f[(int64_t)(c0 + rbase + u) * R + k] = (float)s;
+  }
 }
 
 // ---- layout conversions ---------------------------------------------------------------
@@ -476,16 +524,16 @@ __global__ void __launch_bounds__(kThreads) k_b_store_rows(int64_t m, int R, int
 
 // W = G - W with the per-chunk partials of W . W (the residual of C x = g when W = C x;
 // with W = 0 beforehand it copies G and gives ||G||^2).
-__global__ void __launch_bounds__(kThreads) k_b_resid(BChunks ch, int R, int Rp, const double* __restrict__ G,
+__global__ void __launch_bounds__(kCT) k_b_resid(BChunks ch, int R, int Rp, const double* __restrict__ G,
                                                       double* __restrict__ W, double* __restrict__ part) {
-  __shared__ double red[kWarps * 32];
+  __shared__ double red[kCW * 32];
   const Lanes L(Rp);
   const int w = threadIdx.x >> 5;
   for (int64_t c = blockIdx.x; c < ch.n; c += gridDim.x) {
     const int64_t s = ch.start[c], e = ch.start[c + 1];
     double d = 0.0;
     if (L.k < R) {
-      for (int64_t j = s + w * L.G + L.g; j < e; j += kWarps * L.G) {
+      for (int64_t j = s + w * L.G + L.g; j < e; j += kCW * L.G) {
         const int64_t x = j * R + L.k;
         const double v = G[x] - W[x];
         W[x] = v;
@@ -1158,39 +1206,42 @@ void launch_b_spmm_csr(const CsrDev& A, const double* X, double* Y, int R, cudaS
 
 void launch_b_spmm_csc(const BChunks& ch, const CscDev& At, const double* Q, double* W, int R, const double* D,
                        double* part, cudaStream_t st) {
-  k_b_spmm_csc<<<grid_chunks(ch.n), kThreads, 0, st>>>(ch, At.col_ptr, At.row, At.val, Q, W, R, pow2_at_least(R), D,
+  k_b_spmm_csc<<<grid_chunks(ch.n), kCT, 0, st>>>(ch, At.col_ptr, At.row, At.val, Q, W, R, pow2_at_least(R), D,
                                                       part);
 }
 
 void launch_b_update(const BChunks& ch, int R, const double* alpha, const double* P, const double* W, double* X,
                      double* Rv, double* Rold, double* part, cudaStream_t st) {
-  k_b_update<<<grid_chunks(ch.n), kThreads, 0, st>>>(ch, R, pow2_at_least(R), alpha, P, W, X, Rv, Rold, part);
+  k_b_update<<<grid_chunks(ch.n), kCT, 0, st>>>(ch, R, pow2_at_least(R), alpha, P, W, X, Rv, Rold, part);
 }
 
 void launch_b_pupdate(const BChunks& ch, int R, const double* beta, const double* Z, double* P, int init,
                       cudaStream_t st) {
-  k_b_pupdate<<<grid_chunks(ch.n), kThreads, 0, st>>>(ch, R, pow2_at_least(R), beta, Z, P, init);
+  k_b_pupdate<<<grid_chunks(ch.n), kCT, 0, st>>>(ch, R, pow2_at_least(R), beta, Z, P, init);
 }
 
 void launch_b_finish(int nprob, const int64_t* pc_off, const double* part, const double* part2, int R,
                      const BScal& s, int mode, int flex, cudaStream_t st) {
-  k_b_finish<<<nprob, kThreads, 0, st>>>(pc_off, part, part2, R, s, mode, flex);
+  k_b_finish<<<nprob, kFT, 0, st>>>(pc_off, part, part2, R, s, mode, flex);
 }
 
 void launch_b_scatter(const BChunks& ch, const BScatterArgs& a, cudaStream_t st) {
-  k_b_scatter<<<grid_chunks(ch.n), kThreads, 0, st>>>(ch, a);
+  k_b_scatter<<<grid_chunks(ch.n), kCT, 0, st>>>(ch, a);
 }
 
-void launch_b_restrict(int N, int R, const int64_t* int_off, const int32_t* int_glob, const int64_t* zoff,
+void launch_b_restrict(int N, int kmax, int R, const int64_t* int_off, const int32_t* int_glob, const int64_t* zoff,
                        const int32_t* coff, const double* Z, const double* Rv, double* R0, cudaStream_t st) {
-  k_b_restrict<<<N, kThreads, 0, st>>>(R, pow2_at_least(R), int_off, int_glob, zoff, coff, Z, Rv, R0);
+  const dim3 grid((unsigned)N, (unsigned)((kmax + kRV - 1) / kRV));
+  if (kmax > 0)
+    k_b_restrict<double><<<grid, kRT, 0, st>>>(R, pow2_at_least(R), int_off, int_glob, zoff, coff, Z, nullptr, nullptr,
+                                               Rv, R0);
 }
 
 void launch_b_coarse(int ntiles, int R, const int32_t* ct_prob, const int32_t* ct_row, const CoarseBlocks& cb,
                      const int32_t* n0q, const double* Xinv, const double* R0, double* Y0, float* Y0f,
                      cudaStream_t st) {
   if (ntiles <= 0) return;
-  k_b_coarse<<<ntiles, kThreads, 0, st>>>(R, ct_prob, ct_row, cb, n0q, Xinv, R0, Y0, Y0f);
+  k_b_coarse<<<dim3((unsigned)ntiles, 32 / kCR), kThreads, 0, st>>>(R, pow2_at_least(R), ct_prob, ct_row, cb, n0q, Xinv, R0, Y0, Y0f);
 }
 
 void launch_b_ztrans(int N, const int64_t* int_off, const int64_t* zoff, const int32_t* coff, const int64_t* zt_off,
@@ -1198,9 +1249,12 @@ void launch_b_ztrans(int N, const int64_t* int_off, const int64_t* zoff, const i
   k_b_ztrans<<<N, kThreads, 0, st>>>(int_off, zoff, coff, zt_off, Z, ZT);
 }
 
-void launch_b_restrict32(int N, int R, const int64_t* int_off, const int32_t* int_glob, const int32_t* coff,
+void launch_b_restrict32(int N, int kmax, int R, const int64_t* int_off, const int32_t* int_glob, const int32_t* coff,
                          const int64_t* zt_off, const float* ZT, const double* Rv, double* R0, cudaStream_t st) {
-  k_b_restrict32<<<N, kThreads, 0, st>>>(R, int_off, int_glob, coff, zt_off, ZT, Rv, R0);
+  const dim3 grid((unsigned)N, (unsigned)((kmax + kRV - 1) / kRV));
+  if (kmax > 0)
+    k_b_restrict<float><<<grid, kRT, 0, st>>>(R, pow2_at_least(R), int_off, int_glob, nullptr, coff, nullptr, zt_off,
+                                              ZT, Rv, R0);
 }
 
 void launch_b_load_rows(int64_t m, int R, const int32_t* perm, const double* Bu, double* Bb, cudaStream_t st) {
@@ -1224,7 +1278,7 @@ void launch_b_store_rows(int64_t m, int R, const int32_t* perm, const double* Yb
 }
 
 void launch_b_resid(const BChunks& ch, int R, const double* G, double* W, double* part, cudaStream_t st) {
-  k_b_resid<<<grid_chunks(ch.n), kThreads, 0, st>>>(ch, R, pow2_at_least(R), G, W, part);
+  k_b_resid<<<grid_chunks(ch.n), kCT, 0, st>>>(ch, R, pow2_at_least(R), G, W, part);
 }
 
 void launch_b_grad_vals(const CsrDev& A, const int64_t* entmap, int R, const double* rho, const double* lam,

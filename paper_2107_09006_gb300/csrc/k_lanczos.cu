@@ -718,6 +718,7 @@ bool run_lanczos_grid(const EigArgs& a, const LanczosGrid& g, cudaStream_t st) {
   bwd.dst = a.vec; bwd.dst_stride = 2 * a.vstride;
   bwd.skip = g.state + 2 * N;
   bwd.sweeps = 2;
+  bwd.R = 1;
   bwd.err = g.err;
   SuperArgs fwd = bwd;
   fwd.src = a.vec + a.vstride;  // x2 <- L^{-1} x2

@@ -149,6 +149,41 @@ __device__ __forceinline__ void send(uint32_t a, double v, uint32_t bar) {
                : "memory");
 }
 
+// NR right-hand sides of one vector entry.
+template <class TA, int NR>
+struct alignas(NR == 1 ? sizeof(TA) : 16) Vec {
+  TA a[NR];
+  __device__ __forceinline__ Vec& operator+=(const Vec& o) {
+#pragma unroll
+    for (int n = 0; n < NR; ++n) a[n] += o.a[n];
+    return *this;
+  }
+  __device__ __forceinline__ Vec operator+(const Vec& o) const {
+    Vec r = *this;
+    r += o;
+    return r;
+  }
+  __device__ __forceinline__ Vec operator-(const Vec& o) const {
+    Vec r;
+#pragma unroll
+    for (int n = 0; n < NR; ++n) r.a[n] = a[n] - o.a[n];
+    return r;
+  }
+  __device__ __forceinline__ void fma(TA t, const Vec& o) {  // += t o
+#pragma unroll
+    for (int n = 0; n < NR; ++n) a[n] += t * o.a[n];
+  }
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int n = 0; n < NR; ++n) a[n] = 0;
+  }
+};
+template <class TA, int NR>
+__device__ __forceinline__ void send(uint32_t at, const Vec<TA, NR>& v, uint32_t bar) {
+#pragma unroll
+  for (int n = 0; n < NR; ++n) send(at + n * (uint32_t)sizeof(TA), v.a[n], bar);
+}
+
 // Units of one storage type: UC columns of 32 rows, U units a tile; a panel tile takes REC
 // bytes, a tile of X RECX, a unit UB (of the types that pass through the ring).
 template <class TF> struct Unit;
@@ -157,18 +192,20 @@ template <> struct Unit<float> { static constexpr int UC = 32, U = 1, REC = 4096
 template <> struct Unit<__nv_bfloat16> { static constexpr int UC = 32, U = 1, REC = 2064, RECX = 4096, UB = 4096; };
 
 // Shared memory: [NW][depth] unit slots | full, empty barriers [NW][depth], message
-// barriers [6], abort flag | red [NW][32] | ub [Q][32] | ws [2][Q][32] | dbuf [2][kItems][32] |
+// barriers [6], abort flag | red [NW][32] | ub [Q][32] | ws [1 or 2][Q][32] | dbuf [1 or 2][kItems][32] |
 // xbuf [2][C][Q][32] (C > 1) | acc4 [Q][ring][32] | v [nb][32] | tf [nb], toff [nb].
-template <class TF, class TA, int NW, int C>
+template <class TF, class V, int NW, int C>
 struct Layout {
   static constexpr int kItems = Unit<TF>::U * kQ * (kQ + 1) / 2;
-  static constexpr int kRed = NW * 32, kUb = kQ * 32, kWs = 2 * kQ * 32, kDb = 2 * kItems * 32,
+  // (a cluster's FP64 X shares and its w_s alternate between two places)
+  static constexpr int kRed = NW * 32, kUb = kQ * 32, kWs = (C > 1 ? 2 : 1) * kQ * 32,
+                       kDb = (C > 1 && sizeof(TF) == 8 ? 2 : 1) * kItems * 32,
                        kXb = C > 1 ? 2 * C * kQ * 32 : 0;
   // (depth 0: no ring, the units are loaded into registers)
   __host__ __device__ static size_t bars(int depth) { return (size_t)NW * depth * Unit<TF>::UB; }
   __host__ __device__ static size_t red(int depth) { return bars(depth) + (size_t)(2 * NW * depth + 6 + 2) * 8; }
   __host__ __device__ static size_t total(int depth, int nb, int ring) {
-    return red(depth) + (size_t)(kRed + kUb + kWs + kDb + kXb + kQ * ring * 32 + nb * kT) * sizeof(TA) +
+    return red(depth) + (size_t)(kRed + kUb + kWs + kDb + kXb + kQ * ring * 32 + nb * kT) * sizeof(V) +
            (size_t)2 * nb * 4;
   }
 };
@@ -183,6 +220,7 @@ struct UnitList {
   const int32_t* toff;
   int nb, nsb, q, cls, clx;
   int sweeps;  // 1 forward, 2 backward, 3 both
+  int64_t back;  // bytes from a unit to its copy for the backward sweep (0: the same)
   int s = 0, sweep = 0, ph = -1, u = 0, end = 0, step = 0;
   int64_t row = 0;  // byte offset that tile column 0 of the row would have, tiles of rec bytes
   int rec = 0;
@@ -225,7 +263,7 @@ struct UnitList {
   }
   __device__ bool done() const { return sweep == 2; }
   __device__ bool is_x() const { return ph != sweep; }
-  __device__ int64_t offset() const { return row + (int64_t)(u / U) * rec + (u % U) * K::UB; }
+  __device__ int64_t offset() const { return row + (int64_t)(u / U) * rec + (u % U) * K::UB + (sweep == 1 ? back : 0); }
   __device__ void next() {
     u += step;
     if (u >= end) seek();
@@ -240,42 +278,64 @@ struct UnitList {
 // FP64 units in shared memory: lane = row, forward; lane (h, c) sums the rows [16 h, 16 h +
 // 16) of column c, backward, 16-byte reads in a lane-rotated order (eight lanes hit eight
 // bank groups).
+template <int NR>
 struct RingUnit {
   using T = double;
+  using V = Vec<double, NR>;
   __device__ __forceinline__ RingUnit& X() { return *this; }
-  double acc;
-  const double* x;
-  __device__ __forceinline__ void zero() { acc = 0.0; }
-  __device__ __forceinline__ void fwd(const unsigned char* unit, const double* v, int lane) {
+  V acc;
+  const V* x;
+  __device__ __forceinline__ void zero() { acc.clear(); }
+  __device__ __forceinline__ void fwd(const unsigned char* unit, const V* v, int lane) {
     const double* t = reinterpret_cast<const double*>(unit) + lane;
-    double s0 = 0.0, s1 = 0.0;
+    if constexpr (NR == 1) {
+      double s0 = 0.0, s1 = 0.0;
 #pragma unroll
-    for (int c = 0; c < 16; c += 2) {
-      const double2 w = *reinterpret_cast<const double2*>(v + c);
-      s0 += t[c * 32] * w.x;
-      s1 += t[(c + 1) * 32] * w.y;
+      for (int c = 0; c < 16; c += 2) {
+        const double2 w = *reinterpret_cast<const double2*>(v + c);
+        s0 += t[c * 32] * w.x;
+        s1 += t[(c + 1) * 32] * w.y;
+      }
+      acc.a[0] += s0 + s1;
+    } else {
+#pragma unroll
+      for (int c = 0; c < 16; ++c) acc.fma(t[c * 32], v[c]);
     }
-    acc += s0 + s1;
   }
-  __device__ __forceinline__ double out(int lane, int& r) {
+  __device__ __forceinline__ V out(int lane, int& r) {
     r = lane;
     return acc;
   }
-  __device__ __forceinline__ void load_x(const double* xs, int) { x = xs; }
-  __device__ __forceinline__ double bwd(const unsigned char* unit, int lane, int& c) const {
+  __device__ __forceinline__ void load_x(const V* xs, int) { x = xs; }
+  __device__ __forceinline__ V bwd(const unsigned char* unit, int lane, int& c) const {
     const double2* t2 = reinterpret_cast<const double2*>(reinterpret_cast<const double*>(unit) + (lane & 15) * 32 + (lane >> 4) * 16);
-    const double2* x2 = reinterpret_cast<const double2*>(x + (lane >> 4) * 16);
-    double s0 = 0.0, s1 = 0.0;
+    V s;
+    if constexpr (NR == 1) {
+      const double2* x2 = reinterpret_cast<const double2*>(x + (lane >> 4) * 16);
+      double s0 = 0.0, s1 = 0.0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int j = (k + lane) & 7;
-      const double2 t = t2[j], y = x2[j];
-      s0 += t.x * y.x;
-      s1 += t.y * y.y;
+      for (int k = 0; k < 8; ++k) {
+        const int j = (k + lane) & 7;
+        const double2 t = t2[j], y = x2[j];
+        s0 += t.x * y.x;
+        s1 += t.y * y.y;
+      }
+      s.a[0] = s0 + s1;
+    } else {
+      const V* xr = x + (lane >> 4) * 16;
+      s.clear();
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int j = (k + lane) & 7;
+        const double2 t = t2[j];
+        s.fma(t.x, xr[2 * j]);
+        s.fma(t.y, xr[2 * j + 1]);
+      }
     }
-    s0 += s1;
     c = lane & 15;
-    return s0 + __shfl_xor_sync(0xffffffffu, s0, 16);
+#pragma unroll
+    for (int n = 0; n < NR; ++n) s.a[n] += __shfl_xor_sync(0xffffffffu, s.a[n], 16);
+    return s;
   }
 };
 
@@ -292,57 +352,81 @@ __device__ __forceinline__ void fold(float* a, int o, int lane) {
 }
 
 // FP32 units in registers: load k of lane l holds rows 4 (l % 8) .. + 3 of column 4 k + l / 8.
+template <int NR>
 struct RegUnit32 {
   using T = float;
+  using V = Vec<float, NR>;
   __device__ __forceinline__ RegUnit32& X() { return *this; }
   float4 t[8];
-  float acc[4], x[4];
+  V acc[4], x[4];
   __device__ __forceinline__ void load(const unsigned char* unit, int lane) {
     const float4* p = reinterpret_cast<const float4*>(unit) + lane;
 #pragma unroll
     for (int k = 0; k < 8; ++k) t[k] = __ldcg(p + 32 * k);
   }
-  __device__ __forceinline__ void zero() { acc[0] = acc[1] = acc[2] = acc[3] = 0.f; }
-  __device__ __forceinline__ void fwd(const unsigned char*, const float* v, int lane) {
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k].clear();
+  }
+  __device__ __forceinline__ void fwd(const unsigned char*, const V* v, int lane) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const float w = v[4 * k + (lane >> 3)];
-      acc[0] += t[k].x * w;
-      acc[1] += t[k].y * w;
-      acc[2] += t[k].z * w;
-      acc[3] += t[k].w * w;
+      const V w = v[4 * k + (lane >> 3)];
+      acc[0].fma(t[k].x, w);
+      acc[1].fma(t[k].y, w);
+      acc[2].fma(t[k].z, w);
+      acc[3].fma(t[k].w, w);
     }
   }
-  __device__ __forceinline__ float out(int lane, int& r) {
-    fold<2>(acc, 16, lane);
-    fold<1>(acc, 8, lane);
-    r = 4 * (lane & 7) + ((lane >> 4) & 1) * 2 + ((lane >> 3) & 1);
-    return acc[0];
-  }
-  __device__ __forceinline__ void load_x(const float* xs, int lane) {
-    const float4 y = *reinterpret_cast<const float4*>(xs + 4 * (lane & 7));
-    x[0] = y.x; x[1] = y.y; x[2] = y.z; x[3] = y.w;
-  }
-  __device__ __forceinline__ float bwd(const unsigned char*, int lane, int& c) const {
-    float p[8];
+  __device__ __forceinline__ V out(int lane, int& r) {
+    V o;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) p[k] = (t[k].x * x[0] + t[k].y * x[1]) + (t[k].z * x[2] + t[k].w * x[3]);
-    fold<4>(p, 4, lane);
-    fold<2>(p, 2, lane);
-    fold<1>(p, 1, lane);
+    for (int n = 0; n < NR; ++n) {
+      float p[4] = {acc[0].a[n], acc[1].a[n], acc[2].a[n], acc[3].a[n]};
+      fold<2>(p, 16, lane);
+      fold<1>(p, 8, lane);
+      o.a[n] = p[0];
+    }
+    r = 4 * (lane & 7) + ((lane >> 4) & 1) * 2 + ((lane >> 3) & 1);
+    return o;
+  }
+  __device__ __forceinline__ void load_x(const V* xs, int lane) {
+    if constexpr (NR == 1) {
+      const float4 y = *reinterpret_cast<const float4*>(xs + 4 * (lane & 7));
+      x[0].a[0] = y.x; x[1].a[0] = y.y; x[2].a[0] = y.z; x[3].a[0] = y.w;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) x[k] = xs[4 * (lane & 7) + k];
+    }
+  }
+  __device__ __forceinline__ V bwd(const unsigned char*, int lane, int& c) const {
+    V o;
+#pragma unroll
+    for (int n = 0; n < NR; ++n) {
+      float p[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        p[k] = (t[k].x * x[0].a[n] + t[k].y * x[1].a[n]) + (t[k].z * x[2].a[n] + t[k].w * x[3].a[n]);
+      fold<4>(p, 4, lane);
+      fold<2>(p, 2, lane);
+      fold<1>(p, 1, lane);
+      o.a[n] = p[0];
+    }
     c = 4 * (lane & 7) + (lane >> 3);
-    return p[0];
+    return o;
   }
 };
 
 // BF16 units in registers: load k of lane l holds rows 8 (l % 4) .. + 7 of column 8 k + l / 4.
 // The tiles of X are FP32 (RegUnit32 in the same registers).
+template <int NR>
 struct RegUnit16 {
   using T = __nv_bfloat16;
-  RegUnit32 f;
+  using V = Vec<float, NR>;
+  RegUnit32<NR> f;
   float sc;
-  float acc[8], x[8];
-  __device__ __forceinline__ RegUnit32& X() { return f; }
+  V acc[8], x[8];
+  __device__ __forceinline__ RegUnit32<NR>& X() { return f; }
   __device__ __forceinline__ void load(const unsigned char* unit, int lane) {
     sc = __ldcg(reinterpret_cast<const float*>(unit));
     const float4* p = reinterpret_cast<const float4*>(unit + 16) + lane;
@@ -351,56 +435,173 @@ struct RegUnit16 {
   }
   __device__ __forceinline__ void zero() {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+    for (int k = 0; k < 8; ++k) acc[k].clear();
   }
   static __device__ __forceinline__ float lo(float w) { return __uint_as_float(__float_as_uint(w) << 16); }
   static __device__ __forceinline__ float hi(float w) { return __uint_as_float(__float_as_uint(w) & 0xffff0000u); }
-  __device__ __forceinline__ void fwd(const unsigned char*, const float* v, int lane) {
+  __device__ __forceinline__ void fwd(const unsigned char*, const V* v, int lane) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const float w = v[8 * k + (lane >> 2)] * sc;
+      V w = v[8 * k + (lane >> 2)];
+#pragma unroll
+      for (int n = 0; n < NR; ++n) w.a[n] *= sc;
       const float4 t = f.t[k];
-      acc[0] += lo(t.x) * w; acc[1] += hi(t.x) * w;
-      acc[2] += lo(t.y) * w; acc[3] += hi(t.y) * w;
-      acc[4] += lo(t.z) * w; acc[5] += hi(t.z) * w;
-      acc[6] += lo(t.w) * w; acc[7] += hi(t.w) * w;
+      acc[0].fma(lo(t.x), w); acc[1].fma(hi(t.x), w);
+      acc[2].fma(lo(t.y), w); acc[3].fma(hi(t.y), w);
+      acc[4].fma(lo(t.z), w); acc[5].fma(hi(t.z), w);
+      acc[6].fma(lo(t.w), w); acc[7].fma(hi(t.w), w);
     }
   }
-  __device__ __forceinline__ float out(int lane, int& r) {
-    fold<4>(acc, 16, lane);
-    fold<2>(acc, 8, lane);
-    fold<1>(acc, 4, lane);
+  __device__ __forceinline__ V out(int lane, int& r) {
+    V o;
+#pragma unroll
+    for (int n = 0; n < NR; ++n) {
+      float p[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) p[k] = acc[k].a[n];
+      fold<4>(p, 16, lane);
+      fold<2>(p, 8, lane);
+      fold<1>(p, 4, lane);
+      o.a[n] = p[0];
+    }
     r = 8 * (lane & 3) + ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
-    return acc[0];
+    return o;
   }
-  __device__ __forceinline__ void load_x(const float* xs, int lane) {
-    const float4 a = *reinterpret_cast<const float4*>(xs + 8 * (lane & 3));
-    const float4 b = *reinterpret_cast<const float4*>(xs + 8 * (lane & 3) + 4);
-    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
-    x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
-  }
-  __device__ __forceinline__ float bwd(const unsigned char*, int lane, int& c) const {
-    float p[4];
+  __device__ __forceinline__ void load_x(const V* xs, int lane) {
+    if constexpr (NR == 1) {
+      const float4 a = *reinterpret_cast<const float4*>(xs + 8 * (lane & 3));
+      const float4 b = *reinterpret_cast<const float4*>(xs + 8 * (lane & 3) + 4);
+      x[0].a[0] = a.x; x[1].a[0] = a.y; x[2].a[0] = a.z; x[3].a[0] = a.w;
+      x[4].a[0] = b.x; x[5].a[0] = b.y; x[6].a[0] = b.z; x[7].a[0] = b.w;
+    } else {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float4 t = f.t[k];
-      p[k] = ((lo(t.x) * x[0] + hi(t.x) * x[1]) + (lo(t.y) * x[2] + hi(t.y) * x[3])) +
-             ((lo(t.z) * x[4] + hi(t.z) * x[5]) + (lo(t.w) * x[6] + hi(t.w) * x[7]));
+      for (int k = 0; k < 8; ++k) x[k] = xs[8 * (lane & 3) + k];
     }
-    fold<2>(p, 2, lane);
-    fold<1>(p, 1, lane);
+  }
+  __device__ __forceinline__ V bwd(const unsigned char*, int lane, int& c) const {
+    V o;
+#pragma unroll
+    for (int n = 0; n < NR; ++n) {
+      float p[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float4 t = f.t[k];
+        p[k] = ((lo(t.x) * x[0].a[n] + hi(t.x) * x[1].a[n]) + (lo(t.y) * x[2].a[n] + hi(t.y) * x[3].a[n])) +
+               ((lo(t.z) * x[4].a[n] + hi(t.z) * x[5].a[n]) + (lo(t.w) * x[6].a[n] + hi(t.w) * x[7].a[n]));
+      }
+      fold<2>(p, 2, lane);
+      fold<1>(p, 1, lane);
+      o.a[n] = p[0] * sc;
+    }
     c = 8 * (lane & 3) + (lane >> 2);
-    return p[0] * sc;
+    return o;
   }
 };
 
-// P: how the units reach the FMAs (RingUnit, RegUnit32, RegUnit16); NW consumer warps, OCC
-// CTAs per SM, C CTAs per subdomain.
-template <class P, class TA, int NW, int OCC, int C>
-__global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_local_super(SuperArgs a) {
+// Eight right-hand sides on the tensor cores (FP32 factors of the multi right-hand-side path):
+// the tile is stored in the order of m16n8k8's A fragments (lane 4 g + t: rows g, g + 8,
+// columns t, t + 4 of every 16 x 8 piece), a second copy transposed for the backward sweep, so
+// a unit goes from memory into the registers the MMAs read and both sweeps are the same
+// product.  The tiles of L are TF32, the vector entries split into a TF32 head and tail; the
+// FP32 tiles of X are split too (the tail-tail product, below 2^-22, is left out).  On the
+// FP32 units eight right-hand sides take 256 FMAs, 64 shared-memory wavefronts and, backward,
+// 56 shuffles a tile; here 16 MMAs and 8 conflict-free reads.
+struct MmaUnit32 {
+  using T = float;
+  using V = Vec<float, 8>;
+  struct Exact {  // the tiles of X
+    MmaUnit32& u;
+    __device__ __forceinline__ void load(const unsigned char* unit, int lane) { u.load(unit, lane); }
+    __device__ __forceinline__ void zero() { u.zero(); }
+    __device__ __forceinline__ void fwd(const unsigned char*, const V* v, int lane) { u.product<true>(v, lane); }
+    __device__ __forceinline__ void load_x(const V* xs, int lane) { u.load_x(xs, lane); }
+  };
+  __device__ __forceinline__ Exact X() { return Exact{*this}; }
+  float4 t[8];  // piece (m, k) in t[4 m + k]
+  float d[2][4], e[2][4];
+  const V* x;
+  __device__ __forceinline__ void load(const unsigned char* unit, int lane) {
+    const float4* p = reinterpret_cast<const float4*>(unit) + lane;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t[k] = __ldcg(p + 32 * k);
+  }
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) d[m][k] = e[m][k] = 0.f;
+  }
+  static __device__ __forceinline__ uint32_t tf32(float v) {
+    uint32_t y;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(y) : "f"(v));
+    return y;
+  }
+  static __device__ __forceinline__ void mma(float c[4], const float4& a, uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(__float_as_uint(a.x)), "r"(__float_as_uint(a.y)), "r"(__float_as_uint(a.z)), "r"(__float_as_uint(a.w)),
+          "r"(b0), "r"(b1));
+  }
+  template <bool kExact>
+  __device__ __forceinline__ void product(const V* v, int lane) {
+    const float* b = reinterpret_cast<const float*>(v) + (lane & 3) * 8 + (lane >> 2);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float v0 = b[k * 64], v1 = b[k * 64 + 32];
+      const uint32_t h0 = tf32(v0), h1 = tf32(v1);
+      const uint32_t l0 = tf32(v0 - __uint_as_float(h0)), l1 = tf32(v1 - __uint_as_float(h1));
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+        float4 a = t[4 * m + k];
+        if constexpr (kExact) {
+          const float4 f = a;
+          a.x = __uint_as_float(tf32(f.x)); a.y = __uint_as_float(tf32(f.y));
+          a.z = __uint_as_float(tf32(f.z)); a.w = __uint_as_float(tf32(f.w));
+          const float4 r = make_float4(__uint_as_float(tf32(f.x - a.x)), __uint_as_float(tf32(f.y - a.y)),
+                                       __uint_as_float(tf32(f.z - a.z)), __uint_as_float(tf32(f.w - a.w)));
+          mma(e[m], r, h0, h1);
+        }
+        mma(d[m], a, h0, h1);
+        mma(e[m], a, l0, l1);
+      }
+    }
+  }
+  __device__ __forceinline__ void fwd(const unsigned char*, const V* v, int lane) { product<false>(v, lane); }
+  __device__ __forceinline__ void load_x(const V* xs, int) { x = xs; }
+};
+template <class P> struct IsMma { static constexpr bool v = false; };
+template <> struct IsMma<MmaUnit32> { static constexpr bool v = true; };
+// A warp's result for the 32 entries at dst: assigned, or added.
+template <bool kAdd>
+__device__ __forceinline__ void mma_put(const MmaUnit32& u, Vec<float, 8>* dst, int lane) {
+  float* o = reinterpret_cast<float*>(dst) + (lane >> 2) * 8 + 2 * (lane & 3);
+#pragma unroll
+  for (int m = 0; m < 2; ++m)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float2* at = reinterpret_cast<float2*>(o + (16 * m + 8 * h) * 8);
+      float2 r = make_float2(u.d[m][2 * h] + u.e[m][2 * h], u.d[m][2 * h + 1] + u.e[m][2 * h + 1]);
+      if (kAdd) {
+        const float2 p = *at;
+        r.x += p.x;
+        r.y += p.y;
+      }
+      *at = r;
+    }
+}
+
+// P: how the units reach the FMAs (RingUnit, RegUnit32, RegUnit16, each for NR right-hand
+// sides at a time: blockIdx.y takes the next NR); NW consumer warps, OCC CTAs per SM, C CTAs
+// per subdomain.
+template <class P, int NR, int NW, int OCC, int C>
+__global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0), OCC) k_local_super(SuperArgs a) {
   using TF = typename P::T;
+  using TA = typename P::V;  // a vector entry: NR values
+  using TS = typename std::conditional<sizeof(TF) == 8, double, float>::type;
   using K = Unit<TF>;
   using LY = Layout<TF, TA, NW, C>;
+  constexpr bool kMma = IsMma<P>::v;
   constexpr bool kRing = sizeof(TF) == 8;  // (else the units are loaded into registers)
   constexpr int kAll = NW * 32 + (kRing ? 32 : 0);
   constexpr int U = K::U, UC = K::UC;
@@ -454,7 +655,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
     // ---- producer: lane k streams the units of consumer warp k, in its order ----------------
     if (lane < NW) {
       const int q = lane / JW, jq = (lane % JW + q) % JW, cls = rank + C * jq;
-      List l{tf, toff, nb, nsb, q, cls, kSplitX ? cls : jq, a.sweeps};
+      List l{tf, toff, nb, nsb, q, cls, kSplitX ? cls : jq, a.sweeps, a.back};
       unsigned char* slots = sm + (size_t)lane * depth * K::UB;
       uint64_t* fb = full + lane * depth;
       uint64_t* eb = empty + lane * depth;
@@ -505,7 +706,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
     uint64_t* eb = empty + w * depth;
     int slot = 0;
     uint32_t par = 0;
-    List l{tf, toff, nb, nsb, q, cls, clx, a.sweeps};
+    List l{tf, toff, nb, nsb, q, cls, clx, a.sweeps, a.back};
     auto fetch = [&]() {  // (registers) the next unit of the list
       if constexpr (!kRing)
         if (!l.done()) {
@@ -534,14 +735,22 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
       }
     };
     // r(Omega_i), scaled by the equilibration, while the first units load
-    if (a.src) {
-      for (int k = tid; k < nb * kT; k += NT) v[k] = (TA)a.src[(int64_t)i * a.src_stride + k];
-    } else
-    for (int k = tid; k < nb * kT; k += NT)
-      v[k] = (k < ni && in_range(a.om_glob[o0 + k], a.n_cols, a.err))
-                 ? (TA)(a.r[a.om_glob[o0 + k]] * a.eqs[o0 + k])
-                 : (TA)0;
-    for (int k = tid; k < kQ * ring * 32; k += NT) acc4[k] = 0;
+    const int kb = blockIdx.y * NR;
+    for (int k = tid; k < nb * kT; k += NT) {
+      TA x;
+      x.clear();
+      if (a.src) {
+        x.a[0] = (TS)a.src[(int64_t)i * a.src_stride + k];
+      } else if (k < ni && in_range(a.om_glob[o0 + k], a.n_cols, a.err)) {
+        const double* r = a.r + (int64_t)a.om_glob[o0 + k] * a.R + kb;
+        const double e = a.eqs[o0 + k];
+#pragma unroll
+        for (int n = 0; n < NR; ++n)
+          if (NR == 1 || kb + n < a.R) x.a[n] = (TS)(r[n] * e);
+      }
+      v[k] = x;
+    }
+    for (int k = tid; k < kQ * ring * 32; k += NT) acc4[k].clear();
     if (C > 1) cluster_wait();  // every CTA's barriers are ready
     all_barrier();
 
@@ -560,9 +769,13 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
           p.fwd(acquire(), v + u * UC, lane);
           release();
         }
-        int row;
-        const TA sum = p.out(lane, row);
-        red[w * 32 + row] = sum;
+        if constexpr (kMma) {
+          mma_put<false>(p, red + w * 32, lane);
+        } else {
+          int row;
+          const TA sum = p.out(lane, row);
+          red[w * 32 + row] = sum;
+        }
         team_barrier();
         if (j == 0) {
           // u_q = r_q - the team's sums (and, in a cluster, the other ranks')
@@ -584,11 +797,15 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
       all_barrier();
       // v_s = X u_s
       if (has) {
-        TA* db = dbuf + ((s & 1) * kItems + U * (q * (q + 1) / 2)) * 32;
+        TA* db = dbuf + ((kSplitX ? (s & 1) * kItems : 0) + U * (q * (q + 1) / 2)) * 32;
         for (int uu = clx; uu < U * (q + 1); uu += SX) {
           p.X().zero();
           p.X().fwd(acquire(), ub + uu * UC, lane);
           release();
+          if constexpr (kMma) {
+            mma_put<false>(p, db + uu * 32, lane);
+            continue;
+          } else {
           int row;
           const TA x = p.X().out(lane, row);
           if constexpr (kSplitX) {
@@ -596,6 +813,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
             for (int r = 0; r < C; ++r) send(peer(db + uu * 32 + row, r), x, peer(&mbar[4 + (s & 1)], r));
           } else {
             db[uu * 32 + row] = x;
+          }
           }
         }
         if (!kSplitX) team_barrier();
@@ -618,7 +836,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
         if (kSplitX) bar_expect(&mbar[4 + (e & 1)], (uint32_t)(U * nr * (nr + 1) / 2 * UC * sizeof(TA)));
       }
       // w_q = v_q - the teams' sums; in a cluster a unit column's sums are with one rank
-      TA* wq = ws + (m & 1) * kQ * 32 + q * 32;
+      TA* wq = ws + (C > 1 ? (m & 1) * kQ * 32 : 0) + q * 32;
       TA* db = dbuf + (kSplitX ? (e & 1) * kItems * 32 : 0);
       if (has) {
         if (j == 0) {
@@ -626,7 +844,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
           const TA x = v[b * 32 + lane] - ((ac[0] + ac[(size_t)ring * 32]) +
                                            (ac[(size_t)ring * 64] + ac[(size_t)ring * 96]));
 #pragma unroll
-          for (int k = 0; k < kQ; ++k) ac[(size_t)k * ring * 32] = 0;
+          for (int k = 0; k < kQ; ++k) ac[(size_t)k * ring * 32].clear();
           if constexpr (C > 1) {
             if ((U * b + lane / UC) % C == rank)
 #pragma unroll
@@ -640,10 +858,18 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
         // x_s = X^T w_s: unit (q, uu) gives UC columns of its row's share
         p.X().load_x(wq, lane);
         for (int uu = clx; uu < U * (q + 1); uu += SX) {
+          TA* d = db + (U * (q * (q + 1) / 2) + uu) * 32;
+          if constexpr (kMma) {
+            p.X().zero();
+            p.X().fwd(acquire(), wq, lane);
+            release();
+            mma_put<false>(p, d, lane);
+            continue;
+          } else {
           int c;
           const TA x = p.X().bwd(acquire(), lane, c);
           release();
-          TA* d = db + (U * (q * (q + 1) / 2) + uu) * 32 + c;
+          d += c;
           if (lane < UC) {
             if constexpr (kSplitX) {
 #pragma unroll
@@ -651,6 +877,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
             } else {
               *d = x;
             }
+          }
           }
         }
       }
@@ -660,7 +887,8 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
           if (kSplitX) bounded_wait<true>(&mbar[4 + (e & 1)], (uint32_t)((e >> 1) & 1), abort_flag);
           // rows p >= q of the superblock reach block q: unit column U q + lane / UC
           const int uu = U * q + lane / UC;
-          TA x = 0;
+          TA x;
+          x.clear();
           for (int p = q; p < nr; ++p) x += db[(U * (p * (p + 1) / 2) + uu) * 32 + (lane & (UC - 1))];
           v[b * 32 + lane] = x;
         }
@@ -669,10 +897,17 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
         TA* ac = acc4 + (size_t)q * ring * 32;
         p.load_x(v + b * 32, lane);
         for (int u = first_u(b); u < lim; u += ST) {
-          int c;
-          const TA x = p.bwd(acquire(), lane, c);
-          release();
-          if (lane < UC) ac[((u / U) % ring) * 32 + (u % U) * UC + c] += x;
+          if constexpr (kMma) {
+            p.zero();
+            p.fwd(acquire(), v + b * 32, lane);
+            release();
+            mma_put<true>(p, ac + (u % ring) * 32, lane);
+          } else {
+            int c;
+            const TA x = p.bwd(acquire(), lane, c);
+            release();
+            if (lane < UC) ac[((u / U) % ring) * 32 + (u % U) * UC + c] += x;
+          }
         }
       }
       all_barrier();
@@ -680,9 +915,15 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(TA) == 8 ? 32 : 0), OCC) k_l
     if (*abort_flag) {
       if (tid == 0 && a.err[0] == 0.0) a.err[0] = kErrTimeout;
     } else if (a.dst) {
-      for (int k = rank * NT + tid; k < nb * kT; k += C * NT) a.dst[(int64_t)i * a.dst_stride + k] = (double)v[k];
+      for (int k = rank * NT + tid; k < nb * kT; k += C * NT) a.dst[(int64_t)i * a.dst_stride + k] = (double)v[k].a[0];
     } else {
-      for (int k = rank * NT + tid; k < ni; k += C * NT) a.y[o0 + k] = (double)v[k] * a.eqs[o0 + k];
+      for (int k = rank * NT + tid; k < ni; k += C * NT) {
+        double* y = a.y + (o0 + k) * a.R + kb;
+        const double e = a.eqs[o0 + k];
+#pragma unroll
+        for (int n = 0; n < NR; ++n)
+          if (NR == 1 || kb + n < a.R) y[n] = (double)v[k].a[n] * e;
+      }
     }
   }
   if (C > 1) {
@@ -728,18 +969,70 @@ __device__ __forceinline__ void round_bf16(double* S, double* redm) {
   __syncthreads();
 }
 
+// Where the tiles of a factor come from: load(D, b, t) leaves L(b, t) (zero left of the block
+// row's envelope), diag(D, b) L_bb^{-1} in the shared tile D (row pitch 33); both end with a
+// barrier.  BandSrc: the FP64 factor as setup leaves it (row-major panels, the inverse diagonal
+// tiles apart).  SolveSrc: the solve storage of the 32-row sweeps (column-major panels, the
+// inverse diagonal tile last; BF16 with a scale per tile).
+struct BandSrc {
+  const int32_t* tf; const int64_t* poff; const double* L; const double* dinv;
+  __device__ void load(double* D, int64_t g0, int b, int t) const {
+    const int t0 = tf[g0 + b];
+    const int64_t width = (int64_t)(b - t0 + 1) * kT;
+    const double* src = L + poff[g0 + b] + (int64_t)(t - t0) * kT;
+    for (int e = threadIdx.x; e < 1024; e += blockDim.x)
+      D[(e >> 5) * 33 + (e & 31)] = t < t0 ? 0.0 : src[(int64_t)(e >> 5) * width + (e & 31)];
+    __syncthreads();
+  }
+  __device__ void diag(double* D, int64_t g0, int b) const {
+    for (int e = threadIdx.x; e < 1024; e += blockDim.x) D[(e >> 5) * 33 + (e & 31)] = dinv[(g0 + b) * 1024 + e];
+    __syncthreads();
+  }
+};
+template <class T>
+struct SolveSrc {
+  const int32_t* tf; const int64_t* poff; const T* L; const float* tsc;
+  __device__ void tile(double* D, int64_t off, bool zero) const {
+    const double sc = tsc && !zero ? (double)tsc[off / 1024] : 1.0;
+    for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
+      double x = 0.0;
+      if (!zero) {
+        if constexpr (sizeof(T) == 2) x = (double)__bfloat162float(L[off + e]) * sc;
+        else x = (double)L[off + e];
+      }
+      D[(e & 31) * 33 + (e >> 5)] = x;
+    }
+    __syncthreads();
+  }
+  __device__ void load(double* D, int64_t g0, int b, int t) const {
+    const int t0 = tf[g0 + b];
+    tile(D, poff[g0 + b] + (int64_t)(t - t0) * 1024, t < t0);
+  }
+  __device__ void diag(double* D, int64_t g0, int b) const { tile(D, poff[g0 + b] + (int64_t)(b - tf[g0 + b]) * 1024, false); }
+};
+
 // One CTA per superblock: its panel tiles converted, its diagonal tiles replaced by those of
 // the inverse, X(t, t) = L_tt^{-1}, X(b, t) = -L_bb^{-1} sum_{t <= k < b} L(b, k) X(k, t), in
-// FP64 from the factor (row-major panels) and the inverse diagonal tiles.  BF16: X is that of
-// the factor as rounded to BF16 (the tiles L(b, k) and L_bb^{-1} of the 32-row sweeps), kept
-// in FP32: the operator stays the one of BF16 factors.
-template <class TF>
-__global__ void __launch_bounds__(kThreads) k_super_pack(const int64_t* __restrict__ blk_off,
-                                                         const int32_t* __restrict__ blk_tf,
-                                                         const int64_t* __restrict__ blk_poff,
+// FP64.  BF16: X is that of the factor as rounded to BF16 (the tiles L(b, k) and L_bb^{-1} of
+// the 32-row sweeps), kept in FP32: the operator stays the one of BF16 factors.  tf32: the
+// tiles L(b, t) are rounded to TF32 first and X is that of the rounded factor: the operator
+// of the tensor-core kernels of the multi right-hand-side path.
+// frag > 0 (FP32): records in the fragment order of MmaUnit32, and at `frag` bytes from each its
+// transposed copy.
+__device__ __forceinline__ void put_fragments(const double* S, unsigned char* dst, int64_t frag) {
+  float* d = reinterpret_cast<float*>(dst);
+  float* b = reinterpret_cast<float*>(dst + frag);
+  for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
+    const int j = e & 3, lane = (e >> 2) & 31, k = (e >> 7) & 3, m = e >> 9;
+    const int r = 16 * m + (lane >> 2) + 8 * (j & 1), c = 8 * k + (lane & 3) + 4 * (j >> 1);
+    d[e] = (float)S[r * 33 + c];
+    b[e] = (float)S[c * 33 + r];
+  }
+}
+template <class TF, class Src>
+__global__ void __launch_bounds__(kThreads) k_super_pack(const int64_t* __restrict__ blk_off, Src src,
                                                          const int32_t* __restrict__ stf,
-                                                         const int64_t* __restrict__ stoff,
-                                                         const double* __restrict__ L, const double* __restrict__ dinv,
+                                                         const int64_t* __restrict__ stoff, int tf32, int64_t frag,
                                                          unsigned char* __restrict__ dst) {
   using K = Unit<TF>;
   constexpr bool kBf16 = sizeof(TF) == 2;
@@ -751,42 +1044,50 @@ __global__ void __launch_bounds__(kThreads) k_super_pack(const int64_t* __restri
   const int nb = (int)(blk_off[i + 1] - g0);
   const int b0 = s * kQ, b1 = min(nb, b0 + kQ);
   if (b0 >= nb) return;
-  auto load_l = [&](double* D, int b, int t) {  // L(b, t) of the factor, zero left of its envelope
-    const int t0 = blk_tf[g0 + b];
-    const int64_t width = (int64_t)(b - t0 + 1) * kT;
-    const double* src = L + blk_poff[g0 + b] + (int64_t)(t - t0) * kT;
-    for (int e = threadIdx.x; e < 1024; e += blockDim.x)
-      D[(e >> 5) * 33 + (e & 31)] = t < t0 ? 0.0 : src[(int64_t)(e >> 5) * width + (e & 31)];
-    __syncthreads();
-  };
-  auto load_d = [&](double* D, int b) {  // L_bb^{-1}
-    for (int e = threadIdx.x; e < 1024; e += blockDim.x) D[(e >> 5) * 33 + (e & 31)] = dinv[(g0 + b) * 1024 + e];
-    __syncthreads();
+  auto round = [&](double* D) {
     if (kBf16) round_bf16(D, redm);
+    if (tf32) {
+      for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
+        double& x = D[(e >> 5) * 33 + (e & 31)];
+        uint32_t y;
+        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(y) : "f"((float)x));
+        x = (double)__uint_as_float(y);
+      }
+      __syncthreads();
+    }
   };
   for (int b = b0; b < b1; ++b)
     for (int t = stf[g0 + b]; t < b0; ++t) {
-      load_l(S, b, t);
+      src.load(S, g0, b, t);
       unsigned char* rec = dst + stoff[g0 + b] + (int64_t)(t - stf[g0 + b]) * K::REC;
-      if constexpr (kBf16) put_bf16(S, rec, redm);
-      else put_tile<TF>(S, rec);
+      if constexpr (kBf16) {
+        put_bf16(S, rec, redm);
+      } else {
+        round(S);
+        if (frag) put_fragments(S, rec, frag);
+        else put_tile<TF>(S, rec);
+      }
       __syncthreads();
     }
   auto put_x = [&](const double* D, int b, int t) {
-    put_tile<TX>(D, dst + stoff[g0 + b] + (int64_t)(b0 - stf[g0 + b]) * K::REC + (int64_t)(t - b0) * K::RECX);
+    unsigned char* rec = dst + stoff[g0 + b] + (int64_t)(b0 - stf[g0 + b]) * K::REC + (int64_t)(t - b0) * K::RECX;
+    if (frag) put_fragments(D, rec, frag);
+    else put_tile<TX>(D, rec);
   };
   for (int t = b0; t < b1; ++t) {
-    load_d(X[0], t);
+    src.diag(X[0], g0, t);
+    if (kBf16) round_bf16(X[0], redm);
     put_x(X[0], t, t);
     for (int b = t + 1; b < b1; ++b) {
       for (int e = threadIdx.x; e < kT * 33; e += blockDim.x) S[e] = 0.0;
       for (int k = t; k < b; ++k) {
-        load_l(P, b, k);
-        if (kBf16) round_bf16(P, redm);
+        src.load(P, g0, b, k);
+        round(P);
         tile_mm<false, false>(S, P, X[k - t], -1);
         __syncthreads();
       }
-      load_d(P, b);
+      src.diag(P, g0, b);
+      if (kBf16) round_bf16(P, redm);
       // X(b, t) = L_bb^{-1} S; the last row's tile is not needed by a later one: over X(t, t)'s place
       double* out = b - t < kQ - 1 ? X[b - t] : X[0];
       tile_mm<false, false>(out, P, S, 0);
@@ -797,10 +1098,10 @@ __global__ void __launch_bounds__(kThreads) k_super_pack(const int64_t* __restri
   }
 }
 
-template <class P, class TA, int NW, int OCC, int C>
+template <class P, int NR, int NW, int OCC, int C>
 bool launch_impl(SuperArgs a, int N, int max_nb, size_t optin, bool probe, cudaStream_t st) {
-  using LY = Layout<typename P::T, TA, NW, C>;
-  constexpr bool kRing = sizeof(TA) == 8;
+  using LY = Layout<typename P::T, typename P::V, NW, C>;
+  constexpr bool kRing = sizeof(typename P::T) == 8;
   // OCC CTAs share what the SM holds, 1 KB of each share the system's
   const size_t limit = (optin + 1024) / OCC - 1024;
   int d = kRing ? 6 : 0;
@@ -809,7 +1110,7 @@ bool launch_impl(SuperArgs a, int N, int max_nb, size_t optin, bool probe, cudaS
   if (bytes > limit) return false;
   a.depth = d;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)N * C, 1, 1);
+  cfg.gridDim = dim3((unsigned)N * C, (unsigned)((a.R + NR - 1) / NR), 1);
   cfg.blockDim = dim3(NW * 32 + (kRing ? 32 : 0), 1, 1);
   cfg.dynamicSmemBytes = bytes;
   cfg.stream = st;
@@ -820,7 +1121,7 @@ bool launch_impl(SuperArgs a, int N, int max_nb, size_t optin, bool probe, cudaS
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = C > 1 ? 1 : 0;
-  auto* fn = k_local_super<P, TA, NW, OCC, C>;
+  auto* fn = k_local_super<P, NR, NW, OCC, C>;
   if (probe) {
     // the kernel's limit is the device's, not this factor's need: handles share the kernels
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)optin) != cudaSuccess) {
@@ -838,27 +1139,40 @@ bool launch_impl(SuperArgs a, int N, int max_nb, size_t optin, bool probe, cudaS
   return cudaLaunchKernelEx(&cfg, fn, a) == cudaSuccess;
 }
 
-// FP32 / BF16: the shapes the rule below picks.
-template <class P>
+// The shapes the rules below pick.
+template <template <int> class P>
 bool by_shape(const SuperArgs& a, const SuperShape& f, int N, int max_nb, size_t optin, bool probe, cudaStream_t st) {
-  if (f.occ == 2) return launch_impl<P, float, 16, 2, 1>(a, N, max_nb, optin, probe, st);
+  if (f.occ == 2) return launch_impl<P<1>, 1, 16, 2, 1>(a, N, max_nb, optin, probe, st);
   if (f.warps == 24)
-    return f.cluster == 2 ? launch_impl<P, float, 24, 1, 2>(a, N, max_nb, optin, probe, st)
-                          : launch_impl<P, float, 24, 1, 1>(a, N, max_nb, optin, probe, st);
-  return f.cluster == 4 ? launch_impl<P, float, 16, 1, 4>(a, N, max_nb, optin, probe, st)
-                        : launch_impl<P, float, 16, 1, 1>(a, N, max_nb, optin, probe, st);
+    return f.cluster == 2 ? launch_impl<P<1>, 1, 24, 1, 2>(a, N, max_nb, optin, probe, st)
+                          : launch_impl<P<1>, 1, 24, 1, 1>(a, N, max_nb, optin, probe, st);
+  return f.cluster == 4 ? launch_impl<P<1>, 1, 16, 1, 4>(a, N, max_nb, optin, probe, st)
+                        : launch_impl<P<1>, 1, 16, 1, 1>(a, N, max_nb, optin, probe, st);
 }
 
 bool by_prec(const SuperArgs& a, const SuperShape& f, int prec, int N, int max_nb, size_t optin, bool probe,
              cudaStream_t st) {
+  if (prec == 1 && f.nr == 8)
+    return f.cluster == 2 ? launch_impl<MmaUnit32, 8, 16, 1, 2>(a, N, max_nb, optin, probe, st)
+                          : launch_impl<MmaUnit32, 8, 16, 1, 1>(a, N, max_nb, optin, probe, st);
   if (prec == 1) return by_shape<RegUnit32>(a, f, N, max_nb, optin, probe, st);
+  if (prec == 2 && f.nr == 4)
+    return f.cluster == 2 ? launch_impl<RegUnit16<4>, 4, 16, 1, 2>(a, N, max_nb, optin, probe, st)
+                          : launch_impl<RegUnit16<4>, 4, 16, 1, 1>(a, N, max_nb, optin, probe, st);
   if (prec == 2) return by_shape<RegUnit16>(a, f, N, max_nb, optin, probe, st);
-  if (f.occ == 2) return launch_impl<RingUnit, double, 8, 2, 1>(a, N, max_nb, optin, probe, st);
+  if (f.nr == 4) {
+    switch (f.cluster) {
+      case 2: return launch_impl<RingUnit<4>, 4, 8, 1, 2>(a, N, max_nb, optin, probe, st);
+      case 4: return launch_impl<RingUnit<4>, 4, 8, 1, 4>(a, N, max_nb, optin, probe, st);
+      default: return launch_impl<RingUnit<4>, 4, 8, 1, 1>(a, N, max_nb, optin, probe, st);
+    }
+  }
+  if (f.occ == 2) return launch_impl<RingUnit<1>, 1, 8, 2, 1>(a, N, max_nb, optin, probe, st);
   switch (f.cluster) {
-    case 2: return launch_impl<RingUnit, double, 16, 1, 2>(a, N, max_nb, optin, probe, st);
-    case 4: return launch_impl<RingUnit, double, 16, 1, 4>(a, N, max_nb, optin, probe, st);
-    case 8: return launch_impl<RingUnit, double, 16, 1, 8>(a, N, max_nb, optin, probe, st);
-    default: return launch_impl<RingUnit, double, 16, 1, 1>(a, N, max_nb, optin, probe, st);
+    case 2: return launch_impl<RingUnit<1>, 1, 16, 1, 2>(a, N, max_nb, optin, probe, st);
+    case 4: return launch_impl<RingUnit<1>, 1, 16, 1, 4>(a, N, max_nb, optin, probe, st);
+    case 8: return launch_impl<RingUnit<1>, 1, 16, 1, 8>(a, N, max_nb, optin, probe, st);
+    default: return launch_impl<RingUnit<1>, 1, 16, 1, 1>(a, N, max_nb, optin, probe, st);
   }
 }
 
@@ -886,9 +1200,10 @@ size_t local_super_record(int prec, bool x) {
 // pair; 571 before).
 bool local_super_plan(int prec, int N, int max_nb, int wmax, double wmean, int sms, size_t optin, SuperShape& out) {
   auto fits = [&](int cluster, int warps, int occ) {
-    out = SuperShape{cluster, warps, occ, wmax + kQ};
+    out = SuperShape{cluster, warps, occ, wmax + kQ, 1};
     SuperArgs a{};
     a.ring = out.ring;
+    a.R = 1;
     return by_prec(a, out, prec, N, max_nb, optin, true, nullptr);
   };
   if (N > sms && fits(1, prec == 0 ? 8 : 16, 2)) return true;
@@ -904,6 +1219,24 @@ bool local_super_plan(int prec, int N, int max_nb, int wmax, double wmean, int s
   return fits(1, 24, 1);
 }
 
+// R right-hand sides: eight per CTA with FP32 factors (one MMA's columns), else four (BF16: eight
+// do not fit the registers; FP64: the ring leaves no room for more, and the FP64 units bound
+// it anyway); clusters while all CTAs then have an SM each.
+bool local_super_plan_multi(int prec, int R, int N, int max_nb, int wmax, int sms, size_t optin, SuperShape& out) {
+  const int nr = prec == 1 ? 8 : 4;
+  auto fits = [&](int cluster) {
+    out = SuperShape{cluster, prec == 0 ? 8 : 16, 1, wmax + kQ, nr};
+    SuperArgs a{};
+    a.ring = out.ring;
+    a.R = R;
+    return by_prec(a, out, prec, N, max_nb, optin, true, nullptr);
+  };
+  const int64_t ctas = (int64_t)N * ((R + nr - 1) / nr);
+  for (int c = prec == 0 ? 4 : 2; c >= 2; c >>= 1)
+    if (ctas * c <= sms && fits(c)) return true;
+  return fits(1);
+}
+
 bool launch_local_super(const SuperArgs& a, const SuperShape& f, int prec, int N, int max_nb, size_t optin,
                         cudaStream_t st) {
   SuperArgs b = a;
@@ -915,9 +1248,25 @@ void launch_super_pack(int prec, int N, int max_nb, const int64_t* blk_off, cons
                        const int64_t* blk_poff, const int32_t* stf, const int64_t* stoff, const double* L,
                        const double* dinv, unsigned char* dst, cudaStream_t st) {
   const dim3 grid((unsigned)((max_nb + kQ - 1) / kQ), (unsigned)N);
-  if (prec == 0) k_super_pack<double><<<grid, kThreads, 0, st>>>(blk_off, blk_tf, blk_poff, stf, stoff, L, dinv, dst);
-  else if (prec == 1) k_super_pack<float><<<grid, kThreads, 0, st>>>(blk_off, blk_tf, blk_poff, stf, stoff, L, dinv, dst);
-  else k_super_pack<__nv_bfloat16><<<grid, kThreads, 0, st>>>(blk_off, blk_tf, blk_poff, stf, stoff, L, dinv, dst);
+  const BandSrc src{blk_tf, blk_poff, L, dinv};
+  if (prec == 0) k_super_pack<double><<<grid, kThreads, 0, st>>>(blk_off, src, stf, stoff, 0, 0, dst);
+  else if (prec == 1) k_super_pack<float><<<grid, kThreads, 0, st>>>(blk_off, src, stf, stoff, 0, 0, dst);
+  else k_super_pack<__nv_bfloat16><<<grid, kThreads, 0, st>>>(blk_off, src, stf, stoff, 0, 0, dst);
+}
+
+void launch_super_pack_solve(int prec, int N, int max_nb, const int64_t* blk_off, const int32_t* blk_tf,
+                             const int64_t* blk_poff, const int32_t* stf, const int64_t* stoff, const void* fac,
+                             const float* tsc, int64_t frag, unsigned char* dst, cudaStream_t st) {
+  const dim3 grid((unsigned)((max_nb + kQ - 1) / kQ), (unsigned)N);
+  if (prec == 0)
+    k_super_pack<double><<<grid, kThreads, 0, st>>>(
+        blk_off, SolveSrc<double>{blk_tf, blk_poff, (const double*)fac, nullptr}, stf, stoff, 0, 0, dst);
+  else if (prec == 1)
+    k_super_pack<float><<<grid, kThreads, 0, st>>>(
+        blk_off, SolveSrc<float>{blk_tf, blk_poff, (const float*)fac, nullptr}, stf, stoff, 1, frag, dst);
+  else
+    k_super_pack<__nv_bfloat16><<<grid, kThreads, 0, st>>>(
+        blk_off, SolveSrc<__nv_bfloat16>{blk_tf, blk_poff, (const __nv_bfloat16*)fac, tsc}, stf, stoff, 0, 0, dst);
 }
 
 }  // namespace lsq

@@ -193,11 +193,13 @@ struct SuperArgs {
   const int64_t* om_off; const int32_t* om_glob; const double* eqs;
   const int64_t* blk_off; const int32_t* tf; const int64_t* toff;
   const unsigned char* fac;
-  const double* r; double* y;
+  const double* r; double* y;  // R right-hand sides, interleaved (entry k of one at k R)
+  int R;
   // or (src, dst set) on vectors in local order, subdomain i's of its padded length at
   // src + i src_stride and dst + i dst_stride, without the scales
   const double* src; int64_t src_stride; double* dst; int64_t dst_stride;
   const int* skip;        // subdomains with skip[i] != 0 are left out (null: none)
+  int64_t back;           // bytes from a record to its copy for the backward sweep (0: the same)
   int sweeps;             // 1 the forward sweep (L^{-1}), 2 the backward one (L^{-T}), 3 both
   double* err;            // error slot
   int depth;              // units in flight per warp (set by the launcher)
@@ -206,15 +208,23 @@ struct SuperArgs {
 };
 size_t local_super_record(int prec, bool x);
 // Launch shape: CTAs per subdomain, consumer warps and CTAs per SM, tile columns of the
-// backward sums.  local_super_plan picks it by rule (block rows of at most wmax tiles, wmean
+// backward sums, right-hand sides per CTA.  local_super_plan picks it by rule (block rows of at most wmax tiles, wmean
 // on average); false if none fits.
-struct SuperShape { int cluster, warps, occ, ring; };
+struct SuperShape { int cluster, warps, occ, ring, nr; };
 bool local_super_plan(int prec, int N, int max_nb, int wmax, double wmean, int sms, size_t optin, SuperShape& out);
+// the same for R interleaved right-hand sides
+bool local_super_plan_multi(int prec, int R, int N, int max_nb, int wmax, int sms, size_t optin, SuperShape& out);
 bool launch_local_super(const SuperArgs& a, const SuperShape& f, int prec, int N, int max_nb, size_t optin,
                         cudaStream_t st);
 void launch_super_pack(int prec, int N, int max_nb, const int64_t* blk_off, const int32_t* blk_tf,
                        const int64_t* blk_poff, const int32_t* stf, const int64_t* stoff, const double* L,
                        const double* dinv, unsigned char* dst, cudaStream_t st);
+// the same from the solve storage of the 32-row sweeps; FP32: tiles rounded to TF32 (the operator
+// of the tensor-core block kernels), the inverse diagonal tiles FP32, in fragment order with a
+// transposed copy frag bytes further on
+void launch_super_pack_solve(int prec, int N, int max_nb, const int64_t* blk_off, const int32_t* blk_tf,
+                             const int64_t* blk_poff, const int32_t* stf, const int64_t* stoff, const void* fac,
+                             const float* tsc, int64_t frag, unsigned char* dst, cudaStream_t st);
 // Block-envelope factor + inverse diagonal tiles (FP64) -> solve storage (prec 0/1/2);
 // tsc receives one scale per 32x32 tile for BF16.
 void launch_to_solve_layout(int prec, int64_t nblocks, const int64_t* poff, const double* L, const double* dinv,
@@ -373,7 +383,8 @@ void launch_b_pupdate(const BChunks& ch, int R, const double* beta, const double
 void launch_b_finish(int nprob, const int64_t* pc_off, const double* part, const double* part2, int R,
                      const BScal& s, int mode, int flex, cudaStream_t st);
 void launch_b_scatter(const BChunks& ch, const BScatterArgs& a, cudaStream_t st);
-void launch_b_restrict(int N, int R, const int64_t* int_off, const int32_t* int_glob, const int64_t* zoff,
+// (kmax: most coarse vectors of a subdomain)
+void launch_b_restrict(int N, int kmax, int R, const int64_t* int_off, const int32_t* int_glob, const int64_t* zoff,
                        const int32_t* coff, const double* Z, const double* Rv, double* R0, cudaStream_t st);
 void launch_b_coarse(int ntiles, int R, const int32_t* ct_prob, const int32_t* ct_row, const CoarseBlocks& cb,
                      const int32_t* n0q, const double* Xinv, const double* R0, double* Y0, float* Y0f,
@@ -382,7 +393,7 @@ void launch_b_coarse(int ntiles, int R, const int32_t* ct_prob, const int32_t* c
 // kp_i = k_i rounded up to 4; restriction with it.
 void launch_b_ztrans(int N, const int64_t* int_off, const int64_t* zoff, const int32_t* coff, const int64_t* zt_off,
                      const double* Z, float* ZT, cudaStream_t st);
-void launch_b_restrict32(int N, int R, const int64_t* int_off, const int32_t* int_glob, const int32_t* coff,
+void launch_b_restrict32(int N, int kmax, int R, const int64_t* int_off, const int32_t* int_glob, const int32_t* coff,
                          const int64_t* zt_off, const float* ZT, const double* Rv, double* R0, cudaStream_t st);
 void launch_b_load_rows(int64_t m, int R, const int32_t* perm, const double* Bu, double* Bb, cudaStream_t st);
 void launch_b_store_cols(int64_t n, int R, const double* Xb, double* Xu, cudaStream_t st);

@@ -56,3 +56,33 @@ def test_super_matches_row_sweeps(name, prec):
         S.close()
     tol = 1e-12 if prec == "f64" else 1e-5
     assert float((z[0] - z[1]).norm() / z[1].norm()) < tol
+
+
+@pytest.mark.parametrize("prec,R", [("f64", 2), ("f64", 5), ("f32", 3), ("f32", 8), ("f32", 19), ("bf16", 4), ("bf16", 7)])
+@pytest.mark.parametrize("name", ["strips", "blocks8", "blocks32-ragged", "n100", "n400"])
+def test_super_many_right_hand_sides(name, prec, R):
+    """Three fixed iterations of R right-hand sides (one to three groups of four or eight,
+    full and partial) against the same operator elsewhere: FP64 and BF16 the single-vector
+    path's, to 1e-10 and 1e-4 (the block path keeps its coarse basis in FP32); FP32 the
+    tensor-core kernel with the same TF32-rounded factor, to 1e-4."""
+    import paper_2107_09006_gb300 as L
+
+    W, H, (k, radius), split = SHAPES[name]
+    m, n, rp, col, val, b, _ = make_grid_ls(W, H, 4, k, radius, 7, nrhs=R)
+    part = split(W, H)
+    mk = lambda **o: L.Solver(m, n, rp, col, val, part, int(part.max()) + 1, nev_max=4, factor_prec=prec,  # noqa: E731
+                              fixed_iters=3, **o)
+    S = mk()
+    X, info = S.solve(b)
+    assert info["local_kernel"] == 0
+    if prec == "f32":
+        S2 = mk(block_kernel=2)
+        ref, info = S2.solve(b)
+        assert info["local_kernel"] == 2
+        S2.close()
+    else:
+        ref = torch.stack([S.solve(b[q])[0] for q in range(R)])
+    S.close()
+    tol = 1e-10 if prec == "f64" else 1e-4
+    for q in range(R):
+        assert float((X[q] - ref[q]).norm() / ref[q].norm()) < tol, q
