@@ -340,7 +340,7 @@ int iteration_launches(const ls_handle* h) {
   return 6 + (coarse ? 1 : 0) + (coarse && h->local_cfg == 4 && h->opt.variant == 0 ? 1 : 0);
 }
 
-void iteration(ls_handle* h, bool flex, bool copy_scalars = true) {
+void iteration(ls_handle* h, bool flex, bool copy_scalars = true, const lsq::LoopTest* loop = nullptr) {
   cudaStream_t st = h->st;
   const bool timed = h->opt.time_kernels != 0;
   if (timed) mark(h, 0);
@@ -349,15 +349,15 @@ void iteration(ls_handle* h, bool flex, bool copy_scalars = true) {
   lsq::launch_cg_update(h->n, h->scal.p, h->p.p, h->w.p, h->x.p, h->r.p, flex ? h->r_old.p : nullptr,
                         site(h, lsq::S_RR, 1), h->ctr.p, h->ahist.p, h->hist_cap, st);
   precond(h, h->r.p, h->z.p, 0, true, flex, timed);
-  lsq::launch_p_update(h->n, h->scal.p, h->ctr.p, h->bhist.p, h->hist_cap, h->z.p, h->p.p, 0, flex ? 1 : 0, st);
+  lsq::launch_p_update(h->n, h->scal.p, h->ctr.p, h->bhist.p, h->hist_cap, h->z.p, h->p.p, 0, flex ? 1 : 0, loop, st);
   if (timed) mark(h, 5);
   if (copy_scalars) CK(cudaMemcpyAsync(h->pin, h->scal.p, sizeof(double) * lsq::S_NSLOT, cudaMemcpyDeviceToHost, st));
 }
 
 // Builds h->gloop: while (loop test) { one PCG iteration }, then the scalar slots to the
-// host.  The body is captured from the same launch sequence as iteration(); the loop test
-// kernel sets the while condition from the device scalars, so the host waits once per
-// pass of the loop instead of once per iteration.  Returns false (and leaves gloop null)
+// host.  The body is captured from the same launch sequence as iteration(); its last kernel
+// sets the while condition from the device scalars, so the host waits once per pass of the
+// loop instead of once per iteration.  Returns false (and leaves gloop null)
 // when the graph cannot be built, e.g. on a driver without conditional nodes.
 bool build_loop_graph(ls_handle* h, bool flex, int limit) {
   cudaStream_t st = h->st;
@@ -378,8 +378,8 @@ bool build_loop_graph(ls_handle* h, bool flex, int limit) {
     if (cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
       break;
     h->stamping = h->opt.time_kernels != 0;
-    iteration(h, flex, false);
-    lsq::launch_cg_continue(h->scal.p, h->ctr.p, limit, hnd, st);
+    const lsq::LoopTest loop{hnd, limit};
+    iteration(h, flex, false, &loop);
     h->stamping = false;
     cudaGraph_t captured = nullptr;
     if (cudaStreamEndCapture(st, &captured) != cudaSuccess) break;
@@ -471,7 +471,7 @@ ls_status solve_core(ls_handle* h, int mode, double rtol, ls_info* info) {
   }
   auto restart = [&]() {
     precond(h, h->r.p, h->z.p, 0, true, false);
-    lsq::launch_p_update(n, h->scal.p, h->ctr.p, h->bhist.p, h->hist_cap, h->z.p, h->p.p, 1, 0, st);
+    lsq::launch_p_update(n, h->scal.p, h->ctr.p, h->bhist.p, h->hist_cap, h->z.p, h->p.p, 1, 0, nullptr, st);
     launches += iteration_launches(h) - 3;
     inf.local_launches += 1;
   };

@@ -72,15 +72,14 @@ bool normal_tiles_prepare(const NormalTilesDev& T);
 void launch_cg_update(int64_t n, double* scal, const double* p, const double* w, double* x, double* r,
                       double* r_old, const DotSite& rr, int* ctr, double* alpha_hist, int hist_cap,
                       cudaStream_t st);
-// beta from the scalar slots (plain or flexible form), p = z + beta p (init: p = z).
+// beta from the scalar slots (plain or flexible form), p = z + beta p (init: p = z).  In the
+// body of the device-side PCG loop (loop != null) the launch is also its test, a conditional
+// while node of a CUDA graph: continue while no breakdown or device timeout is flagged, the
+// recursive residual ||r||^2 = scal[S_RR] is above scal[S_THR] (when that is positive) and
+// fewer than loop->limit iterations have run.
+struct LoopTest { cudaGraphConditionalHandle handle; int limit; };
 void launch_p_update(int64_t n, double* scal, int* ctr, double* beta_hist, int hist_cap, const double* z, double* p,
-                     int init, int flex, cudaStream_t st);
-// The loop test of the device-side PCG loop (a conditional while node of a CUDA graph):
-// continue while no breakdown or device timeout is flagged, the recursive residual
-// ||r||^2 = scal[S_RR] is above scal[S_THR] (when that is positive) and fewer than
-// `limit` iterations have run.
-void launch_cg_continue(const double* scal, const int* ctr, int limit, cudaGraphConditionalHandle hnd,
-                        cudaStream_t st);
+                     int init, int flex, const LoopTest* loop, cudaStream_t st);
 // Writes the global nanosecond timer into stamps[slot * 8 + k], slot = *ctr - after, when
 // 0 <= slot < cap (kernel timing inside graphs, where event records are not allowed).
 void launch_stamp(unsigned long long* stamps, const int* ctr, int cap, int k, int after, cudaStream_t st);

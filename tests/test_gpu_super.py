@@ -74,7 +74,9 @@ def test_super_many_right_hand_sides(name, prec, R):
                               fixed_iters=3, **o)
     S = mk()
     X, info = S.solve(b)
-    assert info["local_kernel"] == 0
+    groups, sms = -(-R // 8), torch.cuda.get_device_properties(0).multi_processor_count
+    wide = prec == "f32" and groups > 2 and groups * (int(part.max()) + 1) > 3 * sms  # a tensor-core kernel's ground
+    assert (info["local_kernel"] == 0) != wide
     if prec == "f32":
         S2 = mk(block_kernel=2)
         ref, info = S2.solve(b)
