@@ -412,16 +412,15 @@ bool build_loop_graph(ls_handle* h, bool flex, int limit) {
 
 // Reads one scalar slot of the device CG state (synchronising the stream).
 double dev_sum(ls_handle* h, int slot = lsq::S_TMP) {
-  double v = 0;
-  CK(cudaMemcpyAsync(&v, h->scal.p + slot, sizeof(double), cudaMemcpyDeviceToHost, h->st));
+  double* v = h->pin + lsq::S_NSLOT;
+  CK(cudaMemcpyAsync(v, h->scal.p + slot, sizeof(double), cudaMemcpyDeviceToHost, h->st));
   CK(cudaStreamSynchronize(h->st));
-  return v;
+  return *v;
 }
 
-// ||g - C x||^2 into the host: mode 0 as ||A^T (b - A x)||^2, mode 1 as ||g - A^T (A x)||^2.
-// Leaves the residual vector in h->w; adds the kernels it launched to *launches.
-double true_residual(ls_handle* h, int mode, int* launches) {
-  Phase phase("true residual");
+// ||g - C x||^2 into scal[S_TMP] (true_residual: and to the host): mode 0 as
+// ||A^T (b - A x)||^2, mode 1 as ||g - A^T (A x)||^2.  Leaves the residual vector in h->w; adds the kernels it launched to *launches.
+void launch_true_residual(ls_handle* h, int mode, int* launches) {
   cudaStream_t st = h->st;
   lsq::launch_spmv_csr(csr(h), h->x.p, h->q.p, h->lanes_csr, h->grid_csr, st);
   if (mode == 0) {
@@ -434,6 +433,11 @@ double true_residual(ls_handle* h, int mode, int* launches) {
     lsq::launch_dot(h->n, h->w.p, h->w.p, site(h, lsq::S_TMP, 3), st);
     *launches += 4;
   }
+}
+
+double true_residual(ls_handle* h, int mode, int* launches) {
+  Phase phase("true residual");
+  launch_true_residual(h, mode, launches);
   return dev_sum(h);
 }
 
@@ -615,13 +619,36 @@ ls_status solve_core(ls_handle* h, int mode, double rtol, ls_info* info) {
   return LS_OK;
 }
 
+// One step of lsqr_core: the bidiagonalization, the vector updates and the report to the host.
+void lsqr_step(ls_handle* h, bool timed) {
+  cudaStream_t st = h->st;
+  double* state = h->lq_k.p;
+  if (timed) mark(h, 0);
+  // beta u = A v - alpha u
+  lsq::launch_spmv_csr(csr(h), h->lq_v.p, h->q.p, h->lanes_csr, h->grid_csr, st);
+  if (timed) record_event(h->ev[6], st);
+  lsq::DotSite ub = site(h, lsq::S_TMP, 3);
+  ub.out = state + lsq::L_BETA2;
+  lsq::launch_lsqr_u(h->m, state, h->q.p, h->lq_u.p, ub, st);
+  // alpha v = M^{-1} (A^T u - beta q)
+  if (timed) record_event(h->ev[7], st);
+  lsq::launch_spmv_csc(csc(h), h->lq_u.p, h->lq_s.p, nullptr, lsq::DotSite{}, h->lanes_csc, h->grid_csc, st);
+  if (timed) mark(h, 1);
+  lsq::launch_lsqr_s(h->n, state, h->lq_q.p, h->lq_s.p, st);
+  precond(h, h->lq_s.p, h->lq_t.p, 0, true, false, timed);
+  lsq::launch_lsqr_step(h->n, 0, state, h->scal.p, h->lq_t.p, h->lq_s.p, h->lq_v.p, h->lq_q.p, h->x.p, h->lq_w.p, st);
+  if (timed) mark(h, 5);
+  CK(cudaMemcpyAsync(h->pin + lsq::S_NSLOT, state + lsq::L_REP, sizeof(double) * lsq::L_NREP, cudaMemcpyDeviceToHost,
+                     st));
+}
+
 // Preconditioned LSQR on min ||A' x - b'|| (b' in h->bv, result in h->x): Golub-Kahan
 // bidiagonalization between R^m and R^n with the inner product of M, so the adjoint of
 // A is M^{-1} A^T and each step applies the preconditioner once (Section 4.1.3 uses
-// left-preconditioned LSQR); the plane-rotation recurrences run on the host, the vector
-// work on the device.  Stopping: the true residual test ||A^T (b - A x)|| <= rtol ||A^T b||,
-// evaluated from the first step at which LSQR's estimate of ||M^{-1} A^T r||_M has
-// fallen below 10 rtol times its initial value.
+// left-preconditioned LSQR).  Scalars and vectors stay on the device; the host reads one
+// report per step and repeats the plane rotation for the stopping test.  Stopping: the true
+// residual test ||A^T (b - A x)|| <= rtol ||A^T b||, evaluated from the first step at which
+// LSQR's estimate of ||M^{-1} A^T r||_M has fallen below 10 rtol times its initial value.
 ls_status lsqr_core(ls_handle* h, double rtol, ls_info* info) {
   cudaStream_t st = h->st;
   const int64_t n = h->n, m = h->m;
@@ -638,6 +665,8 @@ ls_status lsqr_core(ls_handle* h, double rtol, ls_info* info) {
   const double gn = std::sqrt(gg);
   lsq::launch_fill(n, 0.0, h->x.p, st);
   launches += 1;
+  double* state = h->lq_k.p;
+  CK(cudaMemcpyAsync(state + lsq::L_BETA2, h->scal.p + lsq::S_TMP, sizeof(double), cudaMemcpyDeviceToDevice, st));
   CK(cudaMemsetAsync(h->scal.p, 0, sizeof(double) * lsq::S_NSLOT, st));
   auto finish = [&](int it, bool converged, double rel) -> ls_status {
     inf.iters = it;
@@ -660,47 +689,60 @@ ls_status lsqr_core(ls_handle* h, double rtol, ls_info* info) {
     return finish(0, true, 0.0);
   }
   const bool timed = h->opt.time_kernels != 0;
+  bool graph = h->opt.use_graph != 0 && !timed;  // event records of the timing marks stay outside graphs
   const int pl = balanced(h) ? kBalancedLaunches : 2 + ((h->coarse && h->n0 > 0) ? 1 : 0);
-  // u = b / beta, s = A^T u, t = M^{-1} s, alpha = (s.t)^{1/2}, v = t / alpha, q = s / alpha, w = v
+  // u = b (kept unnormalised), s = A^T u / beta, t = M^{-1} s, alpha = (s.t)^{1/2}, v = t / alpha,
+  // q = s / alpha, w = v
+  double* hrep = h->pin + lsq::S_NSLOT;
   double beta = std::sqrt(bb);
-  lsq::launch_axpby(m, 1.0 / beta, h->bv.p, 0.0, nullptr, h->lq_u.p, st);
-  lsq::launch_spmv_csc(csc(h), h->lq_u.p, h->lq_s.p, nullptr, lsq::DotSite{}, h->lanes_csc, h->grid_csc, st);
+  CK(cudaMemcpyAsync(h->lq_u.p, h->bv.p, sizeof(double) * m, cudaMemcpyDeviceToDevice, st));
+  CK(cudaMemcpyAsync(h->lq_s.p, h->r.p, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));  // A^T b
+  lsq::launch_lsqr_s(n, state, nullptr, h->lq_s.p, st);
   precond(h, h->lq_s.p, h->lq_t.p, 0, true, false);
-  double alpha = std::sqrt(dev_sum(h, lsq::S_RZ));
-  CK(cudaMemsetAsync(h->lq_w.p, 0, sizeof(double) * n, st));
-  lsq::launch_lsqr_step(n, 1.0 / alpha, 0.0, -1.0, h->lq_t.p, h->lq_s.p, h->lq_v.p, h->lq_q.p, h->x.p, h->lq_w.p,
-                        st);  // v, q; w = v (x unchanged)
-  launches += 3 + pl + 1;
+  lsq::launch_lsqr_step(n, 1, state, h->scal.p, h->lq_t.p, h->lq_s.p, h->lq_v.p, h->lq_q.p, h->x.p, h->lq_w.p, st);
+  launches += 2 + pl;
   inf.local_launches += 1;
-  std::vector<double> al{alpha}, be{beta};
-  double phibar = beta, rhobar = alpha;
-  const double est0 = alpha * beta;
+  std::vector<double> al, be{beta};
+  double alpha = 0.0, phibar = beta, rhobar = 0.0, est0 = 0.0;
   const int fixed = h->opt.fixed_iters;
   const int maxit = fixed > 0 ? fixed : h->opt.maxit;
   bool converged = false, checking = false, have_rel = false;
   double rel = 1.0;
   int it = 0;
   while (it < maxit) {
-    if (timed) mark(h, 0);
-    // beta u = A v - alpha u
-    lsq::launch_spmv_csr(csr(h), h->lq_v.p, h->q.p, h->lanes_csr, h->grid_csr, st);
-    if (timed) record_event(h->ev[6], st);
-    lsq::launch_axpby(m, 1.0, h->q.p, -alpha, h->lq_u.p, h->lq_u.p, st);
-    lsq::launch_dot(m, h->lq_u.p, h->lq_u.p, site(h, lsq::S_TMP, 3), st);
-    beta = std::sqrt(dev_sum(h));
+    if (graph && !h->lq_exec) {  // built once per handle: a step only touches fixed buffers
+      cudaGraph_t g;
+      CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+      lsqr_step(h, false);
+      CK(cudaStreamEndCapture(st, &g));
+      const cudaError_t e = cudaGraphInstantiate(&h->lq_exec, g, 0);
+      cudaGraphDestroy(g);
+      if (e != cudaSuccess) {
+        h->lq_exec = nullptr;
+        cudaGetLastError();
+        graph = false;
+      }
+    }
+    if (graph) CK(cudaGraphLaunch(h->lq_exec, st));
+    else lsqr_step(h, timed);
+    const bool early = checking;  // the residual test of this step without a second wait
+    if (early) {
+      launch_true_residual(h, 0, &launches);
+      CK(cudaMemcpyAsync(hrep + lsq::L_NREP, h->scal.p + lsq::S_TMP, sizeof(double), cudaMemcpyDeviceToHost, st));
+    }
+    CK(cudaStreamSynchronize(st));
+    beta = hrep[lsq::L_REP_BETA];
     if (!(beta > 0.0) || !std::isfinite(beta)) {
       if (beta == 0.0) { converged = true; break; }  // b lies in range(A V_k): x_k solves the problem
       throw LsError(LS_ERR_NONFINITE, "LSQR breakdown (beta) at iteration " + std::to_string(it + 1));
     }
-    lsq::launch_axpby(m, 1.0 / beta, h->lq_u.p, 0.0, nullptr, h->lq_u.p, st);
-    // alpha v = M^{-1} (A^T u - beta q)
-    if (timed) record_event(h->ev[7], st);
-    lsq::launch_spmv_csc(csc(h), h->lq_u.p, h->lq_s.p, nullptr, lsq::DotSite{}, h->lanes_csc, h->grid_csc, st);
-    if (timed) mark(h, 1);
-    lsq::launch_axpby(n, 1.0, h->lq_s.p, -beta, h->lq_q.p, h->lq_s.p, st);
-    precond(h, h->lq_s.p, h->lq_t.p, 0, true, false, timed);
-    alpha = std::sqrt(dev_sum(h, lsq::S_RZ));
-    if (dev_sum(h, lsq::S_ERR) != 0.0)
+    if (it == 0) {
+      rhobar = hrep[lsq::L_REP_ALPHA0];
+      est0 = rhobar * phibar;
+      al.push_back(rhobar);
+    }
+    alpha = hrep[lsq::L_REP_ALPHA];
+    if (hrep[lsq::L_REP_ERR] != 0.0)
       throw LsError(LS_ERR_DEVICE_TIMEOUT, "a bounded wait in the local-solve kernel gave up at iteration " +
                                                std::to_string(it + 1));
     if (!(alpha > 0.0) || !std::isfinite(alpha))
@@ -708,20 +750,14 @@ ls_status lsqr_core(ls_handle* h, double rtol, ls_info* info) {
     // plane rotation
     const double rho = std::hypot(rhobar, beta);
     const double c = rhobar / rho, sn = beta / rho;
-    const double theta = sn * alpha;
     rhobar = -c * alpha;
-    const double phi = c * phibar;
     phibar = sn * phibar;
-    lsq::launch_lsqr_step(n, 1.0 / alpha, phi / rho, theta / rho, h->lq_t.p, h->lq_s.p, h->lq_v.p, h->lq_q.p,
-                          h->x.p, h->lq_w.p, st);
-    if (timed) mark(h, 5);
     ++it;
-    launches += 6 + pl + 1;
+    launches += 5 + pl;
     inf.local_launches += 1;
     al.push_back(alpha);
     be.push_back(beta);
     if (timed) {
-      CK(cudaStreamSynchronize(st));
       float ta = 0.f, ta2 = 0.f, tb = 0.f, tc = 0.f, td = 0.f;
       CK(cudaEventElapsedTime(&ta, h->ev[0], h->ev[6]));
       CK(cudaEventElapsedTime(&ta2, h->ev[7], h->ev[1]));
@@ -733,7 +769,7 @@ ls_status lsqr_core(ls_handle* h, double rtol, ls_info* info) {
     if (fixed > 0) continue;
     if (!checking && phibar * alpha * std::fabs(c) <= 10.0 * rtol * est0) checking = true;
     if (checking) {
-      rel = std::sqrt(true_residual(h, 0, &launches)) / gn;
+      rel = std::sqrt(early ? hrep[lsq::L_NREP] : true_residual(h, 0, &launches)) / gn;
       have_rel = true;
       if (rel <= rtol) {
         converged = true;
@@ -743,7 +779,7 @@ ls_status lsqr_core(ls_handle* h, double rtol, ls_info* info) {
   }
   if (!converged || fixed > 0 || !have_rel) rel = std::sqrt(true_residual(h, 0, &launches)) / gn;
   // kappa of M^{-1} A^T A from the bidiagonal: B_k^T B_k is the Lanczos matrix
-  const int k = (int)al.size() - 1;
+  const int k = std::max((int)al.size() - 1, 0);
   if (k >= 1) {
     std::vector<double> d(k), e(std::max(k - 1, 0));
     for (int j = 0; j < k; ++j) {
@@ -758,8 +794,8 @@ ls_status lsqr_core(ls_handle* h, double rtol, ls_info* info) {
 
 // Restarted GMRES on C x = A^T b' (b' in h->bv, result in h->x), right-preconditioned in
 // the flexible form (z_j = M^{-1} v_j kept): Arnoldi with classical Gram-Schmidt applied
-// twice (multi-vector dot and update kernels, deterministic), Givens rotations on the
-// host.  |gamma_{j+1}| = ||A^T b - C x_j||, the configs' residual; a pass (or the end of
+// twice (one kernel per pass over the basis, deterministic), Givens rotations on the
+// host, which waits once per step for the coefficients.  |gamma_{j+1}| = ||A^T b - C x_j||, the configs' residual; a pass (or the end of
 // a cycle) updates x, and every cycle starts from the true residual, which confirms
 // the pass.
 ls_status gmres_core(ls_handle* h, double rtol, ls_info* info) {
@@ -783,13 +819,16 @@ ls_status gmres_core(ls_handle* h, double rtol, ls_info* info) {
                : balanced(h) ? kBalancedLaunches : 2 + ((h->coarse && h->n0 > 0) ? 1 : 0);
   const int fixed = h->opt.fixed_iters;
   const int maxit = fixed > 0 ? fixed : h->opt.maxit;
-  std::vector<double> H((size_t)(mr + 1) * mr, 0.0), cs(mr), sn(mr), gam(mr + 1), hv(2 * (size_t)(mr + 1));
+  std::vector<double> H((size_t)(mr + 1) * mr, 0.0), cs(mr), sn(mr), gam(mr + 1);
   auto Hat = [&](int i, int j) -> double& { return H[(size_t)i * mr + j]; };
   double* V = h->gm_V.p;
   double* Z = h->gm_Z.p;
   double* h1 = h->gm_h.p;
   double* h2 = h->gm_h.p + (mr + 1);
-  double* yv = h->gm_h.p + 2 * (mr + 1);
+  double* hn2 = h->gm_h.p + 2 * (mr + 1);  // ||w||^2 and the error slot, read with h1 and h2
+  double* yv = hn2 + 2;
+  double* hv = h->pin + lsq::S_NSLOT;
+  unsigned* counter = h->counters.p + 3;
   int it = 0;
   bool converged = false;
   double rel = 1.0;
@@ -820,21 +859,19 @@ ls_status gmres_core(ls_handle* h, double rtol, ls_info* info) {
       if (timed) record_event(h->ev[6], st);
       apply_C(h, zj, w);
       if (timed) mark(h, 1);
-      lsq::launch_multi_dot(n, V, n, j + 1, w, h->gm_part.p, h1, st);
-      lsq::launch_multi_axpy(n, V, n, j + 1, h1, -1.0, w, st);
-      lsq::launch_multi_dot(n, V, n, j + 1, w, h->gm_part.p, h2, st);
-      lsq::launch_multi_axpy(n, V, n, j + 1, h2, -1.0, w, st);
-      lsq::launch_dot(n, w, w, site(h, lsq::S_TMP, 3), st);
-      CK(cudaMemcpyAsync(hv.data(), h1, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, st));
-      CK(cudaMemcpyAsync(hv.data() + (mr + 1), h2, sizeof(double) * (j + 1), cudaMemcpyDeviceToHost, st));
-      const double hn = std::sqrt(dev_sum(h));  // synchronises the stream
-      if (dev_sum(h, lsq::S_ERR) != 0.0)
+      lsq::launch_gs_pass(n, V, n, j + 1, nullptr, 0.0, w, 1, h->gm_part.p, counter, h1, st);
+      lsq::launch_gs_pass(n, V, n, j + 1, h1, -1.0, w, 1, h->gm_part.p, counter, h2, st);
+      lsq::launch_gs_pass(n, V, n, j + 1, h2, -1.0, w, 2, h->gm_part.p, counter, hn2, st);
+      lsq::launch_gs_scale(n, hn2, h->scal.p + lsq::S_ERR, hn2 + 1, w, st);
+      if (timed) record_event(h->ev[5], st);
+      CK(cudaMemcpyAsync(hv, h1, sizeof(double) * (2 * (mr + 1) + 2), cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+      const double hn = std::sqrt(hv[2 * (mr + 1)]);
+      if (hv[2 * (mr + 1) + 1] != 0.0)
         throw LsError(LS_ERR_DEVICE_TIMEOUT, "a bounded wait in the local-solve kernel gave up at iteration " +
                                                  std::to_string(it + 1));
       if (!std::isfinite(hn)) throw LsError(LS_ERR_NONFINITE, "GMRES breakdown at iteration " + std::to_string(it + 1));
       if (timed) {
-        record_event(h->ev[5], st);
-        CK(cudaStreamSynchronize(st));
         float ta = 0.f, tb = 0.f, tc = 0.f, td = 0.f;
         CK(cudaEventElapsedTime(&ta, h->ev[6], h->ev[1]));
         CK(cudaEventElapsedTime(&tb, h->ev[2], h->ev[3]));
@@ -844,7 +881,6 @@ ls_status gmres_core(ls_handle* h, double rtol, ls_info* info) {
       }
       for (int i = 0; i <= j; ++i) Hat(i, j) = hv[i] + hv[(mr + 1) + i];
       Hat(j + 1, j) = hn;
-      if (hn > 0.0) lsq::launch_axpby(n, 1.0 / hn, w, 0.0, nullptr, w, st);
       for (int i = 0; i < j; ++i) {
         const double t = cs[i] * Hat(i, j) + sn[i] * Hat(i + 1, j);
         Hat(i + 1, j) = -sn[i] * Hat(i, j) + cs[i] * Hat(i + 1, j);
@@ -859,7 +895,7 @@ ls_status gmres_core(ls_handle* h, double rtol, ls_info* info) {
       gam[j] = cs[j] * gam[j];
       ++j;
       ++it;
-      launches += pl + 2 + 4 * 2 + 1 + (hn > 0.0 ? 1 : 0);
+      launches += pl + 2 + 4;
       inf.local_launches += 1;
       if (fixed > 0 && it >= fixed) break;
       if (fixed <= 0 && (std::fabs(gam[j]) <= rtol * gn || it >= maxit)) break;
@@ -873,7 +909,7 @@ ls_status gmres_core(ls_handle* h, double rtol, ls_info* info) {
       y[i] = s / Hat(i, i);
     }
     CK(cudaMemcpyAsync(yv, y.data(), sizeof(double) * j, cudaMemcpyHostToDevice, st));
-    lsq::launch_multi_axpy(n, Z, n, j, yv, 1.0, h->x.p, st);
+    lsq::launch_gs_pass(n, Z, n, j, yv, 1.0, h->x.p, 0, nullptr, nullptr, nullptr, st);
     CK(cudaStreamSynchronize(st));
     launches += 1;
   }
@@ -1555,11 +1591,13 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     h->gm_V.alloc((size_t)h->n * (mr + 1));
     h->gm_Z.alloc((size_t)h->n * mr);
     h->gm_g.alloc(h->n);
-    h->gm_h.alloc(3 * (size_t)(mr + 1));
+    h->gm_h.alloc(3 * (size_t)(mr + 1) + 2);
+    CK(cudaMemsetAsync(h->gm_h.p, 0, sizeof(double) * (3 * (size_t)(mr + 1) + 2), st));
     h->gm_part.alloc((size_t)lsq::multi_dot_grid(h->n) * (mr + 1));
   }
   if (h->opt.solver == 1) {
     h->lq_u.alloc(h->m);
+    h->lq_k.alloc(lsq::L_NSTATE); h->lq_k.zero(st);
     h->lq_v.alloc(h->n); h->lq_q.alloc(h->n); h->lq_s.alloc(h->n); h->lq_t.alloc(h->n); h->lq_w.alloc(h->n);
   }
   h->parts.alloc(2 * (size_t)lsq::kMaxGrid);
@@ -1568,7 +1606,10 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   h->hist_cap = std::max(h->opt.maxit, h->opt.fixed_iters) + 8;
   h->ahist.alloc(h->hist_cap); h->bhist.alloc(h->hist_cap);
   h->ctr.alloc(1);
-  CK(cudaHostAlloc((void**)&h->pin, sizeof(double) * lsq::S_NSLOT, cudaHostAllocDefault));
+  // the scalar slots, and what a solver reads per step: a value, LSQR's report and residual,
+  // GMRES's coefficients
+  const size_t pins = lsq::S_NSLOT + (h->opt.solver == 2 ? 2 * (size_t)(h->opt.restart + 1) + 2 : lsq::L_NREP + 1);
+  CK(cudaHostAlloc((void**)&h->pin, sizeof(double) * pins, cudaHostAllocDefault));
   if (h->opt.time_kernels)
     for (auto& e : h->ev) CK(cudaEventCreate(&e));
   if (h->sb_ok && h->coarse && h->n0 > 0) {
@@ -1576,7 +1617,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&h->ev_coarse, cudaEventDisableTiming));
   }
-  std::memset(h->pin, 0, sizeof(double) * lsq::S_NSLOT);
+  std::memset(h->pin, 0, sizeof(double) * pins);
   phase.next("ls_setup: sparse-product copies and autotuning");
   job.join();
   if (job_failed) throw LsError(LS_ERR_OOM, "host memory for the sparse-product copies");

@@ -226,15 +226,17 @@ struct ls_handle {
   DevBuf<double> x, r, r_old, z, p, q, w, ybuf, r0, y0, tv, bv;
   DevBuf<double> bal_y, bal_t, bal_u, bal_v;  // work vectors of the balanced variant
   DevBuf<double> lq_u, lq_v, lq_q, lq_s, lq_t, lq_w;  // LSQR: u (m), v, M v, s, M^{-1} s, w
+  DevBuf<double> lq_k;                                // its scalar state and the report
   DevBuf<int64_t> own;                                // RAS: local entry of column j in its own subdomain
   DevBuf<double> gm_V, gm_Z, gm_g, gm_h, gm_part;     // GMRES: Arnoldi basis, M^{-1} basis, A^T b, coefs
   DevBuf<double> parts, scal, ahist, bhist;
   DevBuf<unsigned> counters;  // ticket counters of the fused reductions
   DevBuf<int> ctr;
-  double* pin = nullptr;  // pinned copy of the scalar slots
+  double* pin = nullptr;  // pinned copy of the scalar slots, then the values a solver reads per step
   int hist_cap = 0;
 
   cudaGraphExec_t gexec = nullptr;
+  cudaGraphExec_t lq_exec = nullptr;  // one LSQR step
   cudaEvent_t ev[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};  // kernel timing
   // The PCG loop as one graph: a conditional while node whose body is one iteration and
   // the loop test, then the copy of the scalar slots to the host.  Timing inside it uses
@@ -271,6 +273,7 @@ struct ls_handle {
     if (dev >= 0) cudaSetDevice(dev);
     if (gexec) cudaGraphExecDestroy(gexec);
     if (gloop) cudaGraphExecDestroy(gloop);
+    if (lq_exec) cudaGraphExecDestroy(lq_exec);
     for (auto& e : ev)
       if (e) cudaEventDestroy(e);
     if (ev_join) cudaEventDestroy(ev_join);

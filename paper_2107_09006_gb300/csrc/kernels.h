@@ -109,20 +109,34 @@ struct ScatterArgs {
   double* err;          // error slot (bounds-checked build)
 };
 void launch_scatter(const ScatterArgs& a, cudaStream_t st);
-// One preconditioned LSQR step's vector updates: v = t / alpha, q = s / alpha, x += c1 w,
-// w = v - c2 w.
-void launch_lsqr_step(int64_t n, double inv_alpha, double c1, double c2, const double* t, const double* s, double* v,
-                      double* q, double* x, double* w, cudaStream_t st);
+// LSQR with its scalars on the device.  A step's kernels see the state that the last step
+// left in [0, L_PREV) and a copy of it in [L_PREV, 2 L_PREV), which k_lsqr_s makes for
+// k_lsqr_step to read while it writes the first; L_BETA2 = ||u||^2, then a report of L_NREP
+// values for the host.
+enum { L_INVBETA = 0, L_ALPHA = 1, L_PHIBAR = 2, L_RHOBAR = 3, L_PREV = 4, L_BETA2 = 8, L_REP = 9 };
+enum { L_REP_ALPHA = 0, L_REP_BETA = 1, L_REP_ERR = 2, L_REP_ALPHA0 = 3, L_NREP = 4, L_NSTATE = 13 };
+// u = q - alpha (u / beta) of the last step (u is kept unnormalised, beta = ||u||), with
+// ||u||^2 -> ds.out
+void launch_lsqr_u(int64_t m, const double* state, const double* q, double* u, const DotSite& ds, cudaStream_t st);
+// s = s / beta - beta q (q == nullptr: s = s / beta), beta^2 = state[L_BETA2]
+void launch_lsqr_s(int64_t n, double* state, const double* q, double* s, cudaStream_t st);
+// alpha^2 = scal[S_RZ]: the plane rotation, the vector updates v = t / alpha, q = s / alpha,
+// x += phi/rho w, w = v - theta/rho w (none if alpha or beta is not positive and finite), the
+// next state and the report.  first: the start, w = v.
+void launch_lsqr_step(int64_t n, int first, double* state, const double* scal, const double* t, const double* s,
+                      double* v, double* q, double* x, double* w, cudaStream_t st);
 // RAS prolongation z_j = a_j + y[own[j]] (a may be null)
 void launch_ras_combine(int64_t n, const int64_t* own, const double* y, const double* a, double* z, cudaStream_t st);
-// out[c] = V(:, c) . w for the k columns of V (column-major, ld); part holds
-// multi_dot_grid(n) * k partial sums (deterministic order)
+// One pass over the k columns of V (column-major, ld) for the Gram-Schmidt steps:
+// w += sign * V coef (coef != nullptr, on the device), then, of the new w, next = 1:
+// out[c] = V(:, c) . w for every column, next = 2: out[0] = w . w, next = 0: nothing.  part
+// holds multi_dot_grid(n) * max(k, 1) partial sums, added in a fixed order by the last block
+// (counter, zero before and after).
 int multi_dot_grid(int64_t n);
-void launch_multi_dot(int64_t n, const double* V, int64_t ld, int k, const double* w, double* part, double* out,
-                      cudaStream_t st);
-// out += sign * V coef (V column-major, ld; coef on the device)
-void launch_multi_axpy(int64_t n, const double* V, int64_t ld, int k, const double* coef, double sign, double* out,
-                       cudaStream_t st);
+void launch_gs_pass(int64_t n, const double* V, int64_t ld, int k, const double* coef, double sign, double* w, int next,
+                    double* part, unsigned* counter, double* out, cudaStream_t st);
+// w *= 1 / sqrt(*norm2) (if positive and finite); *err_out = *err
+void launch_gs_scale(int64_t n, const double* norm2, const double* err, double* err_out, double* w, cudaStream_t st);
 // r0 = R_0 v (coarse restriction alone, FP64); kmax: most coarse vectors of a subdomain
 void launch_restrict(int N, int kmax, const int64_t* int_off, const int32_t* int_glob, const int64_t* zoff, const int32_t* coff,
                      const double* Z, const double* v, double* r0, cudaStream_t st);
