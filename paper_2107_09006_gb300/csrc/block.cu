@@ -643,7 +643,7 @@ ls_status block_backward(ls_handle* h, const double* b, const double* x, const d
   const double t0 = now_s();
   ensure_buffers(h, R);
   plan_block_super(h, R);
-  B.G.alloc((size_t)h->n * R);
+  if (B.G.n < (size_t)h->n * R) B.G.alloc((size_t)h->n * R);
   ls_info inf{};
   inf.bad_subdomain = -1;
   int launches = 0;
@@ -674,8 +674,8 @@ ls_status block_backward(ls_handle* h, const double* b, const double* x, const d
     lsq::launch_b_load_rows(h->m, R, h->perm.p, device_view(h, b, h->m, R), B.B.p, st);
     lsq::launch_b_spmm_csr(csr(h), B.Z.p, B.Bu.p, R, st);
     lsq::launch_b_sub((int64_t)h->m * R, B.B.p, B.Bu.p, st);
-    DevBuf<double> gout;
-    gout.alloc(h->nnz);
+    DevBuf<double>& gout = h->bk_out;
+    if ((int64_t)gout.n < h->nnz) gout.alloc(h->nnz);
     lsq::launch_b_grad_vals(csr(h), h->entmap.p, R, B.Bu.p, B.X.p, B.Q.p, B.Z.p, gout.p, st);
     CK(cudaMemcpyAsync(grad_vals, gout.p, sizeof(double) * h->nnz, cudaMemcpyDefault, st));
     CK(cudaStreamSynchronize(st));

@@ -228,6 +228,7 @@ struct ls_handle {
   DevBuf<double> lq_u, lq_v, lq_q, lq_s, lq_t, lq_w;  // LSQR: u (m), v, M v, s, M^{-1} s, w
   DevBuf<double> lq_k;                                // its scalar state and the report
   DevBuf<int64_t> own;                                // RAS: local entry of column j in its own subdomain
+  DevBuf<double> bk_x, bk_lam, bk_mu, bk_m, bk_nnz, bk_out;  // adjoint solve, value update (see reserve)
   DevBuf<double> gm_V, gm_Z, gm_g, gm_h, gm_part;     // GMRES: Arnoldi basis, M^{-1} basis, A^T b, coefs
   DevBuf<double> parts, scal, ahist, bhist;
   DevBuf<unsigned> counters;  // ticket counters of the fused reductions
