@@ -559,53 +559,225 @@ __global__ void __cluster_dims__(kOrthCluster, 1, 1) __launch_bounds__(kThreads)
   }
 }
 
-// Rayleigh-Ritz of the subdomains whose expansion is complete (one CTA each): eigenvalues and
-// vectors of the projected matrix, convergence count, whether it is done, and the restarted
-// projected matrix.
-__global__ void __launch_bounds__(kThreads) k_lz_ritz(EigArgs a, LanczosGrid g, int use_smem) {
-  extern __shared__ __align__(16) double lsm[];
-  __shared__ double cs[kMaxK / 2], sn[kMaxK / 2], red[kWarps], th[kMaxK];
-  __shared__ int pp[kMaxK / 2], qq[kMaxK / 2], ord[kMaxK];
-  const int i = blockIdx.x;
+// Rayleigh-Ritz of the subdomains whose expansion is complete: eigenvalues and vectors of the
+// projected matrix, convergence count, whether it is done, and the restarted projected matrix.
+// The rotations are those of jacobi(), bound by the FP64 units of the SM that makes them (3.7 ms
+// for a basis of 58 on one CTA), so a pair of CTAs shares them: rank 0 holds the matrix and
+// makes the rotations, rank 1 applies them to the eigenvectors while rank 0 updates the
+// matrix.  The update takes two pairs' 2 x 2 block at a time and uses the symmetry (16 FP64
+// instructions for its four entries and their mirror images; 32 by rows, then columns), and
+// pairs whose entry is so small that all such entries together pass the convergence test are
+// left alone (at first most of a Lanczos matrix, near the end most pairs): 1.8 ms so.
+constexpr int kMaxHalf = kMaxK / 2;
+struct RotMsg {  // the rotations of one round, from rank 0 to rank 1
+  int n;         // -1: no more rounds
+  int pq[kMaxHalf];
+  double c[kMaxHalf], s[kMaxHalf];
+};
+template <class T>
+__device__ __forceinline__ uint32_t lz_remote(const T* p, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void lz_put(uint32_t at, int v) {
+  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(at), "r"(v) : "memory");
+}
+__device__ __forceinline__ void lz_put(uint32_t at, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(v) : "memory");
+}
+__device__ __forceinline__ void lz_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void lz_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Rank 1: S <- S R for every round's rotations R, St = S^T (K x K) in shared memory.  The
+// ranks' barrier counts match: one arrive and wait per round and one for the end.
+__device__ void ritz_vectors(double* St, int K, int np, RotMsg* msg) {
+  for (int e = threadIdx.x; e < np * np; e += kThreads) St[(e / np) * K + e % np] = e / np == e % np ? 1.0 : 0.0;
+  for (int turn = 0;; ++turn) {
+    lz_arrive();  // the last round's update is done
+    lz_wait();    // this round's rotations have come
+    const RotMsg& m = msg[turn & 1];
+    if (m.n < 0) return;
+    for (int e = threadIdx.x; e < m.n * np; e += kThreads) {
+      const int k = e / np, row = e - k * np;
+      const double c = m.c[k], sn = m.s[k];
+      double* a = St + (m.pq[k] & 0xffff) * K + row;
+      double* b = St + (m.pq[k] >> 16) * K + row;
+      const double sp = *a, sq = *b;
+      *a = c * sp - sn * sq;
+      *b = sn * sp + c * sq;
+    }
+  }
+}
+
+// Rank 0: the rotations, H <- R^T H R (H np x np in a K x K buffer, upper triangle valid on
+// entry) until it is diagonal.
+__device__ void ritz_matrix(double* H, int K, int n, int np, RotMsg* msg, double* cs, double* sn, int* pp, int* qq,
+                            int (*cnt)[2], double* red) {
+  for (int e = threadIdx.x; e < np * np; e += kThreads) {
+    const int r = e / np, c = e % np;
+    if (r > c && r < n) H[r * K + c] = H[c * K + r];
+    if (r >= n || c >= n) H[r * K + c] = 0.0;
+  }
+  if (threadIdx.x < 2) cnt[0][threadIdx.x] = 0;
+  __syncthreads();
+  const int half = np / 2;
+  int turn = 0;
+  for (int sweep = 0; sweep < 40; ++sweep) {
+    double off = 0.0, dia = 0.0;
+    for (int e = threadIdx.x; e < np * np; e += kThreads) {
+      const int r = e / np, c = e % np;
+      const double v = H[r * K + c];
+      if (r != c) off += v * v; else dia += v * v;
+    }
+    off = block_sum(off, red);
+    dia = block_sum(dia, red);
+    if (off <= 1e-30 * (dia + off) || off == 0.0) break;
+    const double small = 0.25e-30 * (dia + off) / ((double)np * np);
+    for (int round = 0; round < np - 1; ++round, ++turn) {
+      RotMsg& out = msg[turn & 1];
+      int* count = cnt[turn & 1];
+      if (threadIdx.x >= kThreads - 2) cnt[(turn + 1) & 1][kThreads - 1 - threadIdx.x] = 0;
+      if ((int)threadIdx.x < half) {
+        const int k = threadIdx.x;
+        int p, q;
+        if (k == 0) { p = round; q = np - 1; }
+        else { p = (round + k) % (np - 1); q = (round - k + np - 1) % (np - 1); }
+        if (p > q) { const int t = p; p = q; q = t; }
+        const double apq = H[p * K + q];
+        if (!(apq * apq <= small)) {  // (a NaN is rotated, as in jacobi)
+          const double app = H[p * K + p], aqq = H[q * K + q];
+          const double th = (aqq - app) / (2.0 * apq);
+          const double t = (th >= 0 ? 1.0 : -1.0) / (fabs(th) + sqrt(1.0 + th * th));
+          const double c = 1.0 / sqrt(1.0 + t * t), s = t * c;
+          H[p * K + p] = app - t * apq;
+          H[q * K + q] = aqq + t * apq;
+          H[p * K + q] = 0.0;
+          H[q * K + p] = 0.0;
+          const int at = atomicAdd(count, 1);
+          pp[at] = p; qq[at] = q; cs[at] = c; sn[at] = s;
+          lz_put(lz_remote(&out.pq[at], 1), p | q << 16);
+          lz_put(lz_remote(&out.c[at], 1), c);
+          lz_put(lz_remote(&out.s[at], 1), s);
+        } else {
+          const int at = half - 1 - atomicAdd(count + 1, 1);
+          pp[at] = p; qq[at] = q; cs[at] = 1.0; sn[at] = 0.0;
+        }
+      }
+      __syncthreads();
+      const int na = count[0], rest = half - na;
+      if (threadIdx.x == 0) lz_put(lz_remote(&out.n, 1), na);
+      lz_arrive();  // the rotations have gone (and the last round's are read: the wait below)
+      const int mixed = na * rest, items = mixed + na * (na - 1) / 2;
+      for (int e = threadIdx.x; e < items; e += kThreads) {
+        int k, l;  // two different pairs, k < l, the first of them rotated
+        if (e < mixed) {
+          k = e / rest;
+          l = na + e - k * rest;
+        } else {
+          const int x = e - mixed;  // triangular number: x = l (l - 1) / 2 + k
+          l = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)x)) * 0.5f);
+          if (l * (l - 1) / 2 > x) --l;
+          if (l * (l + 1) / 2 <= x) ++l;
+          k = x - l * (l - 1) / 2;
+        }
+        const int p = pp[k], q = qq[k], u = pp[l], v = qq[l];
+        const double ck = cs[k], sk = sn[k], cl = cs[l], sl = sn[l];
+        const double a = H[p * K + u], b = H[p * K + v], c = H[q * K + u], d = H[q * K + v];
+        const double a1 = ck * a - sk * c, b1 = ck * b - sk * d, c1 = sk * a + ck * c, d1 = sk * b + ck * d;
+        const double a2 = cl * a1 - sl * b1, b2 = sl * a1 + cl * b1, c2 = cl * c1 - sl * d1, d2 = sl * c1 + cl * d1;
+        H[p * K + u] = a2; H[u * K + p] = a2;
+        H[p * K + v] = b2; H[v * K + p] = b2;
+        H[q * K + u] = c2; H[u * K + q] = c2;
+        H[q * K + v] = d2; H[v * K + q] = d2;
+      }
+      __syncthreads();
+      lz_wait();
+    }
+  }
+  if (threadIdx.x == 0) lz_put(lz_remote(&msg[turn & 1].n, 1), -1);
+  lz_arrive();
+  lz_wait();
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads) k_lz_ritz(EigArgs a, LanczosGrid g) {
+  extern __shared__ __align__(16) double M[];  // rank 0: the projected matrix, rank 1: its eigenvectors, transposed
+  __shared__ RotMsg msg[2];
+  __shared__ double cs[kMaxHalf], sn[kMaxHalf], red[kWarps], th[kMaxK], res[kMaxK];
+  __shared__ int pp[kMaxHalf], qq[kMaxHalf], ord[kMaxK], cnt[2][2];
+  const int i = blockIdx.x / 2, rank = blockIdx.x % 2;
   const LzState st = lz_state(g, a.P.N);
-  if (st.phase[i] != 1) return;
+  if (st.phase[i] != 1) return;  // (both CTAs)
   const int ni = (int)(a.P.om_off[i + 1] - a.P.om_off[i]);
   const int K = a.Kmax, nV = st.nV[i], steps = st.steps[i];
+  const int np = nV + (nV & 1);  // even size; the extra index is an isolated zero
   const int kw = min(a.kwant_cap, ni), Keff = min(K, ni);
   const int keep = max(kw, min(a.keep, Keff - 1));
   double* Hg = a.H + (int64_t)i * K * K;
   double* Sg = a.S + (int64_t)i * K * K;
-  double* H = use_smem ? lsm : Hg;
-  double* S = use_smem ? lsm + K * K : Sg;
-  Shared s{};
-  s.cs = cs; s.sn = sn; s.red = red; s.pp = pp; s.qq = qq; s.ord = ord;
-  if (use_smem) {
-    for (int e = threadIdx.x; e < K * K; e += kThreads) H[e] = Hg[e];
+  if (rank == 1) {
+    lz_arrive();  // both ranks run: their shared memory may be written
+    lz_wait();
+    ritz_vectors(M, K, np, msg);
     __syncthreads();
+    lz_arrive();  // rank 0 may read the last row
+    for (int e = threadIdx.x; e < K * K; e += kThreads) {
+      const int r = e / K, c = e % K;
+      Sg[e] = r < nV && c < nV ? M[c * K + r] : 0.0;
+    }
+    lz_wait();
+    lz_arrive();  // rank 0 has read it
+    lz_wait();
+    return;
   }
-  jacobi(H, S, K, nV, s);
+  for (int e = threadIdx.x; e < K * K; e += kThreads) M[e] = Hg[e];
+  __syncthreads();
+  lz_arrive();
+  lz_wait();
+  ritz_matrix(M, K, nV, np, msg, cs, sn, pp, qq, cnt, red);
+  for (int t = threadIdx.x; t < nV; t += kThreads) ord[t] = t;
+  __syncthreads();
+  for (int t = threadIdx.x; t < nV; t += kThreads) {
+    const double v = M[t * K + t];
+    int r = 0;
+    for (int u = 0; u < nV; ++u) {
+      const double w = M[u * K + u];
+      if (w > v || (w == v && u < t)) ++r;
+    }
+    ord[r] = t;
+  }
+  __syncthreads();
   const double beta = g.beta[i];
   const int kk = min(kw, nV);
-  int nconv = 0;
-  const double th0 = fabs(H[ord[0] * K + ord[0]]);
-  for (int t = 0; t < kk; ++t) {
-    const double res = beta * fabs(S[(nV - 1) * K + ord[t]]);
-    if (res <= a.tol * fmax(th0, 1e-300)) ++nconv; else break;
+  lz_arrive();
+  lz_wait();
+  for (int t = threadIdx.x; t < kk; t += kThreads) res[t] = beta * fabs(lz_peer(&M[ord[t] * K + nV - 1], 1));
+  for (int t = threadIdx.x; t < nV; t += kThreads) {
+    th[t] = M[ord[t] * K + ord[t]];
+    g.ord[(int64_t)i * K + t] = ord[t];
   }
-  const bool done = nconv >= kk || nV >= ni || steps >= a.maxit;
-  const int cnt = done ? kk : keep;
-  for (int t = threadIdx.x; t < cnt; t += kThreads) th[t] = H[ord[t] * K + ord[t]];
-  for (int t = threadIdx.x; t < nV; t += kThreads) g.ord[(int64_t)i * K + t] = ord[t];
   __syncthreads();
+  lz_arrive();
+  lz_wait();
+  int nconv = 0;
+  const double bound = a.tol * fmax(fabs(th[0]), 1e-300);
+  while (nconv < kk && res[nconv] <= bound) ++nconv;
+  const bool done = nconv >= kk || nV >= ni || steps >= a.maxit;
+  const int cntk = done ? kk : keep;
   for (int e = threadIdx.x; e < K * K; e += kThreads) {
     const int r = e / K, c = e % K;
-    if (use_smem) Sg[e] = (r < nV && c < nV) ? S[e] : 0.0;
-    Hg[e] = (r == c && r < cnt) ? th[r] : 0.0;
+    Hg[e] = (r == c && r < cntk) ? th[r] : 0.0;
   }
   if (done)
     for (int t = threadIdx.x; t < kk; t += kThreads) a.lam[(int64_t)i * a.kwant_cap + t] = th[t];
   if (threadIdx.x == 0) {
-    g.rr[i] = cnt;
+    g.rr[i] = cntk;
     g.rr[a.P.N + i] = done ? 1 : 0;
     a.nconv[i] = nconv;
     a.steps[i] = steps;
@@ -725,9 +897,7 @@ bool run_lanczos_grid(const EigArgs& a, const LanczosGrid& g, cudaStream_t st) {
   fwd.dst = a.vec + a.vstride;
   fwd.sweeps = 1;
   const size_t orth_sm = (size_t)((a.vstride / kT + kOrthCluster - 1) / kOrthCluster * kT) * sizeof(double);
-  const size_t ritz_full = 2 * (size_t)K * K * sizeof(double);
-  const int ritz_use = ritz_full <= 200 * 1024;
-  const size_t ritz_sm = ritz_use ? ritz_full : 0;
+  const size_t ritz_sm = (size_t)K * K * sizeof(double);  // (K <= 160: at most 200 KB)
   if (cudaFuncSetAttribute(k_lz_orth, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess ||
       cudaFuncSetAttribute(k_lz_ritz, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
     return false;
@@ -748,7 +918,7 @@ bool run_lanczos_grid(const EigArgs& a, const LanczosGrid& g, cudaStream_t st) {
     }
     steps += run;
     basis = a.keep + 1;
-    k_lz_ritz<<<N, kThreads, ritz_sm, st>>>(a, g, ritz_use);
+    k_lz_ritz<<<2 * N, kThreads, ritz_sm, st>>>(a, g);
     k_lz_rotate<<<rot_grid, kThreads, 0, st>>>(a, g);
     k_lz_flip<<<(N + 127) / 128, 128, 0, st>>>(a, g);
     k_lz_orth<<<N * kOrthCluster, kThreads, orth_sm, st>>>(a, g);  // (the restarting ones append their residual)

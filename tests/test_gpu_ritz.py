@@ -1,0 +1,33 @@
+"""The projected eigenproblems of the local eigensolves on a pair of CTAs: the smallest basis
+(48), the usual one (58), the largest (160), subdomains smaller than the basis and of odd
+size.  Eigenvalues against the oracle's dense solver, with the bound of the parity tests, and
+the preconditioner with the coarse space they select."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - CPU containers
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import paper_2107_09006_gb300 as L  # noqa: E402
+import oracle as O  # noqa: E402
+from workloads import make_grid_ls, block_partition  # noqa: E402
+
+
+@pytest.mark.parametrize("W,H,piece,nev", [(30, 30, 15, 4), (30, 30, 15, 16), (40, 24, 20, 67), (15, 9, 5, 6), (7, 7, 3, 3)])
+def test_projected_eigenproblem(W, H, piece, nev):
+    m, n, rp, c, v, b, _ = make_grid_ls(W, H, 4, 6, 2, 11)
+    part = block_partition(W, H, piece, piece)
+    N = int(part.max()) + 1
+    S = L.Solver(m, n, rp, c, v, part, N, nev_max=nev)
+    M = O.build_two_level(O.schwarz.as_csr(m, n, rp, c, v), part, N, tau=0.0, nev_max=nev)
+    for i in range(N):
+        lg = S.eigvals(i)
+        lo = M.lams[i][: len(lg)]
+        assert np.max(np.abs(lg - lo)) <= 1e-10 * max(1.0, np.abs(lo).max())
+    r = np.random.default_rng(3).standard_normal(n)
+    z, ref = S.apply_preconditioner(r, 0).cpu().numpy(), M.apply(r)
+    assert np.linalg.norm(z - ref) <= 1e-9 * np.linalg.norm(ref)
+    S.close()
