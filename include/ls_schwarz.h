@@ -108,8 +108,11 @@ typedef struct {
                           returns with nothing in flight, and the solve returns
                           LS_ERR_DEVICE_TIMEOUT.  The CUDA context stays usable.      */
     int block_kernel;  /* local solve of the multi right-hand-side path with FP32 factors:
-                          0 (the default) times both at the first block solve and keeps
-                          the faster; 1 TF32 mma.sync tiles, left-looking sweeps; 2
+                          0 (the default) takes the sweeps over superblocks of 128 rows
+                          (all factor precisions; local_kernel reports 0) where they fit
+                          and the solve is not so wide that the 32-row sweeps fill the
+                          chip several times over, else times both of those at the first
+                          block solve and keeps the faster; 1 TF32 mma.sync tiles, left-looking sweeps; 2
                           tcgen05 MMAs (M = 128, accumulator in tensor memory),
                           right-looking sweeps (LS_ERR_UNSUPPORTED if the widest factor
                           block row does not fit its shared-memory window).  Both round
@@ -171,8 +174,8 @@ typedef struct {
     int launches;            /* kernels launched by the last solve (all of this library's)  */
     double ms_iter;          /* with time_kernels: total ms of whole CG iterations (kernels) */
     int lanes_csr, lanes_csc;/* kernel codes of the products with A / A^T (option spmv)    */
-    int local_kernel;        /* local-solve kernel of the last solve: 0 the single-vector or
-                                CUDA-core block kernel, 1 TF32 mma.sync block kernel, 2
+    int local_kernel;        /* local-solve kernel of the last solve: 0 the single-vector,
+                                superblock or CUDA-core block kernel, 1 TF32 mma.sync block kernel, 2
                                 tcgen05 block kernel                                       */
     int normal_product;      /* form of the A^T (A v) products: 1 two products, 2 row tiles */
     int local_config;        /* configuration of the single-vector local solve (option)      */

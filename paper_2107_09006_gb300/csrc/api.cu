@@ -1210,6 +1210,11 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     }
   });
 
+  if (h->coarse) {
+    CK(cudaStreamCreateWithFlags(&h->st2, cudaStreamNonBlocking));
+    CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
+    CK(cudaEventCreateWithFlags(&h->ev_coarse, cudaEventDisableTiming));
+  }
   // local plan
   phase.next("ls_setup: local matrices and Cholesky factors");
   h->total_local = hs.om_off[N];
@@ -1282,9 +1287,10 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   Ctst.alloc(h->fac_elems); Ctst.zero(st);
   lsq::launch_assemble(plan, csr(h), csc(h), h->part.p, h->total_local, Cst.p, Ctst.p, st);
   check_launch("assembly");
-  DevBuf<double> cn2, ctn2, sdev;
+  DevBuf<double> cn2, ctn2, sdev, dinv;
   cn2.alloc(N); ctn2.alloc(N);
-  lsq::launch_norms(plan, Cst.p, Ctst.p, cn2.p, ctn2.p, st);
+  dinv.alloc((size_t)h->total_blocks * 1024);  // (its first use: the partial sums of the norms)
+  lsq::launch_norms(plan, h->max_nb, Cst.p, Ctst.p, dinv.p, cn2.p, ctn2.p, st);
   std::vector<double> hcn2(N), hctn2(N);
   CK(cudaMemcpyAsync(hcn2.data(), cn2.p, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(hctn2.data(), ctn2.p, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
@@ -1306,14 +1312,26 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   sdev.upload(hs_shift, st);
   h->eqs.alloc(h->total_local);
   Bst.alloc(h->fac_elems);  // prep always writes B = C~_ii + s I
-  lsq::launch_prep(plan, h->dsub.p, sdev.p, Cst.p, h->eqs.p, Ctst.p, Bst.p, st);
+  lsq::launch_prep(plan, h->max_nb, h->dsub.p, sdev.p, Cst.p, h->eqs.p, Ctst.p, Bst.p, st);
   check_launch("prep");
-  DevBuf<double> dinv, Bidiag, idiag;
-  DevBuf<int> status;
-  dinv.alloc((size_t)h->total_blocks * 1024);
+  DevBuf<double> Bidiag, Bdinv, idiag;
+  DevBuf<int> status, Bstatus;
   status.alloc(N);
   idiag.alloc((size_t)h->total_blocks * 32);
+  if (h->coarse) {
+    // The two factorisations, each a chain of small launches, run beside one another; the
+    // solve's stream waits for both before anything else.  (16 subdomains of 1,450 columns:
+    // 9.3 ms one after the other, about 6 so)
+    Bidiag.alloc((size_t)h->total_blocks * 32);
+    Bdinv.alloc((size_t)h->total_blocks * 1024);
+    Bstatus.alloc(N);
+    CK(cudaEventRecord(h->ev_fork, st));
+    CK(cudaStreamWaitEvent(h->st2, h->ev_fork, 0));
+    lsq::launch_band_cholesky(plan, h->max_nb, h->wmax, Bst.p, Bidiag.p, Bdinv.p, Bstatus.p, h->st2);
+    CK(cudaEventRecord(h->ev_coarse, h->st2));
+  }
   lsq::launch_band_cholesky(plan, h->max_nb, h->wmax, Cst.p, idiag.p, dinv.p, status.p, st);
+  if (h->coarse) CK(cudaStreamWaitEvent(st, h->ev_coarse, 0));
   std::vector<int> hst(N);
   CK(cudaMemcpyAsync(hst.data(), status.p, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -1372,9 +1390,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   if (h->coarse) {
     const double te0 = now_s();
     phase.next("ls_setup: local eigensolves and coarse operator");
-    Bidiag.alloc((size_t)h->total_blocks * 32);
-    lsq::launch_band_cholesky(plan, h->max_nb, h->wmax, Bst.p, Bidiag.p, dinv.p, status.p, st);
-    CK(cudaMemcpyAsync(hst.data(), status.p, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(hst.data(), Bstatus.p, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     check_launch("Cholesky of C~_ii + s I");
     for (int i = 0; i < N; ++i)
@@ -1382,6 +1398,14 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
         h->sinfo.bad_subdomain = i;
         throw LsError(LS_ERR_FACTOR, "Cholesky of C~_ii + s I failed in subdomain " + std::to_string(i));
       }
+    DevBuf<int64_t> xi_off;
+    DevBuf<int32_t> xi, xi_sub;
+    xi_off.upload(hs.xi_off, st);
+    xi.upload(hs.xi, st);
+    std::vector<int32_t> xs(hs.xi_off[N]);
+    for (int i = 0; i < N; ++i)
+      for (int64_t a = hs.xi_off[i]; a < hs.xi_off[i + 1]; ++a) xs[a] = i;
+    xi_sub.upload(xs, st);
     const int kw = h->kwant_cap;
     int K = std::max(48, 2 * kw + 24);
     K += K & 1;
@@ -1404,11 +1428,13 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     // CTA per subdomain
     lsq::LanczosGrid lg{};
     DevBuf<int> lz_state, lz_rr, lz_ord;
-    DevBuf<double> lz_beta, lz_err;
+    DevBuf<double> lz_beta, lz_err, lz_rows;
+    DevBuf<int32_t> lz_xpos;
     {
       int optin = 0;
       CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
-      if (lsq::local_super_plan(0, N, h->max_nb, std::max(h->wmax, lsq::kSuperRows),
+      if (hs.xi_off[N] < INT32_MAX &&
+          lsq::local_super_plan(0, N, h->max_nb, std::max(h->wmax, lsq::kSuperRows),
                                 (double)h->fac_elems / 1024.0 / (double)h->total_blocks, sms, (size_t)optin, lg.shape)) {
         Ctst.release();  // (the operator runs from A)
         const lsi::SuperHost sh = lsi::super_storage(hs.blk_off, hs.blk_tf, N, LS_PREC_F64);
@@ -1418,7 +1444,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
         etf.upload(sh.tf, st); eoff.upload(sh.off, st); eorder.upload(sh.order, st);
         efac.alloc((size_t)sh.bytes);
         lsq::launch_super_pack(LS_PREC_F64, N, h->max_nb, h->blk_off.p, h->blk_tf.p, h->blk_poff.p, etf.p, eoff.p,
-                               Bst.p, dinv.p, efac.p, st);
+                               Bst.p, Bdinv.p, efac.p, st);
         std::vector<int32_t> lp((size_t)h->n, 0);
         for (int i = 0; i < N; ++i)
           for (int64_t a = hs.int_off[i]; a < hs.int_off[i + 1]; ++a)
@@ -1426,6 +1452,9 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
         locpos.upload(lp, st);
         lz_state.alloc((size_t)N * lsq::kLanczosState); lz_rr.alloc((size_t)N * 2); lz_ord.alloc((size_t)N * K);
         lz_beta.alloc(N); lz_err.alloc(1); lz_err.zero(st);
+        lz_rows.alloc((size_t)std::max<int64_t>(hs.xi_off[N], 1)); lz_xpos.alloc((size_t)nnz);
+        lg.total_xi = hs.xi_off[N];
+        lg.xi_off = xi_off.p; lg.xi = xi.p; lg.xi_sub = xi_sub.p; lg.xpos = lz_xpos.p; lg.rows = lz_rows.p;
         lg.fac.order = eorder.p;
         lg.fac.om_off = h->om_off.p; lg.fac.om_glob = h->om_glob.p; lg.fac.eqs = h->eqs.p;
         lg.fac.blk_off = h->blk_off.p; lg.fac.tf = etf.p; lg.fac.toff = eoff.p; lg.fac.fac = efac.p;
@@ -1501,18 +1530,10 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     check_launch("coarse basis");
     V.release(); V2.release(); H.release(); S.release(); vec.release();
     if (h->n0 > 0) {
-      DevBuf<int64_t> woff, xi_off, poff;
-      DevBuf<int32_t> xi, xi_sub, pi, pj, ppi, ppj;
+      DevBuf<int64_t> woff, poff;
+      DevBuf<int32_t> pi, pj, ppi, ppj;
       DevBuf<double> W;
       woff.upload(hwoff, st);
-      xi_off.upload(hs.xi_off, st);
-      xi.upload(hs.xi, st);
-      {
-        std::vector<int32_t> xs(hs.xi_off[N]);
-        for (int i = 0; i < N; ++i)
-          for (int64_t a = hs.xi_off[i]; a < hs.xi_off[i + 1]; ++a) xs[a] = i;
-        xi_sub.upload(xs, st);
-      }
       W.alloc(std::max<int64_t>(hwoff[N], 1));
       lsq::launch_coarse_w(N, xi_off.p, xi.p, h->coff.p, woff.p, h->zoff.p, h->nI.p, csr(h), h->part.p, h->jj_of.p,
                            h->Z.p, W.p, hs.xi_off[N], xi_sub.p, st);
@@ -1619,11 +1640,6 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   CK(cudaHostAlloc((void**)&h->pin, sizeof(double) * pins, cudaHostAllocDefault));
   if (h->opt.time_kernels)
     for (auto& e : h->ev) CK(cudaEventCreate(&e));
-  if (h->sb_ok && h->coarse && h->n0 > 0) {
-    CK(cudaStreamCreateWithFlags(&h->st2, cudaStreamNonBlocking));
-    CK(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&h->ev_coarse, cudaEventDisableTiming));
-  }
   std::memset(h->pin, 0, sizeof(double) * pins);
   phase.next("ls_setup: sparse-product copies and autotuning");
   job.join();

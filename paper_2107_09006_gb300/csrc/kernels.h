@@ -159,12 +159,12 @@ struct BandPlan {
 void launch_assemble(const BandPlan& P, const CsrDev& A, const CscDev& At, const int32_t* part,
                      int64_t total_local, double* Cst, double* Ctst, cudaStream_t st);
 // Per subdomain: cn2[i] = sum over interior rows of C of squared row norms (so that
-// sum_i cn2[i] = ||C||_F^2); ctn2[i] = ||C~_ii||_F^2.
-void launch_norms(const BandPlan& P, const double* Cst, const double* Ctst, double* cn2,
+// sum_i cn2[i] = ||C||_F^2); ctn2[i] = ||C~_ii||_F^2.  parts: two doubles per block row.
+void launch_norms(const BandPlan& P, int max_nb, const double* Cst, const double* Ctst, double* parts, double* cn2,
                   double* ctn2, cudaStream_t st);
 // C_ii += delta_i I (dsub: one shift per subdomain, the shift of its problem),
 // equilibrate C_ii with eqs = diag(C_ii)^{-1/2}; B_i = C~_ii + s_i I.
-void launch_prep(const BandPlan& P, const double* dsub, const double* s, double* Cst, double* eqs,
+void launch_prep(const BandPlan& P, int max_nb, const double* dsub, const double* s, double* Cst, double* eqs,
                  const double* Ctst, double* Bst, cudaStream_t st);
 // In-place Cholesky of every subdomain's matrix; idiag = 1 / diag(L);
 // status[i] = 0 or 1 + the local row of the first nonpositive pivot.
@@ -272,6 +272,10 @@ struct LanczosGrid {
   const int32_t* part;
   const int32_t* locpos;  // position of column j in its own subdomain's Omega
   int64_t total_local;
+  int64_t total_xi;       // rows that touch a subdomain's interior columns, all subdomains
+  const int64_t* xi_off; const int32_t* xi; const int32_t* xi_sub;
+  int32_t* xpos;          // [nnz] of entry (r, j) of A^T: the place of r among the rows of j's subdomain
+  double* rows;           // [total_xi]
   int* state;             // [5][N]: basis size, steps, phase, buffer (0: V, 1: V2), fresh starts
   int* rr;                // [2][N]: kept vectors, done
   int* ord;               // [N][K] Ritz order
