@@ -108,10 +108,11 @@ struct BlockState {
   DevBuf<double> X, Rv, Rold, Z, P, W, Q, B, Y, R0, Y0, Bu, G;
   DevBuf<unsigned char> Vg;          // forward-sweep spill of the local solves
   DevBuf<double> parts, sc;          // chunk partials; per (problem, rhs) scalars
-  DevBuf<int> act, its, stat;        // active mask, iterations, {nact, flag, err}
+  DevBuf<int> act, its, stat;        // active mask, iterations, {nact, flag, iterations of the loop}
   DevBuf<unsigned> qctr;             // work counter of the persistent local solve
-  int* pin = nullptr;                // pinned copy of stat
-  cudaGraphExec_t gexec = nullptr;
+  int* pin = nullptr;                // pinned: stat, and from [4] on the error slot (a double)
+  cudaGraphExec_t gexec = nullptr;   // one iteration, or (loop) the device-side loop over it
+  bool loop = false;
   int gR = 0;
   // reduction chunks: column ranges inside one problem
   int64_t nchunks = 0;

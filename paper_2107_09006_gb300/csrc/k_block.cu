@@ -183,12 +183,20 @@ __global__ void __launch_bounds__(kCT) k_b_update(BChunks ch, int R, int Rp, con
   }
 }
 
-// P = Z + beta P (init: P = Z).
+// P = Z + beta P (init: P = Z).  In the body of the device-side loop (loop.limit > 0) the
+// launch is also its test: continue while a pair is active, none has broken down, no wait has
+// timed out and fewer than loop.limit iterations have run.
 __global__ void __launch_bounds__(kCT) k_b_pupdate(BChunks ch, int R, int Rp, const double* __restrict__ beta,
                                                         const double* __restrict__ Z, double* __restrict__ P,
-                                                        int init) {
+                                                        int init, BLoopTest loop) {
   const Lanes L(Rp);
   const int w = threadIdx.x >> 5;
+  if (loop.limit > 0 && blockIdx.x == 0 && threadIdx.x == 0) {
+    const int done = loop.stat[2] + 1;
+    loop.stat[2] = done;
+    const bool go = loop.stat[0] > 0 && loop.stat[1] == 0 && *loop.err == 0.0 && done < loop.limit;
+    cudaGraphSetConditional(loop.handle, go ? 1u : 0u);
+  }
   if (L.k >= R) return;
   for (int64_t c = blockIdx.x; c < ch.n; c += gridDim.x) {
     const int64_t s = ch.start[c], e = ch.start[c + 1];
@@ -200,37 +208,66 @@ __global__ void __launch_bounds__(kCT) k_b_pupdate(BChunks ch, int R, int Rp, co
   }
 }
 
-// Finishing block per problem: sums the chunk partials (in chunk order within each of its 32
-// warps, then the warps) and applies the CG scalar step of `mode` to every right-hand side of
-// the problem.
+// Finishing block per problem: sums the chunk partials (in chunk order within the lanes of its
+// 32 warps, then over them in a fixed order) and applies the CG scalar step of `mode` to every
+// right-hand side of the problem.  A chain of FP64 additions, each 64 cycles of a warp's
+// sub-partition: a warp takes 32 / Rp chunks at a time and eight warps add the warps' sums
+// first (256 chunks, R = 8: 5.7 us, 7.2 with a chunk per warp and one chain of 32).
 constexpr int kFT = 1024, kFW = kFT / 32;
 __global__ void __launch_bounds__(kFT) k_b_finish(const int64_t* __restrict__ pc_off,
                                                        const double* __restrict__ part,
-                                                       const double* __restrict__ part2, int R, BScal s, int mode,
-                                                       int flex) {
+                                                       const double* __restrict__ part2, int R, int Rp, BScal s,
+                                                       int mode, int flex) {
   __shared__ double red[kFW][32], red2[kFW][32];
   __shared__ int cnt;
   const int q = blockIdx.x;
-  const int w = threadIdx.x >> 5, k = threadIdx.x & 31;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t c0 = pc_off[q], c1 = pc_off[q + 1];
   double a = 0.0, b = 0.0;
-  if (k < R) {
+  {
+    const Lanes L(Rp);
+    if (L.k < R) {
 #pragma unroll 4
-    for (int64_t c = c0 + w; c < c1; c += kFW) {
-      a += part[c * 32 + k];
-      if (part2) b += part2[c * 32 + k];
+      for (int64_t c = c0 + w * L.G + L.g; c < c1; c += kFW * L.G) {
+        a += part[c * 32 + L.k];
+        if (part2) b += part2[c * 32 + L.k];
+      }
+    }
+    for (int o = Rp; o < 32; o <<= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (part2) b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (lane < Rp) {
+      red[w][lane] = a;
+      red2[w][lane] = b;
     }
   }
-  red[w][k] = a;
-  red2[w][k] = b;
-  if (threadIdx.x == 0) cnt = 0;
+  if (threadIdx.x == 0) {
+    cnt = 0;
+    if (mode == kFinAlpha && q == 0) s.stat[0] = 0;  // (counted anew by this iteration's kFinRR)
+  }
+  __syncthreads();
+  if (w < kFW / 4) {
+    a = 0.0;
+    b = 0.0;
+    if (lane < Rp) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        a += red[w + u * (kFW / 4)][lane];
+        if (part2) b += red2[w + u * (kFW / 4)][lane];
+      }
+      red[w][lane] = a;
+      red2[w][lane] = b;
+    }
+  }
   __syncthreads();
   if ((int)threadIdx.x < R) {
+    const int k = threadIdx.x;
     double x = 0.0, y = 0.0;
 #pragma unroll
-    for (int u = 0; u < kFW; ++u) {
+    for (int u = 0; u < kFW / 4; ++u) {
       x += red[u][k];
-      y += red2[u][k];
+      if (part2) y += red2[u][k];
     }
     const int64_t i = (int64_t)q * R + k;
     const int act = s.act[i];
@@ -1216,13 +1253,13 @@ void launch_b_update(const BChunks& ch, int R, const double* alpha, const double
 }
 
 void launch_b_pupdate(const BChunks& ch, int R, const double* beta, const double* Z, double* P, int init,
-                      cudaStream_t st) {
-  k_b_pupdate<<<grid_chunks(ch.n), kCT, 0, st>>>(ch, R, pow2_at_least(R), beta, Z, P, init);
+                      const BLoopTest* loop, cudaStream_t st) {
+  k_b_pupdate<<<grid_chunks(ch.n), kCT, 0, st>>>(ch, R, pow2_at_least(R), beta, Z, P, init, loop ? *loop : BLoopTest{});
 }
 
 void launch_b_finish(int nprob, const int64_t* pc_off, const double* part, const double* part2, int R,
                      const BScal& s, int mode, int flex, cudaStream_t st) {
-  k_b_finish<<<nprob, kFT, 0, st>>>(pc_off, part, part2, R, s, mode, flex);
+  k_b_finish<<<nprob, kFT, 0, st>>>(pc_off, part, part2, R, pow2_at_least(R), s, mode, flex);
 }
 
 void launch_b_scatter(const BChunks& ch, const BScatterArgs& a, cudaStream_t st) {

@@ -395,8 +395,11 @@ void launch_b_spmm_csc(const BChunks& ch, const CscDev& At, const double* Q, dou
                        double* part, cudaStream_t st);
 void launch_b_update(const BChunks& ch, int R, const double* alpha, const double* P, const double* W, double* X,
                      double* Rv, double* Rold, double* part, cudaStream_t st);
+// The test of the device-side loop of the block path (see launch_p_update): stat = {active
+// pairs, breakdown, iterations}, err the device-timeout slot.
+struct BLoopTest { cudaGraphConditionalHandle handle; int limit; int* stat; const double* err; };
 void launch_b_pupdate(const BChunks& ch, int R, const double* beta, const double* Z, double* P, int init,
-                      cudaStream_t st);
+                      const BLoopTest* loop, cudaStream_t st);
 void launch_b_finish(int nprob, const int64_t* pc_off, const double* part, const double* part2, int R,
                      const BScal& s, int mode, int flex, cudaStream_t st);
 void launch_b_scatter(const BChunks& ch, const BScatterArgs& a, cudaStream_t st);
