@@ -458,14 +458,17 @@ ls_status solve_core(ls_handle* h, int mode, double rtol, ls_info* info) {
     CK(cudaMemcpyAsync(h->r.p, h->tv.p, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
     lsq::launch_dot(n, h->r.p, h->r.p, site(h, lsq::S_TMP, 3), st);
   }
-  const double gg = dev_sum(h);
-  launches += 1;
-  if (!std::isfinite(gg)) throw LsError(LS_ERR_NONFINITE, "right-hand side is not finite");
-  const double gn = std::sqrt(gg);
+  // (what does not need ||g|| is queued before the wait for it)
+  double* read = h->pin + lsq::S_NSLOT;
+  CK(cudaMemcpyAsync(read, h->scal.p + lsq::S_TMP, sizeof(double), cudaMemcpyDeviceToHost, st));
   lsq::launch_fill(n, 0.0, h->x.p, st);
-  launches += 1;
   CK(cudaMemsetAsync(h->ctr.p, 0, sizeof(int), st));
   CK(cudaMemsetAsync(h->scal.p, 0, sizeof(double) * lsq::S_NSLOT, st));
+  CK(cudaStreamSynchronize(st));
+  const double gg = *read;
+  launches += 2;
+  if (!std::isfinite(gg)) throw LsError(LS_ERR_NONFINITE, "right-hand side is not finite");
+  const double gn = std::sqrt(gg);
   if (gn == 0.0) {
     CK(cudaStreamSynchronize(st));
     inf.t_solve = now_s() - t0;
@@ -484,7 +487,7 @@ ls_status solve_core(ls_handle* h, int mode, double rtol, ls_info* info) {
   const int fixed = h->opt.fixed_iters;
   const int maxit = fixed > 0 ? fixed : h->opt.maxit;
   const bool timed = h->opt.time_kernels != 0;
-  bool converged = false;
+  bool converged = false, have_hist = false;
   int it = 0, restarts = 0;
   double rr = gg;
   bool graph_this = h->opt.use_graph != 0;
@@ -578,7 +581,17 @@ ls_status solve_core(ls_handle* h, int mode, double rtol, ls_info* info) {
       throw LsError(LS_ERR_NONFINITE, "CG breakdown: non-finite or non-positive p.Cp at iteration " + std::to_string(it));
     if (fixed > 0) continue;
     if (rr <= thr2) {
-      const double tt = true_residual(h, mode, &launches);
+      // the true residual, and with it the coefficients for kappa, behind one wait
+      Phase phase("true residual");
+      launch_true_residual(h, mode, &launches);
+      CK(cudaMemcpyAsync(read, h->scal.p + lsq::S_TMP, sizeof(double), cudaMemcpyDeviceToHost, st));
+      have_hist = restarts == 0 && it <= h->pin_hist;
+      if (have_hist) {
+        CK(cudaMemcpyAsync(read + 1, h->ahist.p, sizeof(double) * it, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(read + 1 + h->pin_hist, h->bhist.p, sizeof(double) * it, cudaMemcpyDeviceToHost, st));
+      }
+      CK(cudaStreamSynchronize(st));
+      const double tt = *read;
       inf.relres_true = std::sqrt(tt) / gn;
       if (std::sqrt(tt) <= rtol * gn) { converged = true; break; }
       CK(cudaMemcpyAsync(h->r.p, h->w.p, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
@@ -595,9 +608,14 @@ ls_status solve_core(ls_handle* h, int mode, double rtol, ls_info* info) {
   const int nh = std::min(it, h->hist_cap);
   if (restarts == 0 && nh > 0) {
     std::vector<double> al(nh), be(nh);
-    CK(cudaMemcpyAsync(al.data(), h->ahist.p, sizeof(double) * nh, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(be.data(), h->bhist.p, sizeof(double) * nh, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
+    if (converged && have_hist) {
+      std::copy(read + 1, read + 1 + nh, al.begin());
+      std::copy(read + 1 + h->pin_hist, read + 1 + h->pin_hist + nh, be.begin());
+    } else {
+      CK(cudaMemcpyAsync(al.data(), h->ahist.p, sizeof(double) * nh, cudaMemcpyDeviceToHost, st));
+      CK(cudaMemcpyAsync(be.data(), h->bhist.p, sizeof(double) * nh, cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+    }
     std::vector<double> d(nh), e(std::max(nh - 1, 0));
     for (int j = 0; j < nh; ++j) {
       d[j] = 1.0 / al[j] + (j > 0 ? be[j - 1] / al[j - 1] : 0.0);
@@ -1634,9 +1652,11 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   h->hist_cap = std::max(h->opt.maxit, h->opt.fixed_iters) + 8;
   h->ahist.alloc(h->hist_cap); h->bhist.alloc(h->hist_cap);
   h->ctr.alloc(1);
-  // the scalar slots, and what a solver reads per step: a value, LSQR's report and residual,
-  // GMRES's coefficients
-  const size_t pins = lsq::S_NSLOT + (h->opt.solver == 2 ? 2 * (size_t)(h->opt.restart + 1) + 2 : lsq::L_NREP + 1);
+  // the scalar slots, and what a solver reads: a value and PCG's first coefficients, LSQR's
+  // report and residual, GMRES's coefficients
+  h->pin_hist = std::min(h->hist_cap, 512);
+  const size_t pins = lsq::S_NSLOT + std::max<size_t>(h->opt.solver == 2 ? 2 * (size_t)(h->opt.restart + 1) + 2 : lsq::L_NREP + 1,
+                                                      1 + 2 * (size_t)h->pin_hist);
   CK(cudaHostAlloc((void**)&h->pin, sizeof(double) * pins, cudaHostAllocDefault));
   if (h->opt.time_kernels)
     for (auto& e : h->ev) CK(cudaEventCreate(&e));

@@ -329,8 +329,8 @@ int iteration_launches(const ls_handle* h) { return 7 + precond_launches(h); }
 
 // Builds B.gexec as while (loop test) { one iteration }, then the status to the host, so that
 // the host waits once per pass of the loop (a wait and two copies per iteration before: 8
-// right-hand sides, 65 thousand columns, 18 iterations: 7.18 ms a solve,
-// 6.80 so).  False if the graph is refused.
+// right-hand sides, 65 thousand columns, 18 iterations: 7.18 ms a solve, 6.80 so).  False if
+// the graph is refused.
 bool build_block_loop(ls_handle* h, int R, bool flex, int limit) {
   BlockState& B = h->blk;
   cudaStream_t st = h->st;

@@ -235,7 +235,7 @@ struct ls_handle {
   DevBuf<unsigned> counters;  // ticket counters of the fused reductions
   DevBuf<int> ctr;
   double* pin = nullptr;  // pinned copy of the scalar slots, then the values a solver reads per step
-  int hist_cap = 0;
+  int hist_cap = 0, pin_hist = 0;
 
   cudaGraphExec_t gexec = nullptr;
   cudaGraphExec_t lq_exec = nullptr;  // one LSQR step
