@@ -950,7 +950,7 @@ ls_status gmres_core(ls_handle* h, double rtol, ls_info* info) {
 
 // A work vector of the handle, allocated by the first call that needs it: allocating and
 // freeing the six of an adjoint solve and the one of a value update on each call cost
-// 0.7 ms of a training step of 9.4 ms (103 thousand columns).
+// 0.7 ms of a training step of 9.4 ms (102 thousand columns).
 void reserve(DevBuf<double>& b, int64_t count) {
   if ((int64_t)b.n < count) b.alloc(count);
 }
@@ -1338,7 +1338,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   idiag.alloc((size_t)h->total_blocks * 32);
   if (h->coarse) {
     // The two factorisations, each a chain of small launches, run beside one another; the
-    // solve's stream waits for both before anything else.  (16 subdomains of 1,450 columns:
+    // solve's stream waits for both before anything else.  (16 subdomains of 1,900 columns:
     // 9.3 ms one after the other, about 6 so)
     Bidiag.alloc((size_t)h->total_blocks * 32);
     Bdinv.alloc((size_t)h->total_blocks * 1024);

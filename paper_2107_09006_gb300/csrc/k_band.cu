@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kThreads) k_assemble(BandPlan P, CsrDev A, Csc
 }
 
 // One CTA per block row (blockIdx.y) of a subdomain (blockIdx.x): the row's part of the two sums,
-// added per subdomain in row order by k_norms_sum.  (16 subdomains of 1,450 columns: one CTA
+// added per subdomain in row order by k_norms_sum.  (16 subdomains of 1,900 columns: one CTA
 // per subdomain took 1.42 ms, 0.10 so; the same split of k_prep 1.46 ms, 0.07.)
 __global__ void __launch_bounds__(kThreads) k_norms(BandPlan P, const double* __restrict__ C,
                                                     const double* __restrict__ Ct, double* __restrict__ parts) {

@@ -22,7 +22,7 @@ __device__ __forceinline__ unsigned seg_mask(int V) {
 // Block sums of one or two values in thread 0: the warps' sums meet in shared memory and eight
 // lanes add them (a sub-partition issues one FP64 warp instruction per 64 cycles, so the sum
 // of block_sum, formed by every warp, costs more than everything else in a small kernel: the
-// vector update of 17 thousand columns takes 5.7 us, 6.6 with block_sum; 103 thousand 8.2 and 10.3).
+// vector update of 37 thousand columns takes 5.7 us, 6.6 with block_sum; 102 thousand 8.2 and 10.3).
 __device__ __forceinline__ void block_sums(double& s1, double& s2, bool two, double* red) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   s1 = warp_sum(s1);
@@ -194,28 +194,57 @@ __global__ void __launch_bounds__(kThreads) k_spmv_sell(SellDev S, const double*
   if (ds.parts) finish_dots(dacc, 0.0, false, ds);
 }
 
-// alpha = rz / pw; x += alpha p; r_old = r; r -= alpha w; rr = r.r
+// alpha = rz / pw; x += alpha p; r_old = r; r -= alpha w; rr = r.r.  One thread of a block
+// divides (a division in every thread is FP64 issue of the same order as the update) while
+// the others' loads, four entries each, are in flight; the same in k_p_update (102 thousand
+// columns: 8.1 -> 6.9 and 5.5 -> 4.1 us; a million: 21.8 -> 20.2 and 9.9 -> 6.9).
+constexpr int kVecUnroll = 4;
 __global__ void __launch_bounds__(kThreads) k_cg_update(int64_t n, double* scal, const double* __restrict__ p,
                                                         const double* __restrict__ w, double* __restrict__ x,
                                                         double* __restrict__ r, double* __restrict__ r_old,
                                                         DotSite rr, int* ctr, double* alpha_hist, int cap) {
-  const double rz = scal[S_RZ], pw = scal[S_PW];
-  const double alpha = rz / pw;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    scal[S_RZOLD] = rz;
-    scal[S_ALPHA] = alpha;
-    const int it = *ctr;
-    if (it >= 0 && it < cap) alpha_hist[it] = alpha;
-    if (!(pw > 0.0) || !isfinite(alpha)) scal[S_FLAG] = 1.0;
+  __shared__ double sh;
+  if (threadIdx.x == 0) {
+    const double rz = scal[S_RZ], pw = scal[S_PW];
+    const double al = rz / pw;
+    sh = al;
+    if (blockIdx.x == 0) {
+      scal[S_RZOLD] = rz;
+      scal[S_ALPHA] = al;
+      const int it = *ctr;
+      if (it >= 0 && it < cap) alpha_hist[it] = al;
+      if (!(pw > 0.0) || !isfinite(al)) scal[S_FLAG] = 1.0;
+    }
   }
-  double acc = 0.0;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    x[k] += alpha * p[k];
-    double rk = r[k];
-    if (r_old) r_old[k] = rk;
-    rk -= alpha * w[k];
-    r[k] = rk;
-    acc += rk * rk;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  double acc = 0.0, alpha = 0.0;
+  bool first = true;
+  for (int64_t k0 = (int64_t)blockIdx.x * blockDim.x; k0 < n; k0 += kVecUnroll * step) {
+    double pk[kVecUnroll], wk[kVecUnroll], xk[kVecUnroll], rk[kVecUnroll];
+#pragma unroll
+    for (int u = 0; u < kVecUnroll; ++u) {
+      const int64_t k = k0 + u * step + threadIdx.x;
+      const bool in = k < n;
+      pk[u] = in ? p[k] : 0.0;
+      wk[u] = in ? w[k] : 0.0;
+      xk[u] = in ? x[k] : 0.0;
+      rk[u] = in ? r[k] : 0.0;
+    }
+    if (first) {  // (the whole block)
+      __syncthreads();
+      alpha = sh;
+      first = false;
+    }
+#pragma unroll
+    for (int u = 0; u < kVecUnroll; ++u) {
+      const int64_t k = k0 + u * step + threadIdx.x;
+      if (k >= n) continue;
+      x[k] = xk[u] + alpha * pk[u];
+      if (r_old) r_old[k] = rk[u];
+      const double rn = rk[u] - alpha * wk[u];
+      r[k] = rn;
+      acc += rn * rn;
+    }
   }
   finish_dots(acc, 0.0, false, rr);
 }
@@ -224,11 +253,12 @@ __global__ void __launch_bounds__(kThreads) k_cg_update(int64_t n, double* scal,
 __global__ void __launch_bounds__(kThreads) k_p_update(int64_t n, double* scal, int* ctr, double* beta_hist,
                                                        int cap, const double* __restrict__ z, double* __restrict__ p,
                                                        int init, int flex, LoopTest loop) {
-  double beta = 0.0;
-  if (!init) {
+  __shared__ double sh;
+  if (!init && threadIdx.x == 0) {
     const double num = flex ? scal[S_RZ] - scal[S_RZO] : scal[S_RZ];
-    beta = num / scal[S_RZOLD];
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const double beta = num / scal[S_RZOLD];
+    sh = beta;
+    if (blockIdx.x == 0) {
       scal[S_BETA] = beta;
       const int it = *ctr;
       if (it >= 0 && it < cap) beta_hist[it] = beta;
@@ -243,8 +273,28 @@ __global__ void __launch_bounds__(kThreads) k_p_update(int64_t n, double* scal, 
       }
     }
   }
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    p[k] = init ? z[k] : z[k] + beta * p[k];
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  double beta = 0.0;
+  bool first = !init;
+  for (int64_t k0 = (int64_t)blockIdx.x * blockDim.x; k0 < n; k0 += kVecUnroll * step) {
+    double zk[kVecUnroll], pk[kVecUnroll];
+#pragma unroll
+    for (int u = 0; u < kVecUnroll; ++u) {
+      const int64_t k = k0 + u * step + threadIdx.x;
+      zk[u] = k < n ? z[k] : 0.0;
+      pk[u] = k < n && !init ? p[k] : 0.0;
+    }
+    if (first) {  // (the whole block)
+      __syncthreads();
+      beta = sh;
+      first = false;
+    }
+#pragma unroll
+    for (int u = 0; u < kVecUnroll; ++u) {
+      const int64_t k = k0 + u * step + threadIdx.x;
+      if (k < n) p[k] = init ? zk[u] : zk[u] + beta * pk[u];
+    }
+  }
 }
 
 __global__ void k_stamp(unsigned long long* stamps, const int* ctr, int cap, int k, int after) {
@@ -312,7 +362,7 @@ __global__ void __launch_bounds__(kThreads) k_scatter(ScatterArgs a) {
       const double* Zi = a.Z + a.zoff[i] + a.jj_of[j];
       int t = 0;
       // Four basis entries loaded ahead of their products: one chain of dependent loads per
-      // entry bound the launch (17k columns, basis of 464: 12.7 us, 17.0 one at a time; 103k
+      // entry bound the launch (37k columns, basis of 464: 12.7 us, 17.0 one at a time; 102k
       // columns: 15.1 against 21.4; a million columns: 67.6 against 77).
       for (; t + 3 < k; t += 4) {
         double v[4], y[4];

@@ -348,9 +348,9 @@ __global__ void __launch_bounds__(kThreads) k_lanczos(EigArgs a, int use_smem) {
 // bound by its two FP64 FMAs per cycle (2 ms a step, 226 ms in all).  Here every stage of a
 // step is a kernel over all subdomains: the triangular solves on the clusters of the
 // superblock kernel, the product with D C~ D as two sparse products with the subdomain's
-// part of A (264 multiplications per interior column instead of the 1,088 entries its row of
-// the band holds), the re-orthogonalisation on a cluster of eight CTAs per subdomain.  The
-// recurrences, tolerances, restarts and start vectors are those of k_lanczos.
+// part of A (about 90 multiplications per interior column instead of the 1,088 entries its
+// row of the band holds), the re-orthogonalisation on a cluster of eight CTAs per subdomain.
+// The recurrences, tolerances, restarts and start vectors are those of k_lanczos.
 
 // Phases of a subdomain: 0 expanding, 1 expansion complete (Rayleigh-Ritz next), 2 done, 3
 // restarting (its kept vectors are rotated, the residual direction is to be appended).
