@@ -403,7 +403,8 @@ def run_ours(args):
         ms_local = sum(i["ms_local"] for i in tinfos) / max(nl, 1)
         its = sum(i["iters"] for i in tinfos)
         ms_spmv = sum(i["ms_spmv"] for i in tinfos) / max(its, 1)
-        lb = local_solve_bytes(st, form, restrict=variant == 0)
+        # (configuration 4, the superblocks, restricts in a kernel of its own on a second stream)
+        lb = local_solve_bytes(st, form, restrict=variant == 0 and tinfos[-1]["local_config"] != 4)
         tiles = St.normal_tiles()
         sb = tile_bytes(P.n, tiles) if tinfos[-1]["normal_product"] == 2 else spmv_bytes(P.m, P.n, P.nnz)
         loc_gbs = lb / (ms_local * 1e-3) / 1e9
@@ -440,7 +441,9 @@ def run_ours(args):
                      "traffic": LOCAL_SOLVE_TRAFFIC.get((P.name, args.prec, head["local_solve"]["config"])),
                      "traffic_source": TRAFFIC_SOURCE if (P.name, args.prec, head["local_solve"]["config"]) in
                      LOCAL_SOLVE_TRAFFIC else None,
-                     "kernel": "k_local_solve (batched envelope trisolves, one CTA per subdomain)",
+                     "kernel": "k_local_super (local solves over superblocks of 128 rows)"
+                     if head["local_solve"]["config"] == 4 else
+                     "k_local_solve (batched envelope trisolves, one CTA per subdomain)",
                      "bytes_per_launch": head["local_solve"]["bytes_per_launch"],
                      "ms_per_launch": head["local_solve"]["ms_per_launch"], "peak_source": peak_src},
         "gpu_launches": launches, "clocks": clocks, "e2e": e2e,
