@@ -639,8 +639,8 @@ __device__ __forceinline__ void lz_wait() {
 __device__ void ritz_vectors(double* St, int K, int np, RotMsg* msg) {
   for (int e = threadIdx.x; e < np * np; e += kThreads) St[(e / np) * K + e % np] = e / np == e % np ? 1.0 : 0.0;
   for (int turn = 0;; ++turn) {
-    lz_arrive();  // the last round's update is done
-    lz_wait();    // this round's rotations have come
+    lz_arrive();  // the last rotations are applied
+    lz_wait();    // the next rotations have come
     const RotMsg& m = msg[turn & 1];
     if (m.n < 0) return;
     for (int e = threadIdx.x; e < m.n * np; e += kThreads) {
@@ -712,7 +712,7 @@ __device__ void ritz_matrix(double* H, int K, int n, int np, RotMsg* msg, double
       __syncthreads();
       const int na = count[0], rest = half - na;
       if (threadIdx.x == 0) lz_put(lz_remote(&out.n, 1), na);
-      lz_arrive();  // the rotations have gone (and the last round's are read: the wait below)
+      lz_arrive();  // the rotations have gone (and the last ones are read: the wait below)
       const int mixed = na * rest, items = mixed + na * (na - 1) / 2;
       for (int e = threadIdx.x; e < items; e += kThreads) {
         int k, l;  // two different pairs, k < l, the first of them rotated
