@@ -1942,6 +1942,18 @@ ls_status ls_update_values(ls_handle* h, const double* val) {
 
 void ls_free(ls_handle* h) { delete h; }
 
+#ifdef LS_DEBUG_BOUNDS
+// Device-memory ceiling for tests (see AllocHook); *seen and *peak: the allocations and the
+// largest sum of the library's buffers since the last call.
+void ls_debug_alloc(int64_t fail_at, int64_t capacity, int64_t* seen, int64_t* peak) {
+  AllocHook& a = g_alloc_hook;
+  *seen = a.seen.exchange(0);
+  *peak = a.peak.exchange(a.used.load());
+  a.fail_at = fail_at;
+  a.capacity = capacity;
+}
+#endif
+
 ls_status ls_handle_info(const ls_handle* h, ls_info* info) {
   if (!h || !info) return LS_ERR_INVALID;
   *info = h->sinfo;

@@ -121,6 +121,34 @@ void swizzle_prepare(ls_handle* h) {
   check_launch("swizzled factor copy");
 }
 
+// The superblock storage of the block local solve, from the solve storage: built aside and
+// moved into the handle when it is complete.
+void pack_block_super(ls_handle* h) {
+  BlockState& B = h->blk;
+  cudaStream_t st = h->st;
+  std::vector<int64_t> boff((size_t)h->N + 1);
+  std::vector<int32_t> tf((size_t)h->total_blocks);
+  CK(cudaMemcpyAsync(boff.data(), h->blk_off.p, sizeof(int64_t) * boff.size(), cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(tf.data(), h->blk_tf.p, sizeof(int32_t) * tf.size(), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  const SuperHost sh = super_storage(boff, tf, h->N, h->prec);
+  DevBuf<int32_t> mtf, morder;
+  DevBuf<int64_t> mtoff;
+  DevBuf<unsigned char> mfac;
+  mtf.upload(sh.tf, st); mtoff.upload(sh.off, st); morder.upload(sh.order, st);
+  const int64_t back = h->prec == LS_PREC_F32 ? sh.bytes : 0;
+  mfac.alloc((size_t)(sh.bytes + back));
+  lsq::launch_super_pack_solve(h->prec, h->N, h->max_nb, h->blk_off.p, h->blk_tf.p, h->blk_poff.p, mtf.p, mtoff.p,
+                               h->prec == LS_PREC_F64 ? (const void*)h->L64.p
+                               : h->prec == LS_PREC_F32 ? (const void*)h->L32.p : (const void*)h->L16.p,
+                               h->prec == LS_PREC_BF16 ? h->tsc.p : nullptr, back, mfac.p, st);
+  CK(cudaStreamSynchronize(st));
+  check_launch("superblock storage of the block path");
+  B.m_tf.take(mtf); B.m_toff.take(mtoff); B.m_order.take(morder);
+  B.m_back = back;
+  B.m_fac.take(mfac);
+}
+
 // Whether the block local solve of R right-hand sides runs over superblocks (by rule), its
 // storage made from the solve storage at the first use.  With a forced block_kernel or the
 // stalled test hook it does not.  FP32 factors (eight right-hand sides per CTA): not where
@@ -129,40 +157,30 @@ void swizzle_prepare(ls_handle* h) {
 // against 438 for the tcgen05 kernel; R = 8: 163 against 432; N = 256, R = 8: 284 against
 // 774), and on a batched handle from four right-hand sides on: below, the automatic choice is
 // pinned by a test to one of the two tensor-core kernels (64 subdomains and R = 2: 430 us,
-// the superblocks 164).
+// the superblocks 164).  The plan counts only when all of it has
+// succeeded: after an error the next call plans anew.
 void plan_block_super(ls_handle* h, int R) {
   BlockState& B = h->blk;
   if (B.m_R == R) return;
-  B.m_R = R;
+  B.m_R = 0;
   B.m_ok = false;
-  if (h->opt.block_kernel != 0 || h->opt.test_stall) return;
-  if (h->prec == LS_PREC_F32 && h->nprob > 1 && R < 4) return;
-  int optin = 0, sms = 0;
-  CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
-  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev));
-  h->sb_optin = optin;
+  B.gR = 0;  // (a graph of the last plan is not replayed)
+  lsq::SuperShape shape{};
   const int64_t groups = (R + 7) / 8;
-  if (h->prec == LS_PREC_F32 && groups > 2 && groups * h->N > 3 * (int64_t)sms) return;
-  B.m_ok = lsq::local_super_plan_multi(h->prec, R, h->N, h->max_nb, std::max(h->wmax, lsq::kSuperRows), sms,
-                                       (size_t)optin, B.m_shape);
-  if (!B.m_ok || B.m_fac.p) return;
-  cudaStream_t st = h->st;
-  std::vector<int64_t> boff((size_t)h->N + 1);
-  std::vector<int32_t> tf((size_t)h->total_blocks);
-  CK(cudaMemcpyAsync(boff.data(), h->blk_off.p, sizeof(int64_t) * boff.size(), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(tf.data(), h->blk_tf.p, sizeof(int32_t) * tf.size(), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  const SuperHost sh = super_storage(boff, tf, h->N, h->prec);
-  B.m_tf.upload(sh.tf, st); B.m_toff.upload(sh.off, st); B.m_order.upload(sh.order, st);
-  B.m_back = h->prec == LS_PREC_F32 ? sh.bytes : 0;
-  B.m_fac.alloc((size_t)(sh.bytes + B.m_back));
-  lsq::launch_super_pack_solve(h->prec, h->N, h->max_nb, h->blk_off.p, h->blk_tf.p, h->blk_poff.p, B.m_tf.p,
-                               B.m_toff.p,
-                               h->prec == LS_PREC_F64 ? (const void*)h->L64.p
-                               : h->prec == LS_PREC_F32 ? (const void*)h->L32.p : (const void*)h->L16.p,
-                               h->prec == LS_PREC_BF16 ? h->tsc.p : nullptr, B.m_back, B.m_fac.p, st);
-  CK(cudaStreamSynchronize(st));
-  check_launch("superblock storage of the block path");
+  bool ok = h->opt.block_kernel == 0 && !h->opt.test_stall && !(h->prec == LS_PREC_F32 && h->nprob > 1 && R < 4);
+  if (ok) {
+    int optin = 0, sms = 0;
+    CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev));
+    h->sb_optin = optin;
+    ok = !(h->prec == LS_PREC_F32 && groups > 2 && groups * h->N > 3 * (int64_t)sms) &&
+         lsq::local_super_plan_multi(h->prec, R, h->N, h->max_nb, std::max(h->wmax, lsq::kSuperRows), sms,
+                                     (size_t)optin, shape);
+  }
+  if (ok && !B.m_fac.p) pack_block_super(h);
+  B.m_shape = shape;
+  B.m_ok = ok;
+  B.m_R = R;
 }
 
 void launch_block_super(ls_handle* h, int R, const double* Rin) {

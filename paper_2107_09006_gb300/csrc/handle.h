@@ -6,9 +6,13 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#ifdef LS_DEBUG_BOUNDS
+#include <atomic>
+#endif
 #include <chrono>
 #include <stdexcept>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/ls_schwarz.h"
@@ -29,6 +33,29 @@ struct LsError : std::runtime_error {
                     std::string(#call) + ": " + cudaGetErrorString(e_));                      \
   } while (0)
 
+// Device-memory ceiling of the bounds-checked build's tests (ls_debug_alloc): refuses the
+// fail_at-th allocation from then on (0: none) and what would take the library's buffers
+// above `capacity` bytes (0: no ceiling).  The product build has none of it.
+#ifdef LS_DEBUG_BOUNDS
+struct AllocHook {
+  std::atomic<int64_t> fail_at{0}, seen{0}, capacity{0}, used{0}, peak{0};
+};
+inline AllocHook g_alloc_hook;
+inline bool alloc_refused(size_t bytes) {
+  AllocHook& a = g_alloc_hook;
+  if (++a.seen == a.fail_at) return true;
+  return a.capacity > 0 && a.used + (int64_t)bytes > a.capacity;
+}
+inline void alloc_count(size_t bytes, bool add) {
+  AllocHook& a = g_alloc_hook;
+  a.used += add ? (int64_t)bytes : -(int64_t)bytes;
+  if (a.used > a.peak) a.peak = a.used.load();
+}
+#else
+inline bool alloc_refused(size_t) { return false; }
+inline void alloc_count(size_t, bool) {}
+#endif
+
 template <class T>
 struct DevBuf {
   T* p = nullptr;
@@ -38,20 +65,31 @@ struct DevBuf {
   DevBuf& operator=(const DevBuf&) = delete;
   ~DevBuf() { release(); }
   void release() {
-    if (p) cudaFree(p);
+    if (p) {
+      cudaFree(p);
+      alloc_count(n * sizeof(T), false);
+    }
     p = nullptr;
     n = 0;
   }
   void alloc(size_t count) {
     release();
     if (count == 0) count = 1;
-    cudaError_t e = cudaMalloc(&p, count * sizeof(T));
+    cudaError_t e = alloc_refused(count * sizeof(T)) ? cudaErrorMemoryAllocation : cudaMalloc(&p, count * sizeof(T));
     if (e != cudaSuccess) {
       p = nullptr;
       cudaGetLastError();
       throw LsError(LS_ERR_OOM, "cudaMalloc of " + std::to_string(count * sizeof(T)) + " bytes failed");
     }
     n = count;
+    alloc_count(n * sizeof(T), true);
+  }
+  // The storage of o, which is left empty: what is built in parts is built in locals and moved
+  // into the handle when all of it is there.
+  void take(DevBuf& o) {
+    release();
+    std::swap(p, o.p);
+    std::swap(n, o.n);
   }
   void zero(cudaStream_t st) { CK(cudaMemsetAsync(p, 0, n * sizeof(T), st)); }
   void upload(const std::vector<T>& v, cudaStream_t st) {

@@ -1,0 +1,112 @@
+"""Calls that meet a device out-of-memory error, and the calls after them.
+
+The bounds-checked build refuses a chosen allocation of the library on the host
+(ls_debug_alloc).  A child process that loads it refuses, one after the other, every
+allocation that a call makes.  The call must succeed or return LS_ERR_OOM, and the same call
+on the same handle, with nothing refused, must then give the answer: nothing that the failed
+call left half built may be used.  Nothing here makes the GPU itself run out of memory.
+"""
+import os
+import subprocess
+import sys
+
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - CPU containers
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+CHILD = r'''
+import ctypes, sys
+import numpy as np
+sys.path.insert(0, ROOT)
+import torch
+import paper_2107_09006_gb300 as L
+from workloads import make_grid_ls, block_partition
+assert L.LIBRARY_PATH.endswith("libls_schwarz_dbg.so"), L.LIBRARY_PATH
+hook = ctypes.CDLL(L.LIBRARY_PATH).ls_debug_alloc
+hook.restype = None
+hook.argtypes = [ctypes.c_int64, ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p]
+
+def refuse(fail_at=0, capacity=0):
+    """(allocations, peak bytes) since the last call; then refuse as given."""
+    seen, peak = ctypes.c_int64(), ctypes.c_int64()
+    hook(fail_at, capacity, ctypes.byref(seen), ctypes.byref(peak))
+    return seen.value, peak.value
+
+W, H = 40, 36
+m, n, rp, c, v, b, _ = make_grid_ls(W, H, 3, 6, 2, 5, nrhs=12)
+part = block_partition(W, H, 12, 14)
+N = int(part.max()) + 1
+b = np.asarray(b)
+
+def make(**opt):
+    return L.Solver(m, n, rp, c, v, part, N, nev_max=6, spmv=2, **opt)
+
+def solve(S, R):
+    return S.solve(b[:R], rtol=1e-9)[0].cpu().numpy()
+
+ref = None
+
+def check(x, R):
+    global ref
+    if ref is None:
+        S = make()
+        ref = np.stack([S.solve(b[k], rtol=1e-11)[0].cpu().numpy() for k in range(12)])
+        S.close()
+    assert np.isfinite(x).all()
+    # residuals of 1e-9 and 1e-11 of ||A^T b||; ||A^T b|| / (lambda_min(C) ||x||) <= 14 here
+    assert np.linalg.norm(x - ref[:R]) <= 1e-7 * np.linalg.norm(ref[:R])
+
+def refused_one_by_one(opt, R, before=(), after=None):
+    """Every allocation of solve(R) refused in turn, each on a fresh handle (`before`: widths
+    solved first; `after`: the width solved after the failed call, default R)."""
+    k, failed = 1, 0
+    while True:
+        S = make(**opt)
+        for w in before:
+            check(solve(S, w), w)
+        refuse(fail_at=k)
+        ok = True
+        try:
+            x = solve(S, R)
+        except L.LSError as e:
+            assert e.status == L.LS_ERR_OOM, e
+            ok = False
+            failed += 1
+        seen, _ = refuse()
+        if ok:
+            check(x, R)
+        for w in (after or R, R):
+            check(solve(S, w), w)
+        S.close()
+        if seen < k:
+            assert ok and k > 1
+            return failed
+        k += 1
+
+'''
+
+
+def _child(body):
+    import importlib.util
+    spec = importlib.util.spec_from_file_location("_ls_build_a", os.path.join(ROOT, "paper_2107_09006_gb300",
+                                                                              "_build.py"))
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    mod.build(debug_bounds=True)
+    code = CHILD.replace("ROOT", repr(ROOT)) + body + "\nprint('child done')\n"
+    p = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True,
+                       env=dict(os.environ, LS_SCHWARZ_BOUNDS="1"), timeout=900)
+    assert p.returncode == 0 and "child done" in p.stdout, p.stderr[-3000:]
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "bf16"])
+def test_block_solve_after_out_of_memory(prec):
+    """The superblock storage of the block path is made by the first block solve: an error on
+    the way must not leave a plan that names storage which is not there."""
+    _child(f"assert refused_one_by_one(dict(factor_prec={prec!r}), 3) > 0")
