@@ -60,7 +60,8 @@ void ensure_buffers(ls_handle* h, int R) {
 }
 
 // The update tiles of every block step of the right-looking sweeps (tcgen05 kernel) and
-// the copies they are read from, built from the solve storage at the first use.
+// the copies they are read from, built from the solve storage at the first use: aside, and moved
+// into the handle when all are there.
 void umma_prepare(ls_handle* h) {
   BlockState& B = h->blk;
   if (B.Uf.p) return;
@@ -95,30 +96,37 @@ void umma_prepare(ls_handle* h) {
   }
   foff[NB] = (int64_t)frow.size();
   boff2[NB] = (int64_t)brow.size();
-  B.uf_off.upload(foff, st);
-  B.ub_off.upload(boff2, st);
-  B.uf_row.upload(frow, st);
-  B.ub_row.upload(brow, st);
-  DevBuf<int64_t> fs, bs;
+  DevBuf<int64_t> uf_off, ub_off, fs, bs;
+  DevBuf<int32_t> uf_row, ub_row;
+  DevBuf<float> Uf, Ub, Ud;
+  uf_off.upload(foff, st);
+  ub_off.upload(boff2, st);
+  uf_row.upload(frow, st);
+  ub_row.upload(brow, st);
   fs.upload(fsrc, st);
   bs.upload(bsrc, st);
-  B.Uf.alloc(std::max<size_t>(frow.size(), 1) * 1024);
-  B.Ub.alloc(std::max<size_t>(brow.size(), 1) * 1024);
-  B.Ud.alloc((size_t)NB * 2 * 32 * 36);
-  lsq::launch_bu_copy((int64_t)frow.size(), fs.p, h->L32.p, B.Uf.p, 0, st);
-  lsq::launch_bu_copy((int64_t)brow.size(), bs.p, h->L32.p, B.Ub.p, 1, st);
-  lsq::launch_bu_diag(NB, h->blk_poff.p, h->L32.p, B.Ud.p, st);
+  Uf.alloc(std::max<size_t>(frow.size(), 1) * 1024);
+  Ub.alloc(std::max<size_t>(brow.size(), 1) * 1024);
+  Ud.alloc((size_t)NB * 2 * 32 * 36);
+  lsq::launch_bu_copy((int64_t)frow.size(), fs.p, h->L32.p, Uf.p, 0, st);
+  lsq::launch_bu_copy((int64_t)brow.size(), bs.p, h->L32.p, Ub.p, 1, st);
+  lsq::launch_bu_diag(NB, h->blk_poff.p, h->L32.p, Ud.p, st);
   CK(cudaStreamSynchronize(st));
   check_launch("tcgen05 factor copies");
+  B.uf_off.take(uf_off); B.ub_off.take(ub_off); B.uf_row.take(uf_row); B.ub_row.take(ub_row);
+  B.Ub.take(Ub); B.Ud.take(Ud);
+  B.Uf.take(Uf);
 }
 
 void swizzle_prepare(ls_handle* h) {
   BlockState& B = h->blk;
   if (B.Lsw.p) return;
-  B.Lsw.alloc(h->fac_elems);
-  lsq::launch_b_swizzle(h->fac_elems, h->L32.p, B.Lsw.p, h->st);
+  DevBuf<float> Lsw;
+  Lsw.alloc(h->fac_elems);
+  lsq::launch_b_swizzle(h->fac_elems, h->L32.p, Lsw.p, h->st);
   CK(cudaStreamSynchronize(h->st));
   check_launch("swizzled factor copy");
+  B.Lsw.take(Lsw);
 }
 
 // The superblock storage of the block local solve, from the solve storage: built aside and

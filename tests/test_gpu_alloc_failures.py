@@ -110,3 +110,11 @@ def test_block_solve_after_out_of_memory(prec):
     """The superblock storage of the block path is made by the first block solve: an error on
     the way must not leave a plan that names storage which is not there."""
     _child(f"assert refused_one_by_one(dict(factor_prec={prec!r}), 3) > 0")
+
+
+@pytest.mark.parametrize("opt", ["dict(factor_prec='f32', block_kernel=1)", "dict(factor_prec='f32', block_kernel=2)",
+                                 "dict(factor_prec='f64', block_kernel=1)"])
+def test_block_kernel_copies_after_out_of_memory(opt):
+    """The factor copies of the two tensor-core kernels (and the CUDA-core kernel, which
+    makes none)."""
+    _child(f"assert refused_one_by_one({opt}, 3) > 0")
