@@ -49,6 +49,7 @@ void ensure_buffers(ls_handle* h, int R) {
     cudaGraphExecDestroy(B.gexec);
     B.gexec = nullptr;
   }
+  B.R = 0;  // (until all of them are there: the narrower ones go first)
   const size_t n = (size_t)h->n * R, m = (size_t)h->m * R;
   B.X.alloc(n); B.Rv.alloc(n); B.Rold.alloc(n); B.Z.alloc(n); B.P.alloc(n); B.W.alloc(n);
   B.Q.alloc(m); B.B.alloc(m); B.Bu.alloc(m);

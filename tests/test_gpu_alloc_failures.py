@@ -118,3 +118,10 @@ def test_block_kernel_copies_after_out_of_memory(opt):
     """The factor copies of the two tensor-core kernels (and the CUDA-core kernel, which
     makes none)."""
     _child(f"assert refused_one_by_one({opt}, 3) > 0")
+
+
+@pytest.mark.parametrize("opt", ["dict(factor_prec='f64')", "dict(factor_prec='f32', block_kernel=1)"])
+def test_narrow_block_solve_after_a_wider_one_ran_out_of_memory(opt):
+    """A wider block solve replaces the work vectors of a narrower one; after an error on the
+    way the narrower solve must not use those that went."""
+    _child(f"assert refused_one_by_one({opt}, 5, before=(2,), after=2) > 0")
