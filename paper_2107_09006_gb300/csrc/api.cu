@@ -1336,6 +1336,10 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   DevBuf<int> status, Bstatus;
   status.alloc(N);
   idiag.alloc((size_t)h->total_blocks * 32);
+  std::vector<int32_t> corder;
+  const std::vector<lsq::CholGroup> chol = lsq::chol_groups(N, hs.blk_off.data(), hs.blk_tf.data(), corder);
+  DevBuf<int32_t> chol_order;
+  chol_order.upload(corder, st);
   if (h->coarse) {
     // The two factorisations, each a chain of small launches, run beside one another; the
     // solve's stream waits for both before anything else.  (16 subdomains of 1,900 columns:
@@ -1345,10 +1349,10 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     Bstatus.alloc(N);
     CK(cudaEventRecord(h->ev_fork, st));
     CK(cudaStreamWaitEvent(h->st2, h->ev_fork, 0));
-    lsq::launch_band_cholesky(plan, h->max_nb, h->wmax, Bst.p, Bidiag.p, Bdinv.p, Bstatus.p, h->st2);
+    lsq::launch_band_cholesky(plan, chol, chol_order.p, Bst.p, Bidiag.p, Bdinv.p, Bstatus.p, h->st2);
     CK(cudaEventRecord(h->ev_coarse, h->st2));
   }
-  lsq::launch_band_cholesky(plan, h->max_nb, h->wmax, Cst.p, idiag.p, dinv.p, status.p, st);
+  lsq::launch_band_cholesky(plan, chol, chol_order.p, Cst.p, idiag.p, dinv.p, status.p, st);
   if (h->coarse) CK(cudaStreamWaitEvent(st, h->ev_coarse, 0));
   std::vector<int> hst(N);
   CK(cudaMemcpyAsync(hst.data(), status.p, sizeof(int) * N, cudaMemcpyDeviceToHost, st));

@@ -152,10 +152,11 @@ __global__ void __launch_bounds__(kThreads) k_prep(BandPlan P, const double* __r
 // per cycle; one CTA per subdomain ran the whole factor on as many SMs as there were
 // subdomains (16 of 1,936 columns: 33 ms).
 __global__ void __launch_bounds__(kThreads) k_chol_diag(BandPlan P, double* __restrict__ F, double* __restrict__ idiag,
-                                                        double* __restrict__ dinv, int* __restrict__ status, int k) {
+                                                        double* __restrict__ dinv, int* __restrict__ status,
+                                                        const int32_t* __restrict__ order, int k) {
   __shared__ double S[kT * 33], Q[kT * 33];
   __shared__ int fail;
-  const int i = blockIdx.x;
+  const int i = order[blockIdx.x];
   const int64_t b0 = P.blk_off[i];
   if (k >= (int)(P.blk_off[i + 1] - b0)) return;
   const int t0 = P.blk_tf[b0 + k];
@@ -173,9 +174,10 @@ __global__ void __launch_bounds__(kThreads) k_chol_diag(BandPlan P, double* __re
 
 // L(b, k) = A(b, k) L(k, k)^{-T} for the block rows b > k that reach column k.
 __global__ void __launch_bounds__(kThreads) k_chol_col(BandPlan P, double* __restrict__ F,
-                                                       const double* __restrict__ dinv, int k) {
+                                                       const double* __restrict__ dinv,
+                                                       const int32_t* __restrict__ order, int k) {
   __shared__ double S[kT * 33], A[kT * 33], Q[kT * 33];
-  const int i = blockIdx.x, b = k + 1 + blockIdx.y;
+  const int i = order[blockIdx.x], b = k + 1 + blockIdx.y;
   const int64_t b0 = P.blk_off[i];
   if (b >= (int)(P.blk_off[i + 1] - b0)) return;
   const int t0 = P.blk_tf[b0 + b];
@@ -191,28 +193,34 @@ __global__ void __launch_bounds__(kThreads) k_chol_col(BandPlan P, double* __res
   store_tile(S, pan, width, (k - t0) * kT);
 }
 
-// A(b, c) -= L(b, k) L(c, k)^T for k < c <= b, both reaching column k (blockIdx.y enumerates
+// A(b, c) -= L(b, k) L(c, k)^T for k < c <= b, both reaching column k (the CTAs in y stride over
 // the pairs of the window below k).
-__global__ void __launch_bounds__(kThreads) k_chol_update(BandPlan P, double* __restrict__ F, int k) {
+__global__ void __launch_bounds__(kThreads) k_chol_update(BandPlan P, double* __restrict__ F,
+                                                          const int32_t* __restrict__ order, int k, int below) {
   __shared__ double S[kT * 33], A[kT * 33], Q[kT * 33];
-  int ii = (int)((sqrtf(8.f * (float)blockIdx.y + 1.f) - 1.f) * 0.5f);
-  while ((ii + 1) * (ii + 2) / 2 <= (int)blockIdx.y) ++ii;
-  while (ii * (ii + 1) / 2 > (int)blockIdx.y) --ii;
-  const int i = blockIdx.x, b = k + 1 + ii, c = k + 1 + (int)blockIdx.y - ii * (ii + 1) / 2;
+  const int i = order[blockIdx.x];
   const int64_t b0 = P.blk_off[i];
-  if (b >= (int)(P.blk_off[i + 1] - b0)) return;
-  const int tb = P.blk_tf[b0 + b], tc = P.blk_tf[b0 + c];
-  if (tb > k || tc > k) return;
-  const int wb = (b - tb + 1) * kT, wc = (c - tc + 1) * kT;
-  double* panb = F + P.blk_poff[b0 + b];
-  const double* panc = F + P.blk_poff[b0 + c];
-  load_tile(S, panb, wb, (c - tb) * kT);
-  load_tile(A, panb, wb, (k - tb) * kT);
-  load_tile(Q, panc, wc, (k - tc) * kT);
-  __syncthreads();
-  tile_mm<false, true>(S, A, Q, -1);
-  __syncthreads();
-  store_tile(S, panb, wb, (c - tb) * kT);
+  const int nb = (int)(P.blk_off[i + 1] - b0);
+  for (int64_t e = blockIdx.y; e < chol_pairs(below); e += gridDim.y) {
+    int b, c;
+    chol_pair(e, b, c);
+    b += k + 1;
+    c += k + 1;
+    if (b >= nb) return;
+    const int tb = P.blk_tf[b0 + b], tc = P.blk_tf[b0 + c];
+    if (tb > k || tc > k) continue;
+    const int wb = (b - tb + 1) * kT, wc = (c - tc + 1) * kT;
+    double* panb = F + P.blk_poff[b0 + b];
+    const double* panc = F + P.blk_poff[b0 + c];
+    load_tile(S, panb, wb, (c - tb) * kT);
+    load_tile(A, panb, wb, (k - tb) * kT);
+    load_tile(Q, panc, wc, (k - tc) * kT);
+    __syncthreads();
+    tile_mm<false, true>(S, A, Q, -1);
+    __syncthreads();
+    store_tile(S, panb, wb, (c - tb) * kT);
+    __syncthreads();
+  }
 }
 
 int grid_for(int64_t work, int cap) {
@@ -239,15 +247,18 @@ void launch_prep(const BandPlan& P, int max_nb, const double* dsub, const double
   k_prep<<<dim3(P.N, max_nb), kThreads, 0, st>>>(P, s, Cst, eqs, Ctst, Bst);
 }
 
-void launch_band_cholesky(const BandPlan& P, int max_nb, int wmax, double* F, double* idiag, double* dinv, int* status,
-                          cudaStream_t st) {
+void launch_band_cholesky(const BandPlan& P, const std::vector<CholGroup>& groups, const int32_t* order, double* F,
+                          double* idiag, double* dinv, int* status, cudaStream_t st) {
   cudaMemsetAsync(status, 0, sizeof(int) * P.N, st);
-  for (int k = 0; k < max_nb; ++k) {
-    k_chol_diag<<<P.N, kThreads, 0, st>>>(P, F, idiag, dinv, status, k);
-    const int below = wmax - 1 < max_nb - 1 - k ? wmax - 1 : max_nb - 1 - k;  // block rows that can reach column k
-    if (below > 0) {
-      k_chol_col<<<dim3(P.N, below), kThreads, 0, st>>>(P, F, dinv, k);
-      k_chol_update<<<dim3(P.N, below * (below + 1) / 2), kThreads, 0, st>>>(P, F, k);
+  for (const CholGroup& g : groups) {
+    const int32_t* ord = order + g.first;
+    for (int k = 0; k < g.max_nb; ++k) {
+      k_chol_diag<<<g.count, kThreads, 0, st>>>(P, F, idiag, dinv, status, ord, k);
+      const int below = std::min(g.below, g.max_nb - 1 - k);  // block rows that can reach column k
+      if (below > 0) {
+        k_chol_col<<<dim3(g.count, below), kThreads, 0, st>>>(P, F, dinv, ord, k);
+        k_chol_update<<<dim3(g.count, chol_grid_y(below)), kThreads, 0, st>>>(P, F, ord, k, below);
+      }
     }
   }
 }

@@ -4,6 +4,10 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <vector>
+
+#include "chol_window.h"
+
 namespace lsq {
 
 // ---- sparse products and CG vector kernels (k_krylov.cu) ----------------------------
@@ -169,9 +173,9 @@ void launch_prep(const BandPlan& P, int max_nb, const double* dsub, const double
 // In-place Cholesky of every subdomain's matrix; idiag = 1 / diag(L);
 // status[i] = 0 or 1 + the local row of the first nonpositive pivot.
 // dinv: scratch of 1024 doubles per block row (inverse diagonal tiles).
-// max_nb, wmax: most block rows of a subdomain and most tiles of a block row.
-void launch_band_cholesky(const BandPlan& P, int max_nb, int wmax, double* st_fac, double* idiag, double* dinv,
-                          int* status, cudaStream_t st);
+// groups, order (device): see chol_groups.
+void launch_band_cholesky(const BandPlan& P, const std::vector<CholGroup>& groups, const int32_t* order,
+                          double* st_fac, double* idiag, double* dinv, int* status, cudaStream_t st);
 
 // ---- batched local solves (k_local.cu) -----------------------------------------------
 struct LocalArgs {
