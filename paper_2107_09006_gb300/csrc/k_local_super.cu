@@ -1039,7 +1039,7 @@ __global__ void __launch_bounds__(kThreads) k_super_pack(const int64_t* __restri
   using TX = typename std::conditional<kBf16, float, TF>::type;
   __shared__ double X[kQ - 1][kT * 33], P[kT * 33], S[kT * 33];
   __shared__ double redm[kWarps];
-  const int i = blockIdx.y, s = blockIdx.x;
+  const int i = blockIdx.x, s = blockIdx.y;  // (more than 65,535 subdomains: in x)
   const int64_t g0 = blk_off[i];
   const int nb = (int)(blk_off[i + 1] - g0);
   const int b0 = s * kQ, b1 = min(nb, b0 + kQ);
@@ -1247,7 +1247,7 @@ bool launch_local_super(const SuperArgs& a, const SuperShape& f, int prec, int N
 void launch_super_pack(int prec, int N, int max_nb, const int64_t* blk_off, const int32_t* blk_tf,
                        const int64_t* blk_poff, const int32_t* stf, const int64_t* stoff, const double* L,
                        const double* dinv, unsigned char* dst, cudaStream_t st) {
-  const dim3 grid((unsigned)((max_nb + kQ - 1) / kQ), (unsigned)N);
+  const dim3 grid((unsigned)N, (unsigned)((max_nb + kQ - 1) / kQ));
   const BandSrc src{blk_tf, blk_poff, L, dinv};
   if (prec == 0) k_super_pack<double><<<grid, kThreads, 0, st>>>(blk_off, src, stf, stoff, 0, 0, dst);
   else if (prec == 1) k_super_pack<float><<<grid, kThreads, 0, st>>>(blk_off, src, stf, stoff, 0, 0, dst);
@@ -1257,7 +1257,7 @@ void launch_super_pack(int prec, int N, int max_nb, const int64_t* blk_off, cons
 void launch_super_pack_solve(int prec, int N, int max_nb, const int64_t* blk_off, const int32_t* blk_tf,
                              const int64_t* blk_poff, const int32_t* stf, const int64_t* stoff, const void* fac,
                              const float* tsc, int64_t frag, unsigned char* dst, cudaStream_t st) {
-  const dim3 grid((unsigned)((max_nb + kQ - 1) / kQ), (unsigned)N);
+  const dim3 grid((unsigned)N, (unsigned)((max_nb + kQ - 1) / kQ));
   if (prec == 0)
     k_super_pack<double><<<grid, kThreads, 0, st>>>(
         blk_off, SolveSrc<double>{blk_tf, blk_poff, (const double*)fac, nullptr}, stf, stoff, 0, 0, dst);

@@ -64,3 +64,26 @@ def test_wide_block_rows(tiles, narrow, prec, tol):
     zo = one_level(A, part, N, r, S.info()["delta"])
     assert np.linalg.norm(z - zo) <= tol * np.linalg.norm(zo)
     S.close()
+
+
+@pytest.mark.parametrize("prec,tol", [("f64", 1e-9), ("f32", 1e-5)])
+def test_more_subdomains_than_a_launch_dimension_holds(prec, tol):
+    """65,600 subdomains of two columns: the single-vector path over superblocks against the
+    32-row sweeps, which are forced, and two right-hand sides of the block path against it."""
+    N = 65600
+    A, part = chain(2 * N, 2 * np.arange(N + 1), [])
+    args = (A.shape[0], A.shape[1], A.indptr, A.indices, A.data, part, N)
+    rng = np.random.default_rng(1)
+    r = rng.standard_normal(A.shape[1])
+    z, x = {}, {}
+    b = rng.standard_normal((2, A.shape[0]))
+    for config in (0, 1):
+        S = L.Solver(*args, coarse=0, factor_prec=prec, local_config=config, spmv=2)
+        assert S.info()["local_config"] == (4 if config == 0 else 1)
+        z[config] = S.apply_preconditioner(r, 1).cpu().numpy()
+        x[config] = S.solve(b, rtol=1e-9)[0].cpu().numpy() if config == 0 else \
+            np.stack([S.solve(v, rtol=1e-9)[0].cpu().numpy() for v in b])
+        S.close()
+    assert np.linalg.norm(z[0] - z[1]) <= tol * np.linalg.norm(z[1])
+    # two solutions to residuals of 1e-9; C >= 4 I and ||A^T b|| <= sqrt(||C||) ||b||
+    assert np.linalg.norm(x[0] - x[1]) <= 1e-7 * np.linalg.norm(x[1])
