@@ -607,7 +607,7 @@ __global__ void __cluster_dims__(kOrthCluster, 1, 1) __launch_bounds__(kThreads)
 // instructions for its four entries and their mirror images; 32 by rows, then columns), and
 // pairs whose entry is so small that all such entries together pass the convergence test are
 // left alone (at first most of a Lanczos matrix, near the end most pairs): 1.8 ms so.
-constexpr int kMaxHalf = kMaxK / 2;
+constexpr int kMaxHalf = kMaxK / 2, kRitzWarps = (kMaxHalf + 31) / 32;
 struct RotMsg {  // the rotations of one round, from rank 0 to rank 1
   int n;         // -1: no more rounds
   int pq[kMaxHalf];
@@ -658,13 +658,12 @@ __device__ void ritz_vectors(double* St, int K, int np, RotMsg* msg) {
 // Rank 0: the rotations, H <- R^T H R (H np x np in a K x K buffer, upper triangle valid on
 // entry) until it is diagonal.
 __device__ void ritz_matrix(double* H, int K, int n, int np, RotMsg* msg, double* cs, double* sn, int* pp, int* qq,
-                            int (*cnt)[2], double* red) {
+                            int (*cnt)[kRitzWarps], double* red) {
   for (int e = threadIdx.x; e < np * np; e += kThreads) {
     const int r = e / np, c = e % np;
     if (r > c && r < n) H[r * K + c] = H[c * K + r];
     if (r >= n || c >= n) H[r * K + c] = 0.0;
   }
-  if (threadIdx.x < 2) cnt[0][threadIdx.x] = 0;
   __syncthreads();
   const int half = np / 2;
   int turn = 0;
@@ -682,35 +681,53 @@ __device__ void ritz_matrix(double* H, int K, int n, int np, RotMsg* msg, double
     for (int round = 0; round < np - 1; ++round, ++turn) {
       RotMsg& out = msg[turn & 1];
       int* count = cnt[turn & 1];
-      if (threadIdx.x >= kThreads - 2) cnt[(turn + 1) & 1][kThreads - 1 - threadIdx.x] = 0;
-      if ((int)threadIdx.x < half) {
-        const int k = threadIdx.x;
-        int p, q;
+      // The pairs to rotate first, the others from the end, each kind in the order of the pairs
+      // (the order decides how a block of two pairs is rounded): a rank within the warp, and
+      // the counts of the warps before it.
+      const int k = threadIdx.x;
+      const bool mine = k < half;
+      int p = 0, q = 0;
+      bool rot = false;
+      double apq = 0.0;
+      if (mine) {
         if (k == 0) { p = round; q = np - 1; }
         else { p = (round + k) % (np - 1); q = (round - k + np - 1) % (np - 1); }
         if (p > q) { const int t = p; p = q; q = t; }
-        const double apq = H[p * K + q];
-        if (!(apq * apq <= small)) {  // (a NaN is rotated, as in jacobi)
-          const double app = H[p * K + p], aqq = H[q * K + q];
-          const double th = (aqq - app) / (2.0 * apq);
-          const double t = (th >= 0 ? 1.0 : -1.0) / (fabs(th) + sqrt(1.0 + th * th));
-          const double c = 1.0 / sqrt(1.0 + t * t), s = t * c;
-          H[p * K + p] = app - t * apq;
-          H[q * K + q] = aqq + t * apq;
-          H[p * K + q] = 0.0;
-          H[q * K + p] = 0.0;
-          const int at = atomicAdd(count, 1);
-          pp[at] = p; qq[at] = q; cs[at] = c; sn[at] = s;
-          lz_put(lz_remote(&out.pq[at], 1), p | q << 16);
-          lz_put(lz_remote(&out.c[at], 1), c);
-          lz_put(lz_remote(&out.s[at], 1), s);
-        } else {
-          const int at = half - 1 - atomicAdd(count + 1, 1);
-          pp[at] = p; qq[at] = q; cs[at] = 1.0; sn[at] = 0.0;
-        }
+        apq = H[p * K + q];
+        rot = !(apq * apq <= small);  // (a NaN is rotated, as in jacobi)
+      }
+      const int w = k >> 5, nw = (half + 31) / 32;
+      int before = 0;
+      if (w < nw) {
+        const unsigned m = __ballot_sync(0xffffffffu, rot);
+        before = __popc(m & ((1u << (k & 31)) - 1u));
+        if ((k & 31) == 0) count[w] = __popc(m);
+      }
+      if (nw > 1) {
+        __syncthreads();
+        for (int v = 0; v < min(w, nw); ++v) before += count[v];
+      }
+      if (rot) {
+        const double app = H[p * K + p], aqq = H[q * K + q];
+        const double th = (aqq - app) / (2.0 * apq);
+        const double t = (th >= 0 ? 1.0 : -1.0) / (fabs(th) + sqrt(1.0 + th * th));
+        const double c = 1.0 / sqrt(1.0 + t * t), s = t * c;
+        H[p * K + p] = app - t * apq;
+        H[q * K + q] = aqq + t * apq;
+        H[p * K + q] = 0.0;
+        H[q * K + p] = 0.0;
+        pp[before] = p; qq[before] = q; cs[before] = c; sn[before] = s;
+        lz_put(lz_remote(&out.pq[before], 1), p | q << 16);
+        lz_put(lz_remote(&out.c[before], 1), c);
+        lz_put(lz_remote(&out.s[before], 1), s);
+      } else if (mine) {
+        const int at = half - 1 - (k - before);
+        pp[at] = p; qq[at] = q; cs[at] = 1.0; sn[at] = 0.0;
       }
       __syncthreads();
-      const int na = count[0], rest = half - na;
+      int na = 0;
+      for (int v = 0; v < nw; ++v) na += count[v];
+      const int rest = half - na;
       if (threadIdx.x == 0) lz_put(lz_remote(&out.n, 1), na);
       lz_arrive();  // the rotations have gone (and the last ones are read: the wait below)
       const int mixed = na * rest, items = mixed + na * (na - 1) / 2;
@@ -749,7 +766,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads) k_lz_ritz(
   extern __shared__ __align__(16) double M[];  // rank 0: the projected matrix, rank 1: its eigenvectors, transposed
   __shared__ RotMsg msg[2];
   __shared__ double cs[kMaxHalf], sn[kMaxHalf], red[kWarps], th[kMaxK], res[kMaxK];
-  __shared__ int pp[kMaxHalf], qq[kMaxHalf], ord[kMaxK], cnt[2][2];
+  __shared__ int pp[kMaxHalf], qq[kMaxHalf], ord[kMaxK], cnt[2][kRitzWarps];
   const int i = blockIdx.x / 2, rank = blockIdx.x % 2;
   const LzState st = lz_state(g, a.P.N);
   if (st.phase[i] != 1) return;  // (both CTAs)

@@ -31,3 +31,21 @@ def test_projected_eigenproblem(W, H, piece, nev):
     z, ref = S.apply_preconditioner(r, 0).cpu().numpy(), M.apply(r)
     assert np.linalg.norm(z - ref) <= 1e-9 * np.linalg.norm(ref)
     S.close()
+
+
+@pytest.mark.parametrize("nev", [16, 32, 67])
+def test_two_setups_of_a_matrix_give_the_same_bits(nev):
+    """Bases of 58, 90 and 160: the rotations of a round are made by one, two and three warps,
+    and the order in which the warps run must not show."""
+    W = 64
+    m, n, rp, c, v, b, _ = make_grid_ls(W, W, 4, 8, 3, 2)
+    part = block_partition(W, W, 16, 16)
+    r = np.random.default_rng(3).standard_normal(n)
+    out = []
+    for _ in range(4):
+        S = L.Solver(m, n, rp, c, v, part, 16, nev_max=nev, spmv=2)
+        out.append((np.concatenate([S.eigvals(i) for i in range(16)]), S.apply_preconditioner(r, 0).cpu().numpy()))
+        S.close()
+    for lam, z in out[1:]:
+        assert np.array_equal(lam, out[0][0])
+        assert np.array_equal(z, out[0][1])
