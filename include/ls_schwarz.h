@@ -101,12 +101,15 @@ typedef struct {
                           row; -1 / -3 warp-stream (16 / 32 rows per warp); -2 sliced
                           ELL (LS_ERR_INVALID else).  ls_info.lanes_csr / lanes_csc
                           report the codes in use.                                    */
-    int test_stall;    /* test hook, 0 (the default) in normal use: 1 makes the
-                          local-solve kernels (single-vector and block) issue none of
-                          their bulk copies, so every bounded wait for one gives up
-                          (after about two seconds), the kernel sets the error slot and
-                          returns with nothing in flight, and the solve returns
-                          LS_ERR_DEVICE_TIMEOUT.  The CUDA context stays usable.      */
+    int test_stall;    /* test hook, 0 (the default) in normal use: 1 makes the local
+                          solves run the 32-row sweeps (local_config 1 to 3 and the block
+                          kernels, not the superblocks) and issue none of their bulk
+                          copies, so every bounded wait for one gives up (after about
+                          two seconds), the kernel sets the error slot and returns with
+                          nothing in flight, and the solve returns
+                          LS_ERR_DEVICE_TIMEOUT.  The CUDA context stays usable.  (The
+                          superblock kernel has the same bound and error; its hook is in
+                          the bounds-checked build.)                                  */
     int block_kernel;  /* local solve of the multi right-hand-side path with FP32 factors:
                           0 (the default) takes the sweeps over superblocks of 128 rows
                           (all factor precisions; local_kernel reports 0) where they fit

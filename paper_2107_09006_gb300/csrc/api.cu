@@ -1956,6 +1956,9 @@ void ls_debug_alloc(int64_t fail_at, int64_t capacity, int64_t* seen, int64_t* p
   a.fail_at = fail_at;
   a.capacity = capacity;
 }
+
+// Makes the waits of the superblock kernel's launches from now on run out (see g_super_stall).
+void ls_debug_stall(int mode) { lsq::set_super_stall(mode); }
 #endif
 
 ls_status ls_handle_info(const ls_handle* h, ls_info* info) {

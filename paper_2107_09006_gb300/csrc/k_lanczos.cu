@@ -483,7 +483,14 @@ __global__ void __cluster_dims__(kOrthCluster, 1, 1) __launch_bounds__(kThreads)
   const int i = blockIdx.x / kOrthCluster, rank = blockIdx.x % kOrthCluster;
   const LzState st = lz_state(g, a.P.N);
   const int ph = st.phase[i];
-  if (ph == 1 || ph == 2) return;  // (the whole cluster)
+  const bool gave_up = *g.err != 0.0;  // a wait of the sweeps before this launch: every subdomain stops
+  if (ph == 1 || ph == 2 || gave_up) {  // (the whole cluster)
+    if (gave_up) {
+      lz_cluster_sync();  // (every rank has read the phase)
+      if (rank == 0 && threadIdx.x == 0) st.phase[i] = 2;
+    }
+    return;
+  }
   const int ni = (int)(a.P.om_off[i + 1] - a.P.om_off[i]);
   const int npad = (int)(a.P.blk_off[i + 1] - a.P.blk_off[i]) * kT;
   const int K = a.Kmax, Keff = min(K, ni);

@@ -43,7 +43,9 @@
 // between two places, and a rank is never more than one exchange ahead.
 //
 // Every wait is bounded; a warp that gives up sets the CTA's flag, later waits and copies
-// are skipped, all barriers are still met, and the error slot is set.
+// are skipped, all barriers are still met, and the error slot is set.  The thread that arms the
+// message barriers waits on every phase of them itself and stops at the first that does not
+// complete: none is armed again while a phase of it is open.
 #include <type_traits>
 
 #include "common.cuh"
@@ -56,6 +58,16 @@ namespace {
 
 constexpr int kQ = kSuperRows;  // block rows of a superblock
 constexpr long long kSuperWait = 4000000000ll;  // about two seconds at GB300 clocks
+constexpr long long kSuperDrain = 1000000ll;    // about half a millisecond: far above a message's flight
+
+// Test hook of the bounds-checked build (ls_debug_stall): 1 the producer issues no copies, 2 the
+// last CTA of a cluster sends no messages, so that the waits for them run out.
+#ifdef LS_DEBUG_BOUNDS
+int g_super_stall = 0;
+__device__ __forceinline__ int stalled(const SuperArgs& a) { return a.stall; }
+#else
+__device__ __forceinline__ int stalled(const SuperArgs&) { return 0; }
+#endif
 
 __device__ __forceinline__ uint32_t s32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bar_init(uint64_t* bar, uint32_t count) {
@@ -104,17 +116,19 @@ __device__ __forceinline__ bool try_msg(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 template <bool kMsg>
-__device__ __forceinline__ void bounded_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+__device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   auto probe = [&]() { return kMsg ? try_msg(bar, parity) : try_wait(bar, parity); };
-  if (probe() || *abort_flag) return;
+  if (probe()) return true;
+  if (*abort_flag) return false;
   const long long t0 = clock64();
   while (!probe()) {
-    if (*abort_flag) return;
+    if (*abort_flag) return false;
     if (clock64() - t0 > kSuperWait) {
       *abort_flag = 1;
-      return;
+      return false;
     }
   }
+  return true;
 }
 __device__ __forceinline__ void cluster_arrive() {
   __syncwarp();
@@ -664,7 +678,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
       uint32_t par = 1;        // parity of the empty phase a slot waits for (0 after the first wrap)
       int64_t issued = 0;
       long long t0 = clock64();
-      while (!l.done() && !*abort_flag) {
+      while (!l.done() && !*abort_flag && stalled(a) != 1) {
         if (used < depth || test_wait(&eb[slot], par)) {
           if (in_range(base + l.offset(), a.fac_bytes, a.err))
             copy_unit(slots + (size_t)slot * K::UB, fac + l.offset(), K::UB, &fb[slot]);
@@ -754,12 +768,15 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
     if (C > 1) cluster_wait();  // every CTA's barriers are ready
     all_barrier();
 
+    const bool mute = C > 1 && stalled(a) == 2 && rank == C - 1;
+    bool live = true;  // every message that this thread waited for has come
+    auto message = [&](uint64_t* bar, uint32_t parity) { live = bounded_wait<true>(bar, parity, abort_flag) && live; };
     // ---- forward sweep ------------------------------------------------------------------------
     for (int s = 0; s < nsb && (a.sweeps & 1); ++s) {
       const int b0 = s * kQ, b = b0 + q, lim = U * b0, nr = min(nb - b0, kQ);
       const bool has = b < nb;
       const uint32_t mpar = (uint32_t)((s >> 1) & 1);
-      if (C > 1 && tid == 0) {
+      if (C > 1 && tid == 0 && live) {
         bar_expect(&mbar[s & 1], (uint32_t)(nr * 32 * C * sizeof(TA)));
         if (kSplitX) bar_expect(&mbar[4 + (s & 1)], (uint32_t)(U * nr * (nr + 1) / 2 * 32 * sizeof(TA)));
       }
@@ -784,9 +801,10 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
           for (int k = 1; k < JW; ++k) x += red[(w + k) * 32 + lane];
           if constexpr (C > 1) {
             TA* xb = xbuf + (s & 1) * C * kQ * 32 + q * 32 + lane;
+            if (live && !mute)
 #pragma unroll
-            for (int r = 0; r < C; ++r) send(peer(xb + rank * kQ * 32, r), x, peer(&mbar[s & 1], r));
-            bounded_wait<true>(&mbar[s & 1], mpar, abort_flag);
+              for (int r = 0; r < C; ++r) send(peer(xb + rank * kQ * 32, r), x, peer(&mbar[s & 1], r));
+            message(&mbar[s & 1], mpar);
             x = xb[0];
 #pragma unroll
             for (int r = 1; r < C; ++r) x += xb[r * kQ * 32];
@@ -809,8 +827,9 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
           int row;
           const TA x = p.X().out(lane, row);
           if constexpr (kSplitX) {
+            if (live && !mute)
 #pragma unroll
-            for (int r = 0; r < C; ++r) send(peer(db + uu * 32 + row, r), x, peer(&mbar[4 + (s & 1)], r));
+              for (int r = 0; r < C; ++r) send(peer(db + uu * 32 + row, r), x, peer(&mbar[4 + (s & 1)], r));
           } else {
             db[uu * 32 + row] = x;
           }
@@ -818,7 +837,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
         }
         if (!kSplitX) team_barrier();
         if (j == 0) {
-          if (kSplitX) bounded_wait<true>(&mbar[4 + (s & 1)], mpar, abort_flag);
+          if (kSplitX) message(&mbar[4 + (s & 1)], mpar);
           TA x = db[lane];
           for (int k = 1; k < U * (q + 1); ++k) x += db[k * 32 + lane];
           v[b * 32 + lane] = x;
@@ -831,7 +850,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
       const int b0 = s * kQ, b = b0 + q, lim = U * b0, nr = min(nb - b0, kQ);
       const bool has = b < nb;
       const int m = nsb - 1 - s, e = m + ((a.sweeps & 1) ? nsb : 0);  // exchanges so far: of w_s, of X shares
-      if (C > 1 && tid == 0) {
+      if (C > 1 && tid == 0 && live) {
         bar_expect(&mbar[2 + (m & 1)], (uint32_t)(nr * 32 * sizeof(TA)));
         if (kSplitX) bar_expect(&mbar[4 + (e & 1)], (uint32_t)(U * nr * (nr + 1) / 2 * UC * sizeof(TA)));
       }
@@ -846,14 +865,14 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
 #pragma unroll
           for (int k = 0; k < kQ; ++k) ac[(size_t)k * ring * 32].clear();
           if constexpr (C > 1) {
-            if ((U * b + lane / UC) % C == rank)
+            if (live && !mute && (U * b + lane / UC) % C == rank)
 #pragma unroll
               for (int r = 0; r < C; ++r) send(peer(wq + lane, r), x, peer(&mbar[2 + (m & 1)], r));
           } else {
             wq[lane] = x;
           }
         }
-        if (C > 1) bounded_wait<true>(&mbar[2 + (m & 1)], (uint32_t)((m >> 1) & 1), abort_flag);
+        if (C > 1) message(&mbar[2 + (m & 1)], (uint32_t)((m >> 1) & 1));
         else team_barrier();
         // x_s = X^T w_s: unit (q, uu) gives UC columns of its row's share
         p.X().load_x(wq, lane);
@@ -872,8 +891,9 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
           d += c;
           if (lane < UC) {
             if constexpr (kSplitX) {
+              if (live && !mute)
 #pragma unroll
-              for (int r = 0; r < C; ++r) send(peer(d, r), x, peer(&mbar[4 + (e & 1)], r));
+                for (int r = 0; r < C; ++r) send(peer(d, r), x, peer(&mbar[4 + (e & 1)], r));
             } else {
               *d = x;
             }
@@ -884,7 +904,7 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
       if (!kSplitX) all_barrier();
       if (has) {
         if (j == 0) {
-          if (kSplitX) bounded_wait<true>(&mbar[4 + (e & 1)], (uint32_t)((e >> 1) & 1), abort_flag);
+          if (kSplitX) message(&mbar[4 + (e & 1)], (uint32_t)((e >> 1) & 1));
           // rows p >= q of the superblock reach block q: unit column U q + lane / UC
           const int uu = U * q + lane / UC;
           TA x;
@@ -930,6 +950,11 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
     if (kRing && w == NW) cluster_wait();  // (the start's barrier)
     cluster_arrive();             // no CTA leaves while a peer may still write into its shared memory
     cluster_wait();
+    // Every message was waited for, unless a wait gave up: then those that peers sent before the
+    // barrier may still be on their way, and this CTA's shared memory stays until they have come.
+    if (*abort_flag)
+      for (const long long t0 = clock64(); clock64() - t0 < kSuperDrain;) {
+      }
   }
 }
 
@@ -1178,6 +1203,10 @@ bool by_prec(const SuperArgs& a, const SuperShape& f, int prec, int N, int max_n
 
 }  // namespace
 
+#ifdef LS_DEBUG_BOUNDS
+void set_super_stall(int mode) { g_super_stall = mode; }
+#endif
+
 size_t local_super_record(int prec, bool x) {
   if (x) return prec == 0 ? Unit<double>::RECX : Unit<float>::RECX;
   return prec == 0 ? Unit<double>::REC : prec == 1 ? Unit<float>::REC : Unit<__nv_bfloat16>::REC;
@@ -1241,6 +1270,9 @@ bool launch_local_super(const SuperArgs& a, const SuperShape& f, int prec, int N
                         cudaStream_t st) {
   SuperArgs b = a;
   b.ring = f.ring;
+#ifdef LS_DEBUG_BOUNDS
+  b.stall = g_super_stall;
+#endif
   return by_prec(b, f, prec, N, max_nb, optin, false, st);
 }
 

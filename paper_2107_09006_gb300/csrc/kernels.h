@@ -222,7 +222,11 @@ struct SuperArgs {
   int depth;              // units in flight per warp (set by the launcher)
   int ring;               // tile columns of the backward sums (set by the launcher)
   int64_t n_cols, fac_bytes;  // bounds of the gather indices and the records (bounds-checked build)
+  int stall;                  // test hook of that build, set by the launcher
 };
+#ifdef LS_DEBUG_BOUNDS
+void set_super_stall(int mode);
+#endif
 size_t local_super_record(int prec, bool x);
 // Launch shape: CTAs per subdomain, consumer warps and CTAs per SM, tile columns of the
 // backward sums, right-hand sides per CTA.  local_super_plan picks it by rule (block rows of at most wmax tiles, wmean
