@@ -147,7 +147,9 @@ typedef struct {
                           twice the subdomain count does not exceed the SM count); 0 (the
                           default) takes sweeps over superblocks of 128 rows, on one CTA
                           or a cluster per subdomain by rule (reported as 4), where a
-                          subdomain's vector fits their shared memory; else it times
+                          subdomain's vector fits their shared memory and the copy of the
+                          factor that they read fits the device (a call that later runs
+                          out of memory gives the copy up); else it times
                           those of 1 to 3 that fit at the end of setup and keeps the
                           fastest.  Batched handles, whose solves run the multi
                           right-hand-side path, and test_stall take 1.

@@ -199,10 +199,40 @@ void choose_local_config(ls_handle* h, int optin) {
 // handles (whose solves run the multi right-hand-side path) keep the 32-row sweeps.
 void plan_super(ls_handle* h, int optin, int sms) {
   h->sb_optin = optin;
-  h->sb_ok = h->opt.local_config == 0 && !h->opt.test_stall && h->nprob == 1 &&
+  h->sb_ok = h->opt.local_config == 0 && !h->opt.test_stall && h->nprob == 1 && !h->lean &&
              lsq::local_super_plan(h->prec, h->N, h->max_nb, std::max(h->wmax, lsq::kSuperRows),
                                    (double)h->fac_elems / 1024.0 / (double)h->total_blocks, sms, (size_t)optin, h->sb_shape);
 }
+
+}  // namespace
+
+namespace lsi {
+
+bool release_superblocks(ls_handle* h) {
+  BlockState& B = h->blk;
+  if (!h->sb_ok && !B.m_fac.p) return false;
+  h->lean = true;
+  CK(cudaStreamSynchronize(h->st));
+  // the graphs that read them
+  for (cudaGraphExec_t* g : {&h->gexec, &h->gloop, &h->lq_exec, &B.gexec}) {
+    if (*g) cudaGraphExecDestroy(*g);
+    *g = nullptr;
+  }
+  B.m_R = 0;
+  B.m_ok = false;
+  B.m_fac.release(); B.m_tf.release(); B.m_toff.release(); B.m_order.release();
+  if (h->sb_ok) {
+    h->sb_ok = false;
+    h->sb_fac.release(); h->sb_tf.release(); h->sb_toff.release(); h->sb_order.release();
+    choose_local_config(h, h->sb_optin);
+    h->sinfo.local_config = h->local_cfg;
+  }
+  return true;
+}
+
+}  // namespace lsi
+
+namespace {
 
 // out = Q v = R_0^T C_00^{-1} R_0 v (restriction, dense coarse solve, prolongation)
 void coarse_term(ls_handle* h, const double* v, double* out) {
@@ -1340,7 +1370,8 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   const std::vector<lsq::CholGroup> chol = lsq::chol_groups(N, hs.blk_off.data(), hs.blk_tf.data(), corder);
   DevBuf<int32_t> chol_order;
   chol_order.upload(corder, st);
-  if (h->coarse) {
+  const bool both = h->coarse && !h->lean;
+  if (both) {
     // The two factorisations, each a chain of small launches, run beside one another; the
     // solve's stream waits for both before anything else.  (16 subdomains of 1,900 columns:
     // 9.3 ms one after the other, about 6 so)
@@ -1353,7 +1384,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     CK(cudaEventRecord(h->ev_coarse, h->st2));
   }
   lsq::launch_band_cholesky(plan, chol, chol_order.p, Cst.p, idiag.p, dinv.p, status.p, st);
-  if (h->coarse) CK(cudaStreamWaitEvent(st, h->ev_coarse, 0));
+  if (both) CK(cudaStreamWaitEvent(st, h->ev_coarse, 0));
   std::vector<int> hst(N);
   CK(cudaMemcpyAsync(hst.data(), status.p, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -1412,6 +1443,11 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   if (h->coarse) {
     const double te0 = now_s();
     phase.next("ls_setup: local eigensolves and coarse operator");
+    if (!both) {  // (with the first factorisation's scratch)
+      Bidiag.alloc((size_t)h->total_blocks * 32);
+      Bstatus.alloc(N);
+      lsq::launch_band_cholesky(plan, chol, chol_order.p, Bst.p, Bidiag.p, dinv.p, Bstatus.p, st);
+    }
     CK(cudaMemcpyAsync(hst.data(), Bstatus.p, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     check_launch("Cholesky of C~_ii + s I");
@@ -1455,7 +1491,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     {
       int optin = 0;
       CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
-      if (hs.xi_off[N] < INT32_MAX &&
+      if (!h->lean && hs.xi_off[N] < INT32_MAX &&
           lsq::local_super_plan(0, N, h->max_nb, std::max(h->wmax, lsq::kSuperRows),
                                 (double)h->fac_elems / 1024.0 / (double)h->total_blocks, sms, (size_t)optin, lg.shape)) {
         Ctst.release();  // (the operator runs from A)
@@ -1781,56 +1817,71 @@ ls_status setup_entry(int32_t nprob, const int64_t* m_off, const int64_t* n_off,
     if (m < 1 || n < 1 || m < n) throw LsError(LS_ERR_INVALID, "need m >= n >= 1");
     if (nparts < 1 || nparts > n) throw LsError(LS_ERR_INVALID, "nparts must lie in [1, n]");
     if (overlap != 1) throw LsError(LS_ERR_UNSUPPORTED, "only overlap = 1 is defined for the splitting");
-    std::unique_ptr<ls_handle> h(new ls_handle());
-    ls_default_options(&h->opt);
-    if (opt) h->opt = *opt;
-    if (h->opt.factor_prec < 0 || h->opt.factor_prec > 2) throw LsError(LS_ERR_INVALID, "bad factor_prec");
-    if (h->opt.maxit < 1 && h->opt.fixed_iters < 1) throw LsError(LS_ERR_INVALID, "maxit must be positive");
-    if (h->opt.nev_max < 0) throw LsError(LS_ERR_INVALID, "nev_max must be >= 0");
-    if (h->opt.variant < 0 || h->opt.variant > 2) throw LsError(LS_ERR_INVALID, "variant must be 0, 1 or 2");
-    if (h->opt.solver < 0 || h->opt.solver > 2) throw LsError(LS_ERR_INVALID, "solver must be 0, 1 or 2");
-    if (h->opt.variant == 2 && h->opt.solver != 2)
-      throw LsError(LS_ERR_INVALID, "the deflated RAS variant is not symmetric: it needs solver = 2 (GMRES)");
-    if (h->opt.solver == 2 && (h->opt.restart < 1 || h->opt.restart > 1000))
-      throw LsError(LS_ERR_INVALID, "restart must lie in [1, 1000]");
-    if (h->opt.test_stall != 0 && h->opt.test_stall != 1) throw LsError(LS_ERR_INVALID, "test_stall must be 0 or 1");
-    if (h->opt.block_kernel < 0 || h->opt.block_kernel > 2) throw LsError(LS_ERR_INVALID, "block_kernel must be 0, 1 or 2");
-    if (h->opt.normal_product < 0 || h->opt.normal_product > 2)
-      throw LsError(LS_ERR_INVALID, "normal_product must be 0, 1 or 2");
-    if (h->opt.local_config < 0 || h->opt.local_config > 3) throw LsError(LS_ERR_INVALID, "local_config must lie in [0, 3]");
-    if (h->opt.normal_kernel < 0 || h->opt.normal_kernel > 4)
-      throw LsError(LS_ERR_INVALID, "normal_kernel must lie in [0, 4]");
-    if (h->opt.spmv != 0 && !lsq::valid_spmv_code(h->opt.spmv))
-      throw LsError(LS_ERR_INVALID, "spmv must be 0 or a sparse-product kernel code");
-    if (h->opt.variant != 0 && nprob > 1)
-      throw LsError(LS_ERR_UNSUPPORTED, "the balanced and deflated variants are implemented for single-problem handles");
-    if (!(tau < 1.0)) throw LsError(tau >= 1.0 ? LS_ERR_UNSUPPORTED : LS_ERR_INVALID,
-                                    "tau >= 1 keeps the eigenvalue-1 cluster, which the device Lanczos cannot resolve");
-    h->tau = tau;
-    CK(cudaGetDevice(&h->dev));
-    if (stream) {
-      h->st = (cudaStream_t)stream;
-    } else {
-      CK(cudaStreamCreateWithFlags(&h->st, cudaStreamNonBlocking));
-      h->own_stream = true;
-    }
-    h->m = m; h->n = n; h->N = nparts;
-    h->nprob = nprob;
-    if (m_off && n_off) {
-      h->h_m_off.assign(m_off, m_off + nprob + 1);
-      h->h_n_off.assign(n_off, n_off + nprob + 1);
-    } else {
-      h->h_m_off = {0, m};
-      h->h_n_off = {0, n};
-    }
-    h->coarse = h->opt.coarse != 0 && h->opt.nev_max > 0;
-    h->sinfo.bad_subdomain = -1;
+    std::unique_ptr<ls_handle> h;
+    auto attempt = [&](bool lean) {
+      h.reset(new ls_handle());
+      h->lean = lean;
+      ls_default_options(&h->opt);
+      if (opt) h->opt = *opt;
+      if (h->opt.factor_prec < 0 || h->opt.factor_prec > 2) throw LsError(LS_ERR_INVALID, "bad factor_prec");
+      if (h->opt.maxit < 1 && h->opt.fixed_iters < 1) throw LsError(LS_ERR_INVALID, "maxit must be positive");
+      if (h->opt.nev_max < 0) throw LsError(LS_ERR_INVALID, "nev_max must be >= 0");
+      if (h->opt.variant < 0 || h->opt.variant > 2) throw LsError(LS_ERR_INVALID, "variant must be 0, 1 or 2");
+      if (h->opt.solver < 0 || h->opt.solver > 2) throw LsError(LS_ERR_INVALID, "solver must be 0, 1 or 2");
+      if (h->opt.variant == 2 && h->opt.solver != 2)
+        throw LsError(LS_ERR_INVALID, "the deflated RAS variant is not symmetric: it needs solver = 2 (GMRES)");
+      if (h->opt.solver == 2 && (h->opt.restart < 1 || h->opt.restart > 1000))
+        throw LsError(LS_ERR_INVALID, "restart must lie in [1, 1000]");
+      if (h->opt.test_stall != 0 && h->opt.test_stall != 1) throw LsError(LS_ERR_INVALID, "test_stall must be 0 or 1");
+      if (h->opt.block_kernel < 0 || h->opt.block_kernel > 2) throw LsError(LS_ERR_INVALID, "block_kernel must be 0, 1 or 2");
+      if (h->opt.normal_product < 0 || h->opt.normal_product > 2)
+        throw LsError(LS_ERR_INVALID, "normal_product must be 0, 1 or 2");
+      if (h->opt.local_config < 0 || h->opt.local_config > 3) throw LsError(LS_ERR_INVALID, "local_config must lie in [0, 3]");
+      if (h->opt.normal_kernel < 0 || h->opt.normal_kernel > 4)
+        throw LsError(LS_ERR_INVALID, "normal_kernel must lie in [0, 4]");
+      if (h->opt.spmv != 0 && !lsq::valid_spmv_code(h->opt.spmv))
+        throw LsError(LS_ERR_INVALID, "spmv must be 0 or a sparse-product kernel code");
+      if (h->opt.variant != 0 && nprob > 1)
+        throw LsError(LS_ERR_UNSUPPORTED, "the balanced and deflated variants are implemented for single-problem handles");
+      if (!(tau < 1.0)) throw LsError(tau >= 1.0 ? LS_ERR_UNSUPPORTED : LS_ERR_INVALID,
+                                      "tau >= 1 keeps the eigenvalue-1 cluster, which the device Lanczos cannot resolve");
+      h->tau = tau;
+      CK(cudaGetDevice(&h->dev));
+      if (stream) {
+        h->st = (cudaStream_t)stream;
+      } else {
+        CK(cudaStreamCreateWithFlags(&h->st, cudaStreamNonBlocking));
+        h->own_stream = true;
+      }
+      h->m = m; h->n = n; h->N = nparts;
+      h->nprob = nprob;
+      if (m_off && n_off) {
+        h->h_m_off.assign(m_off, m_off + nprob + 1);
+        h->h_n_off.assign(n_off, n_off + nprob + 1);
+      } else {
+        h->h_m_off = {0, m};
+        h->h_n_off = {0, n};
+      }
+      h->coarse = h->opt.coarse != 0 && h->opt.nev_max > 0;
+      h->sinfo.bad_subdomain = -1;
+      try {
+        do_setup(h.get(), row_ptr, col, val, part);
+      } catch (...) {
+        cudaStreamSynchronize(h->st);
+        throw;
+      }
+    };
+    // Where the superblock copies of the factor do not fit, or something after them, setup runs
+    // again without them (three copies of the factor in FP64 while it runs, and the solve storage;
+    // five with them).
+    bool again = false;
     try {
-      do_setup(h.get(), row_ptr, col, val, part);
-    } catch (...) {
-      cudaStreamSynchronize(h->st);
-      throw;
+      attempt(false);
+    } catch (const LsError& e) {
+      if (e.st != LS_ERR_OOM) throw;
+      again = true;
     }
+    if (again) attempt(true);
     *out = h.release();
     return LS_OK;
   });
@@ -1895,8 +1946,10 @@ ls_status ls_backward(ls_handle* h, const double* b, const double* x, const doub
     cudaStream_t st = h->st;
     ls_status last = LS_OK;
     DevBuf<double>&xk = h->bk_x, &lam = h->bk_lam, &mu = h->bk_mu, &tmp = h->bk_m, &gperm = h->bk_nnz, &gout = h->bk_out;
-    reserve(xk, h->n); reserve(lam, h->n); reserve(mu, h->m); reserve(tmp, h->m);
-    if (grad_vals) { reserve(gperm, h->nnz); reserve(gout, h->nnz); }
+    with_room(h, [&] {
+      reserve(xk, h->n); reserve(lam, h->n); reserve(mu, h->m); reserve(tmp, h->m);
+      if (grad_vals) { reserve(gperm, h->nnz); reserve(gout, h->nnz); }
+    });
     for (int k = 0; k < nrhs; ++k) {
       CK(cudaMemcpyAsync(h->tv.p, grad_x + (int64_t)k * h->n, sizeof(double) * h->n, cudaMemcpyDefault, st));
       ls_status s = solve_core(h, 1, rtol, info);
@@ -1934,7 +1987,7 @@ ls_status ls_update_values(ls_handle* h, const double* val) {
     cudaStream_t st = h->st;
     const int64_t nnz = h->nnz;
     DevBuf<double>& tmp = h->bk_nnz;
-    reserve(tmp, nnz);
+    with_room(h, [&] { reserve(tmp, nnz); });
     CK(cudaMemcpyAsync(tmp.p, val, sizeof(double) * nnz, cudaMemcpyDefault, st));
     lsq::launch_gather64(nnz, h->entmap.p, tmp.p, h->val.p, st);  // A' = P A, CSR
     refresh_value_copies(h);

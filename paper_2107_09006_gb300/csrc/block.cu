@@ -176,7 +176,7 @@ void plan_block_super(ls_handle* h, int R) {
   B.gR = 0;  // (a graph of the last plan is not replayed)
   lsq::SuperShape shape{};
   const int64_t groups = (R + 7) / 8;
-  bool ok = h->opt.block_kernel == 0 && !h->opt.test_stall && !(h->prec == LS_PREC_F32 && h->nprob > 1 && R < 4);
+  bool ok = h->opt.block_kernel == 0 && !h->opt.test_stall && !h->lean && !(h->prec == LS_PREC_F32 && h->nprob > 1 && R < 4);
   if (ok) {
     int optin = 0, sms = 0;
     CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
@@ -186,7 +186,14 @@ void plan_block_super(ls_handle* h, int R) {
          lsq::local_super_plan_multi(h->prec, R, h->N, h->max_nb, std::max(h->wmax, lsq::kSuperRows), sms,
                                      (size_t)optin, shape);
   }
-  if (ok && !B.m_fac.p) pack_block_super(h);
+  if (ok && !B.m_fac.p) {
+    try {
+      pack_block_super(h);
+    } catch (const LsError& e) {
+      if (e.st != LS_ERR_OOM) throw;
+      ok = false;  // the 32-row kernels, of the solve storage that is there
+    }
+  }
   B.m_shape = shape;
   B.m_ok = ok;
   B.m_R = R;
@@ -255,16 +262,16 @@ void choose_local_kernel(ls_handle* h, int R, const double* Rin) {
   if (opt == 2 && !B.u_ok)
     throw LsError(LS_ERR_UNSUPPORTED, "the tcgen05 local solve does not fit this factor's widest block row");
   if (opt == 1 || (!B.u_ok && opt == 0)) {
-    swizzle_prepare(h);
+    with_room(h, [&] { swizzle_prepare(h); });
     B.kernel = 1;
     return;
   }
-  umma_prepare(h);
+  with_room(h, [&] { umma_prepare(h); });
   if (opt == 2 || h->opt.test_stall) {
     B.kernel = 2;
     return;
   }
-  swizzle_prepare(h);
+  with_room(h, [&] { swizzle_prepare(h); });
   cudaStream_t st = h->st;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
@@ -689,7 +696,7 @@ ls_status block_solve(ls_handle* h, const double* b, int R, double rtol, double*
   cudaStream_t st = h->st;
   check_block(h, R);
   const double t0 = now_s();
-  ensure_buffers(h, R);
+  with_room(h, [&] { ensure_buffers(h, R); });
   plan_block_super(h, R);
   ls_info inf{};
   inf.bad_subdomain = -1;
@@ -727,9 +734,12 @@ ls_status block_backward(ls_handle* h, const double* b, const double* x, const d
   cudaStream_t st = h->st;
   check_block(h, R);
   const double t0 = now_s();
-  ensure_buffers(h, R);
+  with_room(h, [&] { ensure_buffers(h, R); });
   plan_block_super(h, R);
-  if (B.G.n < (size_t)h->n * R) B.G.alloc((size_t)h->n * R);
+  with_room(h, [&] {
+    if (B.G.n < (size_t)h->n * R) B.G.alloc((size_t)h->n * R);
+    if (grad_vals && (int64_t)h->bk_out.n < h->nnz) h->bk_out.alloc(h->nnz);
+  });
   ls_info inf{};
   inf.bad_subdomain = -1;
   int launches = 0;
@@ -761,7 +771,6 @@ ls_status block_backward(ls_handle* h, const double* b, const double* x, const d
     lsq::launch_b_spmm_csr(csr(h), B.Z.p, B.Bu.p, R, st);
     lsq::launch_b_sub((int64_t)h->m * R, B.B.p, B.Bu.p, st);
     DevBuf<double>& gout = h->bk_out;
-    if ((int64_t)gout.n < h->nnz) gout.alloc(h->nnz);
     lsq::launch_b_grad_vals(csr(h), h->entmap.p, R, B.Bu.p, B.X.p, B.Q.p, B.Z.p, gout.p, st);
     CK(cudaMemcpyAsync(grad_vals, gout.p, sizeof(double) * h->nnz, cudaMemcpyDefault, st));
     CK(cudaStreamSynchronize(st));

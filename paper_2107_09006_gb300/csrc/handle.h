@@ -34,7 +34,7 @@ struct LsError : std::runtime_error {
   } while (0)
 
 // Device-memory ceiling of the bounds-checked build's tests (ls_debug_alloc): refuses the
-// fail_at-th allocation from then on (0: none) and what would take the library's buffers
+// fail_at-th allocation from then on (0: none; below 0: the -fail_at-th and all after) and what would take the library's buffers
 // above `capacity` bytes (0: no ceiling).  The product build has none of it.
 #ifdef LS_DEBUG_BOUNDS
 struct AllocHook {
@@ -43,7 +43,8 @@ struct AllocHook {
 inline AllocHook g_alloc_hook;
 inline bool alloc_refused(size_t bytes) {
   AllocHook& a = g_alloc_hook;
-  if (++a.seen == a.fail_at) return true;
+  const int64_t k = ++a.seen, at = a.fail_at;
+  if (k == at || (at < 0 && k >= -at)) return true;
   return a.capacity > 0 && a.used + (int64_t)bytes > a.capacity;
 }
 inline void alloc_count(size_t bytes, bool add) {
@@ -247,7 +248,9 @@ struct ls_handle {
   DevBuf<__nv_bfloat16> L16;
   int max_nb = 0;
   int local_cfg = 1;  // configuration of the single-vector local solve (option local_config)
-  // superblock storage of the single-vector local solve (local_cfg 4)
+  // superblock storage of the single-vector local solve (local_cfg 4).  lean: memory is short, no
+  // copy of the factor beside the solve storage (see with_room)
+  bool lean = false;
   bool sb_ok = false;
   int sb_optin = 0;
   lsq::SuperShape sb_shape{};
@@ -326,6 +329,23 @@ struct ls_handle {
 };
 
 namespace lsi {
+
+// Frees the copies of the factor that the superblock kernels read and has the handle run the
+// 32-row kernels from then on (api.cu); false if there is none.
+bool release_superblocks(ls_handle* h);
+
+// f(), which allocates.  The superblock copies are for speed only: when memory runs out with
+// them held they go, and f() has what they took.  (f can be called again after LS_ERR_OOM.)
+template <class F>
+inline void with_room(ls_handle* h, F&& f) {
+  try {
+    f();
+    return;
+  } catch (const LsError& e) {
+    if (e.st != LS_ERR_OOM || !release_superblocks(h)) throw;
+  }
+  f();
+}
 
 // Superblock storage of the block-envelope plan in factor precision prec: first tile column
 // (reaching back to the superblock's first) and byte offset of every block row, subdomains by
