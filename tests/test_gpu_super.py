@@ -88,3 +88,43 @@ def test_super_many_right_hand_sides(name, prec, R):
     tol = 1e-10 if prec == "f64" else 1e-4
     for q in range(R):
         assert float((X[q] - ref[q]).norm() / ref[q].norm()) < tol, q
+
+
+# the rest of the rule: name -> as above, here with the counts that select the shape
+SHAPES.update({
+    "n64": (128, 128, (6, 2), lambda W, H: block_partition(W, H, 16, 16)),
+    "n100-32": (320, 320, (8, 3), lambda W, H: block_partition(W, H, 32, 32)),
+})
+
+
+def _rule(name, prec):
+    """(subdomains, mean width of a block row in tiles, SMs)"""
+    import paper_2107_09006_gb300 as L
+
+    W, H, (k, radius), split = SHAPES[name]
+    m, n, rp, col, val, _, _ = make_grid_ls(W, H, 4, k, radius, 7)
+    part = split(W, H)
+    S = L.Solver(m, n, rp, col, val, part, int(part.max()) + 1, coarse=0, factor_prec=prec)
+    st = S.storage()
+    S.close()
+    return (int(part.max()) + 1, st["fac_elems"] / 1024 / st["total_blocks"],
+            torch.cuda.get_device_properties(0).multi_processor_count)
+
+
+def test_super_pair_of_ctas_in_double():
+    N, _, sms = _rule("n64", "f64")
+    assert 2 * N <= sms < 4 * N
+    test_super_matches_row_sweeps("n64", "f64")
+
+
+@pytest.mark.parametrize("prec", ["f32", "bf16"])
+def test_super_one_cta_of_24_warps(prec):
+    N, width, sms = _rule("n100-32", prec)
+    assert N <= sms < 2 * N and width >= 8.0
+    test_super_matches_row_sweeps("n100-32", prec)
+
+
+def test_super_many_right_hand_sides_on_a_pair_in_double():
+    N, _, sms = _rule("n64", "f64")
+    assert 2 * N <= sms < 4 * N
+    test_super_many_right_hand_sides("n64", "f64", 3)
