@@ -112,10 +112,12 @@ typedef struct {
                           the bounds-checked build.)                                  */
     int block_kernel;  /* local solve of the multi right-hand-side path with FP32 factors:
                           0 (the default) takes the sweeps over superblocks of 128 rows
-                          (all factor precisions; local_kernel reports 0) where they fit
-                          and the solve is not so wide that the 32-row sweeps fill the
-                          chip several times over, else times both of those at the first
-                          block solve and keeps the faster; 1 TF32 mma.sync tiles, left-looking sweeps; 2
+                          (all factor precisions; local_kernel reports 0) where they and
+                          their copies of the factor fit, the solve is not so wide that
+                          the 32-row sweeps fill the chip several times over, and, on a
+                          batched handle, from four right-hand sides on; else it times
+                          the two below at the first block solve and keeps the faster;
+                          1 TF32 mma.sync tiles, left-looking sweeps; 2
                           tcgen05 MMAs (M = 128, accumulator in tensor memory),
                           right-looking sweeps (LS_ERR_UNSUPPORTED if the widest factor
                           block row does not fit its shared-memory window).  Both round

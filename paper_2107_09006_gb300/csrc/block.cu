@@ -159,15 +159,17 @@ void pack_block_super(ls_handle* h) {
 }
 
 // Whether the block local solve of R right-hand sides runs over superblocks (by rule), its
-// storage made from the solve storage at the first use.  With a forced block_kernel or the
-// stalled test hook it does not.  FP32 factors (eight right-hand sides per CTA): not where
-// more than two groups of eight make more than three CTAs per SM (N = 256, R = 32: 968 us
-// against 780 for the mma.sync kernel, which reads a tile once for all 32; N = 64, R = 32: 273
-// against 438 for the tcgen05 kernel; R = 8: 163 against 432; N = 256, R = 8: 284 against
-// 774), and on a batched handle from four right-hand sides on: below, the automatic choice is
-// pinned by a test to one of the two tensor-core kernels (64 subdomains and R = 2: 430 us,
-// the superblocks 164).  The plan counts only when all of it has
-// succeeded: after an error the next call plans anew.
+// storage made from the solve storage at the first use.  It does not with a forced
+// block_kernel, the stalled test hook or no room for the storage, nor with FP32 factors (eight
+// right-hand sides per CTA) in two cases:
+// - more than two groups of eight that make more than three CTAs per SM (N = 256, R = 32: 968
+//   us against 780 for the mma.sync kernel, which reads a tile once for all 32; but N = 64, R =
+//   32: 273 against 438 for the tcgen05 kernel; R = 8: 163 against 432; N = 256, R = 8: 284
+//   against 774);
+// - fewer than four right-hand sides on a batched handle, where the automatic choice has been
+//   one of the two tensor-core kernels and callers read which from ls_info.local_kernel (64
+//   subdomains and R = 2: 430 us; the superblocks would take 164).
+// The plan counts only when all of it has succeeded: after an error the next call plans anew.
 void plan_block_super(ls_handle* h, int R) {
   BlockState& B = h->blk;
   if (B.m_R == R) return;

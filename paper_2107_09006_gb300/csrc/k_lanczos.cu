@@ -3,13 +3,17 @@
 //
 // With C~_ii + s I = L L^T, the pencil is the symmetric standard problem
 // T u = lambda u, T = L^{-1} D_i C_ii D_i L^{-T}, v = L^{-T} u (so v is
-// (C~_ii + s I)-normalised).  Each CTA runs a thick-restart Lanczos (Krylov-Schur
-// form) on its subdomain: full re-orthogonalisation in two Gram-Schmidt passes,
+// (C~_ii + s I)-normalised).  Each subdomain runs a thick-restart Lanczos (Krylov-Schur
+// form): full re-orthogonalisation in two Gram-Schmidt passes,
 // Rayleigh-Ritz on the projected matrix by parallel cyclic Jacobi, restart on the
 // best `keep` Ritz vectors.  Only products and solves are needed (Remark 3.2):
 // D C_ii D x = D (C~_ii (D x)) + delta D x, since the interior block of C~_ii equals
 // that of C_ii = A(:,Omega)^T A(:,Omega) + delta I.  Every loop is bounded by
 // maxit; a subdomain that does not converge reports status 2.
+//
+// Two forms with the same recurrences: run_lanczos_grid, every stage of a step a kernel over
+// all subdomains, where a subdomain's FP64 vector fits the superblock kernel; k_lanczos, one
+// CTA per subdomain for the whole iteration, where it does not or memory is short.
 #include <algorithm>
 #include <vector>
 

@@ -824,15 +824,15 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
             mma_put<false>(p, db + uu * 32, lane);
             continue;
           } else {
-          int row;
-          const TA x = p.X().out(lane, row);
-          if constexpr (kSplitX) {
-            if (live && !mute)
+            int row;
+            const TA x = p.X().out(lane, row);
+            if constexpr (kSplitX) {
+              if (live && !mute)
 #pragma unroll
-              for (int r = 0; r < C; ++r) send(peer(db + uu * 32 + row, r), x, peer(&mbar[4 + (s & 1)], r));
-          } else {
-            db[uu * 32 + row] = x;
-          }
+                for (int r = 0; r < C; ++r) send(peer(db + uu * 32 + row, r), x, peer(&mbar[4 + (s & 1)], r));
+            } else {
+              db[uu * 32 + row] = x;
+            }
           }
         }
         if (!kSplitX) team_barrier();
@@ -885,19 +885,19 @@ __global__ void __launch_bounds__(NW * 32 + (sizeof(typename P::T) == 8 ? 32 : 0
             mma_put<false>(p, d, lane);
             continue;
           } else {
-          int c;
-          const TA x = p.X().bwd(acquire(), lane, c);
-          release();
-          d += c;
-          if (lane < UC) {
-            if constexpr (kSplitX) {
-              if (live && !mute)
+            int c;
+            const TA x = p.X().bwd(acquire(), lane, c);
+            release();
+            d += c;
+            if (lane < UC) {
+              if constexpr (kSplitX) {
+                if (live && !mute)
 #pragma unroll
-                for (int r = 0; r < C; ++r) send(peer(d, r), x, peer(&mbar[4 + (e & 1)], r));
-            } else {
-              *d = x;
+                  for (int r = 0; r < C; ++r) send(peer(d, r), x, peer(&mbar[4 + (e & 1)], r));
+              } else {
+                *d = x;
+              }
             }
-          }
           }
         }
       }
@@ -1219,14 +1219,14 @@ size_t local_super_record(int prec, bool x) {
 // against 936, BF16 508 against 748).
 // FP64: the largest cluster whose CTAs all run at once, since the FP64 units bound it (p =
 // 32, N = 16: 443, 276, 207 with 1, 2, 4 CTAs, 711 before; p = 20, N = 9: 106 with 8).
-// FP32, BF16, by the mean width of a block row in tiles: one CTA is bound by the SM's intake,
-// a pair by its exchanges.  Below 8 tiles one CTA of 16 warps (a 211 x 173 grid in 50 uneven
-// pieces, 7.3 tiles: kernel 53, pair 55, 24 warps 62, pair of 24 warps 66; 133 before);
-// from 8 tiles on a pair of 24 warps when two CTAs per subdomain have an SM each (p = 48, 12
-// tiles, N = 64: 178, pair of 16 warps 198, one CTA 202; p = 32, 8.5 tiles: 126, 127, 130),
-// else one CTA of 24 warps (p = 48, N = 144: 280 against 296 with 16); from 13 tiles on four
-// CTAs of 16 warps where there is room (p = 64, 14.5 tiles, N = 16: 225 against 277 for the
-// pair; 571 before).
+// FP32, BF16, by the mean width of a block row in tiles: one CTA is bound by the SM's intake, a
+// pair by its exchanges; near the line of 8 tiles the two are within 4 %.  Below 8 tiles one CTA
+// of 16 warps (a 211 x 173 grid in 50 uneven pieces, 7.3 tiles: kernel 53, pair 55, 24 warps 62,
+// pair of 24 warps 66; 133 before); from 8 tiles on a pair of 24 warps when two CTAs per
+// subdomain have an SM each (p = 48, 12 tiles, N = 64: 178, pair of 16 warps 198, one CTA 202; p
+// = 32, 8.5 tiles: 126, 127, 130), else one CTA of 24 warps (p = 48, N = 144: 280 against 296
+// with 16); from 13 tiles on four CTAs of 16 warps where there is room (p = 64, 14.5 tiles, N =
+// 16: 225 against 277 for the pair; 571 before).
 bool local_super_plan(int prec, int N, int max_nb, int wmax, double wmean, int sms, size_t optin, SuperShape& out) {
   auto fits = [&](int cluster, int warps, int occ) {
     out = SuperShape{cluster, warps, occ, wmax + kQ, 1};
