@@ -115,6 +115,48 @@ __global__ void __launch_bounds__(kThreads) k_spmv_csc(CscDev At, const double* 
   if (ds.parts) finish_dots(dacc, 0.0, false, ds);
 }
 
+// y = B x for a CSR matrix B (A, or A^T through the CSC copy) of unknown row lengths: V lanes
+// per row as in k_spmv_csr, but a row of more than kLongRow entries per lane is left to its
+// whole warp.  V goes by the mean length, and a few lanes on one long row are a chain that
+// the rest of the matrix does not hide (400,000 rows of six entries, 25 us, and one of
+// 100,000: 6.6 ms with two lanes on it, 2.2 with eight, 0.56 so; a column of 100,000 among
+// columns of 24: 3.6 ms with four lanes, 0.40 so; Pareto row lengths: 8, 16 and 32 entries per
+// lane 104, 84 and 86 us).  The bound on the blocks keeps 32 registers where rows are short.
+constexpr int kLongRow = 16;
+template <int V>
+__global__ void __launch_bounds__(kThreads, V <= 2 ? 8 : 6) k_product(int64_t rows, const int64_t* __restrict__ ptr,
+                                                      const int32_t* __restrict__ idx, const double* __restrict__ val,
+                                                      const double* __restrict__ x, double* __restrict__ y) {
+  const int lane = threadIdx.x & 31, sub = lane % V;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x / V;
+  for (int64_t r0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane) / V; r0 < rows; r0 += stride) {
+    const int64_t r = r0 + lane / V;  // (the loop is the warp's)
+    double acc = 0.0;
+    bool longrow = false;
+    if (r < rows) {
+      const int64_t e0 = __ldg(ptr + r), e1 = __ldg(ptr + r + 1);
+      longrow = V < 32 && e1 - e0 > kLongRow * V;
+      if (!longrow) {
+#pragma unroll 4
+        for (int64_t e = e0 + sub; e < e1; e += V) acc += __ldg(val + e) * __ldg(x + __ldg(idx + e));
+      }
+    }
+#pragma unroll
+    for (int o = V / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (r < rows && sub == 0 && !longrow) y[r] = acc;
+    if constexpr (V < 32) {
+      for (unsigned todo = __ballot_sync(0xffffffffu, longrow && sub == 0); todo; todo &= todo - 1) {
+        const int64_t rl = r0 + (__ffs(todo) - 1) / V, e1 = __ldg(ptr + rl + 1);
+        double s = 0.0;
+#pragma unroll 4
+        for (int64_t e = __ldg(ptr + rl) + lane; e < e1; e += 32) s += __ldg(val + e) * __ldg(x + __ldg(idx + e));
+        s = warp_sum(s);
+        if (lane == 0) y[rl] = s;
+      }
+    }
+  }
+}
+
 // Warp-stream product y = B x for a CSR matrix B (A itself, or A^T through the CSC copy):
 // each warp takes R consecutive rows, loads all their entries coalesced (lanes stride the
 // entry range, all loads independent), keeps the products in shared memory, then lane k
@@ -834,6 +876,19 @@ void launch_spmv_csr(const CsrDev& A, const double* x, double* y, int lanes, int
     case 8: k_spmv_csr<8><<<grid, kThreads, 0, st>>>(A, x, y); break;
     case 16: k_spmv_csr<16><<<grid, kThreads, 0, st>>>(A, x, y); break;
     default: k_spmv_csr<32><<<grid, kThreads, 0, st>>>(A, x, y); break;
+  }
+}
+
+void launch_product(int64_t rows, const int64_t* ptr, const int32_t* idx, const double* val, const double* x, double* y,
+                    int lanes, cudaStream_t st) {
+  const int grid = grid_for(rows * lanes, kThreads, kMaxGrid);
+  switch (lanes) {
+    case 1: k_product<1><<<grid, kThreads, 0, st>>>(rows, ptr, idx, val, x, y); break;
+    case 2: k_product<2><<<grid, kThreads, 0, st>>>(rows, ptr, idx, val, x, y); break;
+    case 4: k_product<4><<<grid, kThreads, 0, st>>>(rows, ptr, idx, val, x, y); break;
+    case 8: k_product<8><<<grid, kThreads, 0, st>>>(rows, ptr, idx, val, x, y); break;
+    case 16: k_product<16><<<grid, kThreads, 0, st>>>(rows, ptr, idx, val, x, y); break;
+    default: k_product<32><<<grid, kThreads, 0, st>>>(rows, ptr, idx, val, x, y); break;
   }
 }
 

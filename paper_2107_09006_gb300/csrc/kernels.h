@@ -48,6 +48,8 @@ constexpr int kVecGrid = 1216;   // grid cap of the n-vector kernels (8 blocks o
 // out[0] and out[out2].
 struct DotSite { double* parts; int stride; unsigned* counter; double* out; int out2; };
 
+void launch_product(int64_t rows, const int64_t* ptr, const int32_t* idx, const double* val, const double* x, double* y,
+                    int lanes, cudaStream_t st);  // y = B x, B in CSR, long rows on whole warps
 void launch_spmv_csr(const CsrDev& A, const double* x, double* y, int lanes, int grid, cudaStream_t st);
 // w = A^T q; with ds.parts != nullptr also (d . w) -> *ds.out (d = w if d == nullptr).
 void launch_spmv_csc(const CscDev& At, const double* q, double* w, const double* d, const DotSite& ds, int lanes,

@@ -137,16 +137,13 @@ extern "C" ls_status ls_normal_product_noalloc(int64_t m, int64_t n, const int64
     q = a.ptr;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const lsq::CsrDev A{m, n, row_ptr, col, val};
-  const lsq::CscDev At{m, n, col_ptr, row, cval};
-  lsq::launch_spmv_csr(A, p, q, product_lanes(m, (double)nnz / (double)m), 0, st);
+  lsq::launch_product(m, row_ptr, col, val, p, q, product_lanes(m, (double)nnz / (double)m), st);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
     g_msg = std::string("launch of q = A p failed: ") + cudaGetErrorString(e);
     return LS_ERR_CUDA;
   }
-  lsq::launch_spmv_csc(At, q, w, nullptr, lsq::DotSite{}, product_lanes(n, (double)nnz / (double)n), 0,
-                       st);
+  lsq::launch_product(n, col_ptr, row, cval, q, w, product_lanes(n, (double)nnz / (double)n), st);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
     g_msg = std::string("launch of w = A^T q failed: ") + cudaGetErrorString(e);
