@@ -1369,7 +1369,7 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
   std::vector<int32_t> corder;
   const std::vector<lsq::CholGroup> chol = lsq::chol_groups(N, hs.blk_off.data(), hs.blk_tf.data(), corder);
   DevBuf<int32_t> chol_order;
-  chol_order.upload(corder, st);
+  if (chol.size() > 1) chol_order.upload(corder, st);
   const bool both = h->coarse && !h->lean;
   if (both) {
     // The two factorisations, each a chain of small launches, run beside one another; the

@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kThreads) k_chol_diag(BandPlan P, double* __re
                                                         const int32_t* __restrict__ order, int k) {
   __shared__ double S[kT * 33], Q[kT * 33];
   __shared__ int fail;
-  const int i = order[blockIdx.x];
+  const int i = order ? order[blockIdx.x] : blockIdx.x;
   const int64_t b0 = P.blk_off[i];
   if (k >= (int)(P.blk_off[i + 1] - b0)) return;
   const int t0 = P.blk_tf[b0 + k];
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kThreads) k_chol_col(BandPlan P, double* __res
                                                        const double* __restrict__ dinv,
                                                        const int32_t* __restrict__ order, int k) {
   __shared__ double S[kT * 33], A[kT * 33], Q[kT * 33];
-  const int i = order[blockIdx.x], b = k + 1 + blockIdx.y;
+  const int i = order ? order[blockIdx.x] : blockIdx.x, b = k + 1 + blockIdx.y;
   const int64_t b0 = P.blk_off[i];
   if (b >= (int)(P.blk_off[i + 1] - b0)) return;
   const int t0 = P.blk_tf[b0 + b];
@@ -198,10 +198,11 @@ __global__ void __launch_bounds__(kThreads) k_chol_col(BandPlan P, double* __res
 __global__ void __launch_bounds__(kThreads) k_chol_update(BandPlan P, double* __restrict__ F,
                                                           const int32_t* __restrict__ order, int k, int below) {
   __shared__ double S[kT * 33], A[kT * 33], Q[kT * 33];
-  const int i = order[blockIdx.x];
+  const int i = order ? order[blockIdx.x] : blockIdx.x;
   const int64_t b0 = P.blk_off[i];
   const int nb = (int)(P.blk_off[i + 1] - b0);
-  for (int64_t e = blockIdx.y; e < chol_pairs(below); e += gridDim.y) {
+  const int64_t pairs = chol_pairs(below);
+  for (int64_t e = blockIdx.y; e < pairs; e += gridDim.y) {
     int b, c;
     chol_pair(e, b, c);
     b += k + 1;
@@ -251,7 +252,7 @@ void launch_band_cholesky(const BandPlan& P, const std::vector<CholGroup>& group
                           double* idiag, double* dinv, int* status, cudaStream_t st) {
   cudaMemsetAsync(status, 0, sizeof(int) * P.N, st);
   for (const CholGroup& g : groups) {
-    const int32_t* ord = order + g.first;
+    const int32_t* ord = groups.size() > 1 ? order + g.first : nullptr;  // (one group: all, in any order)
     for (int k = 0; k < g.max_nb; ++k) {
       k_chol_diag<<<g.count, kThreads, 0, st>>>(P, F, idiag, dinv, status, ord, k);
       const int below = std::min(g.below, g.max_nb - 1 - k);  // block rows that can reach column k

@@ -617,7 +617,7 @@ __global__ void __cluster_dims__(kOrthCluster, 1, 1) __launch_bounds__(kThreads)
 // matrix.  The update takes two pairs' 2 x 2 block at a time and uses the symmetry (16 FP64
 // instructions for its four entries and their mirror images; 32 by rows, then columns), and
 // pairs whose entry is so small that all such entries together pass the convergence test are
-// left alone (at first most of a Lanczos matrix, near the end most pairs): 1.8 ms so.
+// left alone (at first most of a Lanczos matrix, near the end most pairs): 1.9 ms so.
 constexpr int kMaxHalf = kMaxK / 2, kRitzWarps = (kMaxHalf + 31) / 32;
 struct RotMsg {  // the rotations of one round, from rank 0 to rank 1
   int n;         // -1: no more rounds

@@ -175,7 +175,7 @@ void launch_prep(const BandPlan& P, int max_nb, const double* dsub, const double
 // In-place Cholesky of every subdomain's matrix; idiag = 1 / diag(L);
 // status[i] = 0 or 1 + the local row of the first nonpositive pivot.
 // dinv: scratch of 1024 doubles per block row (inverse diagonal tiles).
-// groups, order (device): see chol_groups.
+// groups, order (device; not read when there is one group): see chol_groups.
 void launch_band_cholesky(const BandPlan& P, const std::vector<CholGroup>& groups, const int32_t* order,
                           double* st_fac, double* idiag, double* dinv, int* status, cudaStream_t st);
 
