@@ -169,16 +169,26 @@ void pack_block_super(ls_handle* h) {
 // - fewer than four right-hand sides on a batched handle, where the automatic choice has been
 //   one of the two tensor-core kernels and callers read which from ls_info.local_kernel (64
 //   subdomains and R = 2: 430 us; the superblocks would take 164).
+// A 32-row kernel reads a tile once for all right-hand sides, the superblocks once per group of
+// four or eight, so with several groups on a full chip the faster one depends on the size of
+// the subdomains: the first apply of a width times both there (choose_block_super).  Times of
+// an iteration over those with the 32-row kernel, pieces of 4 x 4 to 32 x 32 columns: BF16,
+// four groups, N = 1,024: 0.69 to 0.92, N = 400: 0.91 to 1.07; FP64, eight groups, N = 1,024:
+// 0.72 to 0.88, N = 144: 0.98 to 1.02, four groups 1.30 to 1.92; FP32, two groups, N = 1,024:
+// 0.80 to 1.05, N = 144: 1.08 to 1.33.  One group, or CTAs for few rounds of the SMs: up to ten
+// times faster, never slower.
 // The plan counts only when all of it has succeeded: after an error the next call plans anew.
 void plan_block_super(ls_handle* h, int R) {
   BlockState& B = h->blk;
   if (B.m_R == R) return;
   B.m_R = 0;
   B.m_ok = false;
+  B.m_try = false;
   B.gR = 0;  // (a graph of the last plan is not replayed)
   lsq::SuperShape shape{};
   const int64_t groups = (R + 7) / 8;
-  bool ok = h->opt.block_kernel == 0 && !h->opt.test_stall && !h->lean && !(h->prec == LS_PREC_F32 && h->nprob > 1 && R < 4);
+  bool ok = h->opt.block_kernel == 0 && !h->opt.test_stall && !h->lean && B.m_choice[R] != 2 && !(h->prec == LS_PREC_F32 && h->nprob > 1 && R < 4);
+  bool even = false;  // neither kernel is known to be the faster one
   if (ok) {
     int optin = 0, sms = 0;
     CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
@@ -187,6 +197,9 @@ void plan_block_super(ls_handle* h, int R) {
     ok = !(h->prec == LS_PREC_F32 && groups > 2 && groups * h->N > 3 * (int64_t)sms) &&
          lsq::local_super_plan_multi(h->prec, R, h->N, h->max_nb, std::max(h->wmax, lsq::kSuperRows), sms,
                                      (size_t)optin, shape);
+    const int64_t ctas = (int64_t)h->N * ((R + shape.nr - 1) / std::max(shape.nr, 1));
+    even = h->prec == LS_PREC_F32 ? R > 8 && 2 * ctas > 5 * (int64_t)sms
+                                  : R > (h->prec == LS_PREC_F64 ? 16 : 4) && ctas > 5 * (int64_t)sms;
   }
   if (ok && !B.m_fac.p) {
     try {
@@ -198,6 +211,7 @@ void plan_block_super(ls_handle* h, int R) {
   }
   B.m_shape = shape;
   B.m_ok = ok;
+  B.m_try = ok && even && B.m_choice[R] == 0;
   B.m_R = R;
 }
 
@@ -301,10 +315,43 @@ void choose_local_kernel(ls_handle* h, int R, const double* Rin) {
   }
 }
 
+// Times the superblock kernel against the 32-row kernel for R right-hand sides (see
+// plan_block_super), on the first block apply's right-hand side, and keeps the faster for all
+// solves of that width.
+void choose_block_super(ls_handle* h, int R, const double* Rin) {
+  BlockState& B = h->blk;
+  B.m_try = false;
+  choose_local_kernel(h, R, Rin);
+  if (!B.m_ok) return;  // (its copies took the room of the superblocks')
+  cudaStream_t st = h->st;
+  cudaEvent_t e0, e1;
+  CK(cudaEventCreate(&e0));
+  CK(cudaEventCreate(&e1));
+  float ms[2] = {0.f, 0.f};
+  for (int k = 0; k < 2; ++k) {
+    auto launch = [&]() {
+      if (k == 0) launch_block_super(h, R, Rin);
+      else launch_local_kernel(h, B.use_tc ? B.kernel : 0, R, Rin);
+    };
+    launch();  // warm-up
+    CK(cudaEventRecord(e0, st));
+    launch();
+    CK(cudaEventRecord(e1, st));
+    CK(cudaEventSynchronize(e1));
+    CK(cudaEventElapsedTime(&ms[k], e0, e1));
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  check_launch("block local-solve timing");
+  B.m_ok = ms[0] <= ms[1];
+  B.m_choice[R] = B.m_ok ? 1 : 2;
+}
+
 // z = M^{-1} r for all pairs, with the partials of r.z (and rold.z when flexible).
 void precond_block(ls_handle* h, int R, const double* Rin, double* Zout, bool flex, bool timed) {
   BlockState& B = h->blk;
   cudaStream_t st = h->st;
+  if (B.m_try) choose_block_super(h, R, Rin);
   if (!B.m_ok) choose_local_kernel(h, R, Rin);
   if (timed) record_event(h->ev[2], st);
   if (B.m_ok) launch_block_super(h, R, Rin);

@@ -181,6 +181,8 @@ struct BlockState {
   // first block solve that uses it
   int m_R = 0;
   bool m_ok = false;
+  bool m_try = false;                // the next apply times it against the 32-row kernel
+  signed char m_choice[33] = {};     // what that found for R right-hand sides: 1 superblocks, 2 not
   int64_t m_back = 0;  // FP32: the transposed copy's distance
   lsq::SuperShape m_shape{};
   DevBuf<int32_t> m_tf, m_order;

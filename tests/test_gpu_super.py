@@ -128,3 +128,43 @@ def test_super_many_right_hand_sides_on_a_pair_in_double():
     N, _, sms = _rule("n64", "f64")
     assert 2 * N <= sms < 4 * N
     test_super_many_right_hand_sides("n64", "f64", 3)
+
+
+@pytest.mark.parametrize("prec,tol", [("f64", 1e-10), ("f32", 1e-4), ("bf16", 1e-4)])
+def test_super_timed_choice_for_wide_block_solves(prec, tol):
+    """1,024 subdomains of 4 x 4 columns: with several groups of right-hand sides the superblocks
+    can be the slower kernel, and the first solve of a width times both.  Whichever ran, three
+    iterations agree with the 32-row kernel's (tolerances as above), also when the widths
+    alternate, and the solve is not slower than that one's by more than the spread of timing
+    (it was up to 2.9 times slower with BF16 factors, 1.5 with FP64)."""
+    import time
+
+    import paper_2107_09006_gb300 as L
+
+    m, n, rp, col, val, b, _ = make_grid_ls(128, 128, 4, 6, 2, 7, nrhs=32)
+    b = torch.as_tensor(np.asarray(b), device="cuda")
+    part = block_partition(128, 128, 4, 4)
+    mk = lambda **o: L.Solver(m, n, rp, col, val, part, 1024, coarse=0, factor_prec=prec, fixed_iters=3,  # noqa: E731
+                              spmv=2, **o)
+    S, S1 = mk(), mk(block_kernel=1)
+    out = {}
+    for R in (32, 12, 32, 8, 12):
+        X, X1 = S.solve(b[:R])[0], S1.solve(b[:R])[0]
+        assert float((X - X1).norm() / X1.norm()) < tol, R
+        assert R not in out or torch.equal(out[R], X)
+        out[R] = X
+
+    def seconds(solver, R):
+        best = 1e9
+        for _ in range(7):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            solver.solve(b[:R])
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t)
+        return best
+
+    for R in (12, 32):
+        assert seconds(S, R) <= 1.25 * seconds(S1, R), R
+    S.close()
+    S1.close()
