@@ -1482,8 +1482,11 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     ea.kwant_cap = kw; ea.Kmax = K; ea.keep = keep; ea.maxit = h->opt.eig_maxit; ea.tol = h->opt.eig_tol;
     ea.V = V.p; ea.V2 = V2.p; ea.vstride = vs; ea.H = H.p; ea.S = S.p; ea.vec = vec.p; ea.lam = lam.p;
     ea.nconv = nconv.p; ea.steps = steps.p; ea.status = est.p;
-    // over the whole GPU where a subdomain's FP64 vector fits the superblock kernel, else one
-    // CTA per subdomain
+    // Over the whole GPU where a subdomain's FP64 vector fits the superblock kernel, else one
+    // CTA per subdomain; so too more subdomains than SMs of less than 5.5 block rows on average,
+    // whose steps are too short for a kernel per stage and fill the chip as they are (1,024
+    // subdomains of 2.9 block rows 26.6 ms against 40.0, of 4.9 41.3 against 43.8, of 5.9 46.3
+    // against 42.5; 144 of 4.0 10.7 against 8.7).
     lsq::LanczosGrid lg{};
     DevBuf<int> lz_state, lz_rr, lz_ord;
     DevBuf<double> lz_beta, lz_err, lz_rows;
@@ -1491,7 +1494,8 @@ void do_setup(ls_handle* h, const int64_t* row_ptr_in, const int32_t* col_in, co
     {
       int optin = 0;
       CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev));
-      if (!h->lean && hs.xi_off[N] < INT32_MAX &&
+      const bool tiny = N > sms && 2 * h->total_blocks < 11 * (int64_t)N;
+      if (!h->lean && !tiny && hs.xi_off[N] < INT32_MAX &&
           lsq::local_super_plan(0, N, h->max_nb, std::max(h->wmax, lsq::kSuperRows),
                                 (double)h->fac_elems / 1024.0 / (double)h->total_blocks, sms, (size_t)optin, lg.shape)) {
         Ctst.release();  // (the operator runs from A)
