@@ -5,7 +5,9 @@ Sources compile in parallel into ``_build/`` next to this file and link into
 source or header is newer than the library.  ``build(debug_bounds=True)`` makes the
 bounds-checked variant ``libls_schwarz_dbg.so`` (compiled with -DLS_DEBUG_BOUNDS into
 ``_build_dbg/``): its gather, scatter and local-solve kernels check every index and copy
-range and report an out-of-range one as LS_ERR_INVALID instead of using it.
+range and report an out-of-range one as LS_ERR_INVALID instead of using it; it also exports
+the tests' hooks (ls_debug_alloc: refuse allocations; ls_debug_stall: waits of the superblock
+kernel that run out).
 """
 from __future__ import annotations
 
